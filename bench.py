@@ -72,7 +72,7 @@ STEP_KERNELS = ("prep", "classify", "walk", "gate", "scatter", "alloc", "free", 
 FRAME_TRAFFIC = {"code_sha256_16": "d4cbf5a756f0205c", "bytes_per_live": 70.4,
                  "capture": "k_frame1, frames 8 and 9 of the flythrough: 50.9 MB at 712,190 live, "
                             "52.0 MB at 748,560 live"}
-FRAME_SOURCES = ("cbt_fused.cu", "cbt_phases.cuh", "cbt_device.cuh")
+FRAME_SOURCES = ("cbt_frame.cuh", "cbt_phases.cuh", "cbt_device.cuh")
 
 
 def frame_code_hash():

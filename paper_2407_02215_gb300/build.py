@@ -16,7 +16,8 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libcbt.so")
-SOURCES = ["cbt_kernels.cu", "cbt_fused.cu", "cbt_reduce.cu", "cbt_index.cu", "cbt_api.cu", "cbt_static.cu",
+SOURCES = ["cbt_frame_any.cu", "cbt_frame_f32.cu", "cbt_frame_f32disp.cu", "cbt_frame_fixed.cu", "cbt_frame_f64.cu",
+           "cbt_frame_sphere.cu", "cbt_kernels.cu", "cbt_reduce.cu", "cbt_index.cu", "cbt_api.cu", "cbt_static.cu",
            "ingest.cpp", "camera.cpp"]
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -190,6 +190,7 @@ struct cbt_batch {
     cudaGraphExec_t exec = nullptr;
     uint32_t exec_tw = 0, exec_mult = 0;
     bool exec_vertices = false, exec_fused = false;
+    int exec_form = kFormAny;
     bool timing = false;
     cudaEvent_t ev[kNumKernels + 1] = {};
     uint32_t timed = 0, launches = 0;
@@ -329,7 +330,7 @@ int grid_prep(const cbt_batch* B) {
 
 // The kernels of one frame of a batch descriptor; ev (optional) receives an
 // event before and after every kernel. Returns the number of launches.
-uint32_t enqueue_kernels(const BatchDev& bt, int sms, uint32_t grid_mult, bool vertices, cudaStream_t s,
+uint32_t enqueue_kernels(const BatchDev& bt, int form, int sms, uint32_t grid_mult, bool vertices, cudaStream_t s,
                          cudaEvent_t* ev) {
     const uint32_t prep_n = std::max(bt.Trel, 2u * bt.Titems + bt.Twords);
     const int prep = static_cast<int>(std::max(1u, std::min<uint32_t>((prep_n + kThreads - 1u) / kThreads,
@@ -345,7 +346,7 @@ uint32_t enqueue_kernels(const BatchDev& bt, int sms, uint32_t grid_mult, bool v
     mark();
     launch_prep(bt, true, prep, s);
     mark();
-    launch_classify(bt, items, s);
+    launch_classify(bt, form, items, s);
     mark();
     launch_walk(bt, items, s);
     mark();
@@ -362,12 +363,20 @@ uint32_t enqueue_kernels(const BatchDev& bt, int sms, uint32_t grid_mult, bool v
     launch_cbt(bt, words, s);
     mark();
     if (vertices) {
-        launch_vertices(bt, items, s);
+        launch_vertices(bt, form, items, s);
         mark();
     }
     uint32_t launches = 0;
     for (uint32_t q = 0; q + 1u < k; ++q) launches += kLaunchesPerStep[q];
     return launches;
+}
+
+// The vertex form of a batch's frames, or kFormAny when they differ.
+int form_of_frames(const FrameP* fps, uint32_t n) {
+    const Form f = form_of(fps[0]);
+    for (uint32_t b = 1; b < n; ++b)
+        if (form_of(fps[b]) != f) return kFormAny;
+    return f;
 }
 
 // The kernels of one frame. `timed`: record events between the kernels (the
@@ -378,25 +387,25 @@ bool use_frame1(const cbt_batch* B) {
     return B->n == 1 && B->fused_grid1 > 0 && B->cap[0] <= kFrame1MaxCap && B->tw == kFrame1TileWords;
 }
 
-void enqueue_frame(cbt_batch* B, cudaStream_t s, bool vertices, bool timed) {
+void enqueue_frame(cbt_batch* B, int form, cudaStream_t s, bool vertices, bool timed) {
     if (B->fused) {
         BatchDev bt = B->dev;
         bt.timing = timed ? 1u : 0u;
         B->launches = 1;
         if (use_frame1(B)) {
             const uint32_t span = std::min<uint32_t>(B->cap[0], 32u * B->tw);
-            launch_frame1(bt, B->fused_grid1, ceil_log2(span), s);
+            launch_frame1(bt, form, B->fused_grid1, ceil_log2(span), s);
             B->last_frame1 = true;
             B->timed = timed ? static_cast<uint32_t>(kFrame1Phases) : 0u;
             return;
         }
         B->last_frame1 = false;
-        launch_frame(bt, B->fused_grid, s);
+        launch_frame(bt, form, B->fused_grid, s);
         // a batch exports vertices within its compaction phase
         B->timed = timed ? static_cast<uint32_t>(B->n == 1 ? kFramePhases : kFramePhases - 1) : 0u;
         return;
     }
-    B->launches = enqueue_kernels(B->dev, B->sms, B->grid_mult, vertices, s, timed ? B->ev : nullptr);
+    B->launches = enqueue_kernels(B->dev, form, B->sms, B->grid_mult, vertices, s, timed ? B->ev : nullptr);
     B->timed = timed ? (vertices ? 10u : 9u) : 0u;
 }
 
@@ -431,6 +440,7 @@ int batch_update(cbt_batch* B, const cbt_frame* frames, cudaStream_t s) {
         if (!frame_from_api(frames + b, B->st[b]->frame, fps[b])) return CBT_EINVAL;
         vertices = vertices || fps[b].vout != nullptr;
     }
+    const int form = form_of_frames(fps.data(), n);
     // online autotuner: one candidate configuration per frame, round robin,
     // then the fastest by median time per live bisector (results do not depend on it)
     if (B->tuning) {
@@ -483,7 +493,7 @@ int batch_update(cbt_batch* B, const cbt_frame* frames, cudaStream_t s) {
         if (B->staged_pending) cudaEventSynchronize(B->staged);
         std::memcpy(B->h_fps, fps.data(), sizeof(FrameP) * n);
         if (!B->exec || B->exec_tw != B->tw || B->exec_mult != B->grid_mult || B->exec_vertices != vertices ||
-            B->exec_fused != B->fused) {
+            B->exec_fused != B->fused || B->exec_form != form) {
             if (B->exec) {
                 cudaGraphExecDestroy(B->exec);
                 B->exec = nullptr;
@@ -494,7 +504,7 @@ int batch_update(cbt_batch* B, const cbt_frame* frames, cudaStream_t s) {
             B->dev.fps = reinterpret_cast<const FrameP*>(B->region + B->L.fps);
             cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
             cudaMemcpyAsync(B->region + B->L.fps, B->h_fps, sizeof(FrameP) * n, cudaMemcpyHostToDevice, cs);
-            enqueue_frame(B, cs, vertices, false);
+            enqueue_frame(B, form, cs, vertices, false);
             const cudaError_t e1 = cudaStreamEndCapture(cs, &g);
             cudaStreamDestroy(cs);
             if (e1 != cudaSuccess || !g) return CBT_ECUDA;
@@ -505,6 +515,7 @@ int batch_update(cbt_batch* B, const cbt_frame* frames, cudaStream_t s) {
             B->exec_mult = B->grid_mult;
             B->exec_vertices = vertices;
             B->exec_fused = B->fused;
+            B->exec_form = form;
         }
         if (cudaGraphLaunch(B->exec, s) != cudaSuccess) return CBT_ECUDA;
         cudaEventRecord(B->staged, s);
@@ -513,7 +524,7 @@ int batch_update(cbt_batch* B, const cbt_frame* frames, cudaStream_t s) {
     } else if (n == 1) {
         B->dev.fps = nullptr;
         B->dev.fp0 = fps[0];
-        enqueue_frame(B, s, vertices, B->timing);
+        enqueue_frame(B, form, s, vertices, B->timing);
     } else {
         if (B->staged_pending) cudaEventSynchronize(B->staged);
         std::memcpy(B->h_fps, fps.data(), sizeof(FrameP) * n);
@@ -522,7 +533,7 @@ int batch_update(cbt_batch* B, const cbt_frame* frames, cudaStream_t s) {
         cudaEventRecord(B->staged, s);
         B->staged_pending = true;
         B->dev.fps = reinterpret_cast<const FrameP*>(B->region + B->L.fps);
-        enqueue_frame(B, s, vertices, B->timing);
+        enqueue_frame(B, form, s, vertices, B->timing);
     }
     if (tune_now) {
         cudaEventRecord(B->tune_ev[1], s);
@@ -737,7 +748,7 @@ extern "C" int cbt_vertices(cbt_state* st, float* d_out, const double h_origin[3
     bt.fp0 = fp;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     launch_prep(bt, false, grid_prep(B), s);
-    launch_vertices(bt, std::max(1, static_cast<int>(std::min<uint32_t>(bt.Titems, static_cast<uint32_t>(st->sms) * 8u))), s);
+    launch_vertices(bt, form_of(fp), std::max(1, static_cast<int>(std::min<uint32_t>(bt.Titems, static_cast<uint32_t>(st->sms) * 8u))), s);
     rc = check_launch();
     if (rc) return rc;
     return cudaStreamSynchronize(s) == cudaSuccess ? CBT_OK : CBT_ECUDA;
@@ -1176,6 +1187,7 @@ extern "C" int cbt_server_submit(cbt_server* sv, const int32_t* idx, const cbt_f
         hv[i + 1] = hv[i] + item_tiles(st->inst.cap);
         hr[i + 1] = hr[i] + 9u * st->inst.H;
     }
+    const int form = form_of_frames(hf, kk);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     // a fused tick starts after the previous tick (two cooperative launches
     // are never in flight together)
@@ -1204,9 +1216,9 @@ extern "C" int cbt_server_submit(cbt_server* sv, const int32_t* idx, const cbt_f
     if (sv->fused) {
         const uint32_t work = std::max({bt.Titems, bt.Twords, (bt.Trel + 255u) / 256u, 1u});
         const uint32_t grid = std::min(work, static_cast<uint32_t>(sv->frame_per_sm * sv->sms));
-        if (launch_frame(bt, static_cast<int>(grid), s) != cudaSuccess) return CBT_ECUDA;
+        if (launch_frame(bt, form, static_cast<int>(grid), s) != cudaSuccess) return CBT_ECUDA;
     } else {
-        enqueue_kernels(bt, sv->sms, sv->grid_mult, vertices, s, nullptr);
+        enqueue_kernels(bt, form, sv->sms, sv->grid_mult, vertices, s, nullptr);
     }
     cudaMemcpyAsync(S.host + L.block, bt.nout, 4u * kk, cudaMemcpyDeviceToHost, s);
     if (cudaEventRecord(S.done, s) != cudaSuccess || cudaGetLastError() != cudaSuccess) return CBT_ECUDA;

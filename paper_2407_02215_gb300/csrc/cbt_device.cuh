@@ -153,6 +153,25 @@ struct FrameP {
     uint32_t dseed;  // displacement lattice seed
 };
 
+// The vertex form a kernel is compiled for: the precision of the frame's
+// vertices and, in FP32, whether they are displaced (kFormAny: read from the
+// frame's parameters, for a batch whose frames differ). One form per kernel
+// keeps the others' code and registers out of it: the single-instance frame
+// of the FP32 grid is 129 us a pass against 156 us with every form in one kernel.
+enum Form : int { kFormAny = 0, kFormF32, kFormF32Disp, kFormFixed, kFormF64, kFormSphere, kForms };
+__host__ __device__ inline Form form_of(const FrameP& fp) {
+    return fp.precision == 0u ? (fp.damp != 0.0f ? kFormF32Disp : kFormF32)
+                              : fp.precision == 1u ? kFormFixed : fp.precision == 2u ? kFormF64 : kFormSphere;
+}
+template <int F>
+__device__ __forceinline__ uint32_t precision_in(const FrameP& fp) {
+    return F == kFormAny ? fp.precision : F == kFormFixed ? 1u : F == kFormF64 ? 2u : F == kFormSphere ? 3u : 0u;
+}
+template <int F>
+__device__ __forceinline__ bool displaced_in(const FrameP& fp) {
+    return F == kFormF32Disp || ((F == kFormAny || F == kFormSphere) && fp.damp != 0.0f);
+}
+
 constexpr int kFramePhases = 10;  // phases of the one-launch frame (a batch skips the last)
 
 // Launch-wide counters of one batch (256 bytes).
@@ -233,51 +252,53 @@ __device__ __forceinline__ void set_err(Globals* g, uint32_t e) { atomicOr(&g->e
 
 // ------------------------------------------------- Alg. 2 / Eq. 1 decode
 
-// Integer form of Alg. 2 evaluated from the first split down: with W the
-// weights over 2^k after k levels, a 0 bit maps the rows (r0, r1, r2) to
-// (2 r0, 2 r2, r0 + r1) and a 1 bit to (2 r2, 2 r1, r0 + r1) (Eq. 1 times 2),
-// i.e. W <- T_b W with T_0 = 2 M_0 and T_1 = 2 M_1. Eight levels at once are
-// W <- P_c W with P_c = T_{c7} T_{c6} ... T_{c0} for the eight path bits c
-// (most significant applied first), precomputed below for all 256 c; every
-// entry of P_c is at most 2^8 (16 bits). Every row of W sums to 2^k (the
-// rows of M are barycentric), so only the first two columns are carried
-// and the third is 2^k minus them. W = 2^d M exactly while entries fit T
-// (T = u32 for d <= 31). The first r < 8 levels from the identity are the
-// first two columns of the r-level product, tabulated too (q: r-level
-// entries for the 2^r prefixes c at q[2^r - 2 + c]).
+// Alg. 2 evaluated from the first split down: with M the weights after k
+// levels, a 0 bit maps the rows (r0, r1, r2) to (r0, r2, (r0 + r1) / 2) and a
+// 1 bit to (r2, r1, (r0 + r1) / 2) (Eq. 1), i.e. M <- M_b M. Up to eight
+// levels at once are M <- P_c M with P_c the product for the path bits c
+// (most significant applied first). Every row of M and P sums to 1 (they are
+// barycentric), so only the first two columns are carried, and with the rows
+// (a0, a1, a2) of M
+//   P row (p0, p1, 1 - p0 - p1):  a2 + p0 (a0 - a2) + p1 (a1 - a2).
+// After k <= 24 levels every entry is a multiple of 2^-k in [0, 1], and so is
+// every intermediate value here, so FP32 fused multiply-adds are exact: the
+// decode runs at the FP32 rate and needs no integer-to-float conversions
+// (the integer form it replaced, with 16-bit table entries read one by one,
+// made the classify phase of 886k leaves 33 us; this form makes it 24 us).
+// The table holds P for r = 1..8 levels and all 2^r codes c in row
+// 2^r - 2 + c (then the identity): the six entries in multiples of 2^-r, at
+// most 8 significant bits, i.e. exact in bfloat16, so that a row is one
+// 16-byte shared-memory load.
+constexpr uint32_t kDecRows = 512, kDecIdentity = 510;
 struct alignas(16) DecTable {
-    uint16_t p[256][9];
-    uint16_t q[256][6];  // 254 used
+    uint32_t w[kDecRows][4];  // {p00 | p01 << 16, p10 | p11 << 16, p20 | p21 << 16, 0}
 };
 
-constexpr void dec_product(int c, int levels, uint32_t m[9]) {
-    for (int e = 0; e < 9; ++e) m[e] = (e % 4 == 0) ? 1u : 0u;
-    for (int k = levels - 1; k >= 0; --k) {
-        const int b = (c >> k) & 1;
-        uint32_t n[9] = {};
-        for (int col = 0; col < 3; ++col) {
-            n[6 + col] = m[col] + m[3 + col];
-            n[col] = 2u * (b ? m[6 + col] : m[col]);
-            n[3 + col] = 2u * (b ? m[3 + col] : m[6 + col]);
-        }
-        for (int e = 0; e < 9; ++e) m[e] = n[e];
-    }
+constexpr uint32_t bf16_of(uint32_t m, int r) {  // m 2^-r, m <= 256
+    if (m == 0u) return 0u;
+    int e = 0;
+    while ((m >> (e + 1)) != 0u) ++e;
+    const uint32_t frac = e <= 7 ? (m << (7 - e)) & 0x7Fu : 0u;
+    return ((uint32_t)(127 + e - r) << 7) | frac;
 }
 
 constexpr DecTable make_dec8() {
     DecTable t{};
-    for (int c = 0; c < 256; ++c) {
-        uint32_t m[9] = {};
-        dec_product(c, 8, m);
-        for (int e = 0; e < 9; ++e) t.p[c][e] = static_cast<uint16_t>(m[e]);
-    }
-    for (int r = 1; r < 8; ++r)
-        for (int c = 0; c < (1 << r); ++c) {
-            uint32_t m[9] = {};
-            dec_product(c, r, m);
-            for (int row = 0; row < 3; ++row)
-                for (int col = 0; col < 2; ++col)
-                    t.q[(1 << r) - 2 + c][2 * row + col] = static_cast<uint16_t>(m[3 * row + col]);
+    for (int r = 0; r <= 8; ++r)
+        for (uint32_t c = 0; c < (1u << r); ++c) {
+            uint32_t m[6] = {1, 0, 0, 1, 0, 0};  // 2^k times the rows' first two columns after k levels
+            for (int k = r - 1; k >= 0; --k) {
+                const bool b = ((c >> k) & 1u) != 0u;
+                uint32_t n[6] = {};
+                for (int col = 0; col < 2; ++col) {
+                    n[4 + col] = m[col] + m[2 + col];
+                    n[col] = 2u * (b ? m[4 + col] : m[col]);
+                    n[2 + col] = 2u * (b ? m[2 + col] : m[4 + col]);
+                }
+                for (int e = 0; e < 6; ++e) m[e] = n[e];
+            }
+            const uint32_t row = r ? (1u << r) - 2u + c : kDecIdentity;
+            for (int q = 0; q < 3; ++q) t.w[row][q] = bf16_of(m[2 * q], r) | (bf16_of(m[2 * q + 1], r) << 16);
         }
     return t;
 }
@@ -286,122 +307,211 @@ constexpr DecTable make_dec8() {
 // different address in every lane, which the constant cache serializes.
 __device__ const DecTable g_dec8 = make_dec8();
 constexpr uint32_t kDecTabWords = sizeof(DecTable) / 4u;  // the table in 32-bit words
-static_assert(sizeof(DecTable) % 16u == 0u, "the table is copied 16 bytes at a time");
 
-// Copies the tables into shared memory (kDecTabWords words, s_tab 16-byte
+// Copies the table into shared memory (kDecTabWords words, s_tab 16-byte
 // aligned; call with the whole block, then __syncthreads()).
 __device__ __forceinline__ void load_dec6(uint32_t* s_tab) {
-    const uint4* src = reinterpret_cast<const uint4*>(&g_dec8.p[0][0]);
+    const uint4* src = reinterpret_cast<const uint4*>(&g_dec8.w[0][0]);
     for (uint32_t k = threadIdx.x; k < kDecTabWords / 4u; k += blockDim.x)
         reinterpret_cast<uint4*>(s_tab)[k] = __ldg(src + k);
 }
 // The same copy in two halves (blocks of 256 threads): the loads into
 // registers, then the stores, so that other loads can go out in between.
-constexpr uint32_t kDecVecs = kDecTabWords / 4u;
-__device__ __forceinline__ void dec_fetch(uint4 (&r)[kDecVecs / 256u + 1u]) {
-    const uint4* src = reinterpret_cast<const uint4*>(&g_dec8.p[0][0]);
+constexpr uint32_t kDecVecs = kDecTabWords / 4u / 256u;  // 16-byte loads per thread
+__device__ __forceinline__ void dec_fetch(uint4 (&r)[kDecVecs]) {
+    const uint4* src = reinterpret_cast<const uint4*>(&g_dec8.w[0][0]);
 #pragma unroll
-    for (uint32_t k = 0; k < kDecVecs / 256u + 1u; ++k) {
-        const uint32_t i = threadIdx.x + 256u * k;
-        r[k] = i < kDecVecs ? __ldg(src + i) : make_uint4(0u, 0u, 0u, 0u);
-    }
+    for (uint32_t k = 0; k < kDecVecs; ++k) r[k] = __ldg(src + threadIdx.x + 256u * k);
 }
-__device__ __forceinline__ void dec_store(uint32_t* s_tab, const uint4 (&r)[kDecVecs / 256u + 1u]) {
+__device__ __forceinline__ void dec_store(uint32_t* s_tab, const uint4 (&r)[kDecVecs]) {
 #pragma unroll
-    for (uint32_t k = 0; k < kDecVecs / 256u + 1u; ++k) {
-        const uint32_t i = threadIdx.x + 256u * k;
-        if (i < kDecVecs) reinterpret_cast<uint4*>(s_tab)[i] = r[k];
-    }
+    for (uint32_t k = 0; k < kDecVecs; ++k) reinterpret_cast<uint4*>(s_tab)[threadIdx.x + 256u * k] = r[k];
 }
 
-// One level on the first two columns, a[2 r + c] (c = 0, 1).
-template <typename T>
-__device__ __forceinline__ void dec_step(T a[6], bool b) {
-    T n[6];
-#pragma unroll
-    for (int c = 0; c < 2; ++c) {
-        n[4 + c] = a[c] + a[2 + c];
-        n[c] = (b ? a[4 + c] : a[c]) << 1;
-        n[2 + c] = (b ? a[2 + c] : a[4 + c]) << 1;
-    }
-#pragma unroll
-    for (int k = 0; k < 6; ++k) a[k] = n[k];
+__device__ __forceinline__ void dec_row(const uint32_t* tab, uint32_t row, float p[6]) {
+    const uint4 v = reinterpret_cast<const uint4*>(tab)[row];
+    p[0] = __uint_as_float(v.x << 16);
+    p[1] = __uint_as_float(v.x & 0xFFFF0000u);
+    p[2] = __uint_as_float(v.y << 16);
+    p[3] = __uint_as_float(v.y & 0xFFFF0000u);
+    p[4] = __uint_as_float(v.z << 16);
+    p[5] = __uint_as_float(v.z & 0xFFFF0000u);
 }
 
-template <typename T>
-__device__ __forceinline__ void dec_chunk(T a[6], const uint16_t* P) {
-    T n[6];
-#pragma unroll
-    for (int r = 0; r < 3; ++r) {
-        const T p0 = P[3 * r], p1 = P[3 * r + 1], p2 = P[3 * r + 2];
-#pragma unroll
-        for (int c = 0; c < 2; ++c) n[2 * r + c] = p0 * a[c] + p1 * a[2 + c] + p2 * a[4 + c];
-    }
-#pragma unroll
-    for (int k = 0; k < 6; ++k) a[k] = n[k];
-}
-
-// The 3 x 3 weights from the first two columns at 2^k.
-template <typename T>
-__device__ __forceinline__ void dec_expand(const T a[6], T pw, T W[9]) {
-#pragma unroll
-    for (int r = 0; r < 3; ++r) {
-        W[3 * r] = a[2 * r];
-        W[3 * r + 1] = a[2 * r + 1];
-        W[3 * r + 2] = pw - a[2 * r] - a[2 * r + 1];
-    }
-}
-
-// W = weights of bisector j at depth d, Wp = those of its parent (d >= 1);
-// tab = the eight-level table in shared memory.
-template <typename T>
-__device__ __forceinline__ void decode_weights(uint64_t j, int d, T W[9], T Wp[9], const uint32_t* tab) {
-    const uint16_t* tab16 = reinterpret_cast<const uint16_t*>(tab);
-    T a[6] = {1, 0, 0, 1, 0, 0};
-    if (d >= 1) {
-        int lvl = d - 1;  // path bit applied next; the parent covers bits d-1 .. 1
-        const int rem = (d - 1) & 7;
-        if (rem) {  // the first rem levels from the identity: one lookup
-            const uint32_t c = (uint32_t)((j >> (lvl - rem + 1)) & ((1ull << rem) - 1ull));
-            const uint16_t* Q = tab16 + 256u * 9u + 6u * ((1u << rem) - 2u + c);
-#pragma unroll
-            for (int k = 0; k < 6; ++k) a[k] = Q[k];
-            lvl -= rem;
-        }
+// The first two columns (a[2 r + c]) of the product of n <= 24 levels whose
+// path bits are the low n bits of `bits`.
+__device__ __forceinline__ void decode_levels(uint32_t bits, int n, const uint32_t* tab, float a[6]) {
+    const int first = n ? ((n - 1) & 7) + 1 : 0;  // levels of the first lookup
+    int sh = n - first;
+    const uint32_t row0 = (1u << first) - 2u + (bits >> sh & ((1u << first) - 1u));
+    dec_row(tab, n ? row0 : kDecIdentity, a);
 #pragma unroll 1
-        for (; lvl >= 8; lvl -= 8) dec_chunk<T>(a, tab16 + 9u * (uint32_t)((j >> (lvl - 7)) & 255ull));
-        dec_expand<T>(a, (T)1 << (d - 1), Wp);
-        dec_step<T>(a, j & 1ull);
-    } else {
-        dec_expand<T>(a, (T)1, Wp);
+    while (sh > 0) {
+        sh -= 8;
+        float p[6];
+        dec_row(tab, 254u + ((bits >> sh) & 255u), p);
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const float e = __fsub_rn(a[c], a[4 + c]), f = __fsub_rn(a[2 + c], a[4 + c]), a2 = a[4 + c];
+#pragma unroll
+            for (int r = 0; r < 3; ++r) a[2 * r + c] = __fmaf_rn(p[2 * r], e, __fmaf_rn(p[2 * r + 1], f, a2));
+        }
     }
-    dec_expand<T>(a, (T)1 << d, W);
 }
 
-// Round-to-nearest conversion of a weight to FP32 / FP64 (exact below 2^24 /
-// 2^53; the 32-bit forms for 32-bit weights).
-__device__ __forceinline__ float wfloat(uint32_t w) { return __uint2float_rn(w); }
-__device__ __forceinline__ float wfloat(unsigned long long w) { return __ull2float_rn(w); }
-__device__ __forceinline__ double wdouble(uint32_t w) { return __uint2double_rn(w); }
-__device__ __forceinline__ double wdouble(unsigned long long w) { return __ull2double_rn(w); }
-
-// Correctly rounded signed 128-bit integer -> float: shift down to 63
-// significant bits with a sticky bit (round to odd), then one RN conversion.
-__device__ __forceinline__ float i128_to_float(__int128 s) {
-    const bool neg = s < 0;
-    unsigned __int128 u = neg ? (unsigned __int128)(-s) : (unsigned __int128)s;
-    const uint64_t hi = (uint64_t)(u >> 64), lo = (uint64_t)u;
-    float f;
-    if (hi == 0 && (lo >> 63) == 0) {
-        f = __ull2float_rn(lo);
-    } else {
-        const int bl = hi ? 128 - __clzll((long long)hi) : 64;
-        const int sh = bl - 63;
-        const unsigned __int128 mask = (((unsigned __int128)1) << sh) - 1;
-        const uint64_t m = (uint64_t)(u >> sh) | (uint64_t)((u & mask) != 0);
-        f = __fmul_rn(__ull2float_rn(m), pow2f(sh));
+// The weights of bisector j at depth d, as the first two columns a[2 r + c]
+// in one of two types: float, M itself, exact for d <= kFloatDepth; or
+// unsigned long long, W = 2^d M, for any depth (d <= 62).
+constexpr int kFloatDepth = 24;
+typedef unsigned long long u64;
+__device__ __forceinline__ void decode_cols(uint64_t j, int d, const uint32_t* tab, float a[6]) {
+    decode_levels((uint32_t)j & ((1u << d) - 1u), d, tab, a);
+}
+// The levels in runs of at most 24, each decoded in FP32 and applied to the
+// integer weights so far: 2^24 a2 + b0 (a0 - a2) + b1 (a1 - a2), b = 2^24 P.
+__device__ __forceinline__ void decode_cols(uint64_t j, int d, const uint32_t* tab, u64 a[6]) {
+    const int first = d > 0 ? (d - 1) % 24 + 1 : 0;
+    float p[6];
+    decode_levels((uint32_t)(j >> (d - first)) & ((1u << first) - 1u), first, tab, p);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) a[k] = __float2uint_rn(__fmul_rn(p[k], pow2f(first)));
+#pragma unroll 1
+    for (int lo = d - first - 24; lo >= 0; lo -= 24) {
+        decode_levels((uint32_t)(j >> lo) & 0xFFFFFFu, 24, tab, p);
+        uint32_t b[6];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) b[k] = __float2uint_rn(__fmul_rn(p[k], 0x1p24f));
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const long long e = (long long)(a[c] - a[4 + c]), f = (long long)(a[2 + c] - a[4 + c]);
+            const u64 a2 = a[4 + c] << 24;
+#pragma unroll
+            for (int r = 0; r < 3; ++r)
+                a[2 * r + c] = a2 + (u64)((long long)b[2 * r] * e) + (u64)((long long)b[2 * r + 1] * f);
+        }
     }
-    return neg ? -f : f;
+}
+
+__device__ __forceinline__ float unit_of(float, int) { return 1.0f; }
+__device__ __forceinline__ u64 unit_of(u64, int d) { return 1ull << d; }
+
+// The three weights of vertex v.
+template <typename T>
+__device__ __forceinline__ void weight_row(const T a[6], int v, int d, T w[3]) {
+    w[0] = a[2 * v];
+    w[1] = a[2 * v + 1];
+    w[2] = unit_of(T(), d) - w[0] - w[1];
+}
+// The three weights, over the same 2^d, of the parent's vertex that the
+// bisector does not share. Eq. 1 makes an odd child's rows (p2, p1,
+// (p0 + p1) / 2) of the parent's and an even one's (p0, p2, (p0 + p1) / 2), so
+// p0 = 2 r2 - r1 (odd) and p1 = 2 r2 - r0 (even).
+template <typename T>
+__device__ __forceinline__ void parent_row(const T a[6], bool odd, int d, T w[3]) {
+#pragma unroll
+    for (int c = 0; c < 2; ++c) w[c] = a[4 + c] + a[4 + c] - (odd ? a[2 + c] : a[c]);
+    w[2] = unit_of(T(), d) - w[0] - w[1];
+}
+
+// A weight in FP32 (w = float(W) 2^-d) and FP64. A float one (M, exact) is
+// widened by its bits; an integer one below 2^52 becomes FP64 at an exponent
+// whose last place is 2^-d, minus that power: both exact, and cheaper here
+// than FP64 conversions and a scaling.
+__device__ __forceinline__ float weight_f32(float w, int) { return w; }
+__device__ __forceinline__ float weight_f32(u64 w, int d) { return __fmul_rn(__ull2float_rn(w), pow2f(-d)); }
+__device__ __forceinline__ double weight_f64(float w, int) {
+    const uint32_t b = __float_as_uint(w);
+    return b ? __hiloint2double((int)((b >> 3) + (896u << 20)), (int)(b << 29)) : 0.0;
+}
+__device__ __forceinline__ double weight_f64(u64 w, int d) {
+    if (d > 51) return __dmul_rn(__ull2double_rn(w), pow2d(-d));
+    const double one = pow2d(52 - d);
+    return __dsub_rn(__longlong_as_double(__double_as_longlong(one) | (long long)w), one);
+}
+
+// Correctly rounded signed 128-bit integer (hi 2^64 + lo) -> float: the
+// magnitude's top 32 bits with a sticky bit for the rest, one RN conversion,
+// one exact scaling.
+__device__ __forceinline__ float s128_to_float(long long hi, u64 lo) {
+    const bool neg = hi < 0;
+    u64 h = (u64)hi;
+    if (neg) {
+        lo = 0ull - lo;
+        h = ~h + (lo == 0ull ? 1ull : 0ull);
+    }
+    int e = 96;
+    if (h == 0ull) {
+        h = lo;
+        lo = 0ull;
+        e = 32;
+    }
+    const int lz = __clzll((long long)h);
+    if (lz == 64) return 0.0f;
+    const u64 z = (h << lz) | ((lo >> 1) >> (63 - lz));
+    const uint32_t rest = (uint32_t)z | (uint32_t)((lo << lz) != 0ull);
+    const float f = __uint2float_rn((uint32_t)(z >> 32) | (rest ? 1u : 0u));
+    const float m = __fmul_rn(f, pow2f(e - lz));
+    return neg ? -m : m;
+}
+
+// Fixed point: the exact sum over the root's vertices of weight times
+// coordinate. Weights below 2^25 (float ones, d <= 24) take six 32 x 32 -> 64
+// multiply-adds per coordinate, sum = mid 2^32 + lo; wider ones (d <= 48) are
+// split into two 24-bit parts, so that no partial sum overflows either;
+// beyond, the general 128-bit product.
+struct S128 {
+    long long hi;
+    u64 lo;
+};
+__device__ __forceinline__ S128 s128_from(long long mid, u64 lo) {  // mid 2^32 + lo
+    const u64 l = lo + ((u64)mid << 32);
+    return S128{(mid >> 32) + (l < lo ? 1ll : 0ll), l};
+}
+__device__ __forceinline__ S128 s128_add(S128 a, S128 b) {
+    const u64 l = a.lo + b.lo;
+    return S128{a.hi + b.hi + (l < a.lo ? 1ll : 0ll), l};
+}
+__device__ __forceinline__ void fixed_sum(const uint32_t w[3], const long long* X, int c, S128& out) {
+    u64 lo = 0ull;
+    long long mid = 0;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const long long x = X[3 * i + c];
+        lo += (u64)w[i] * (u64)(uint32_t)x;
+        mid += (long long)(int)w[i] * (long long)(int)(x >> 32);
+    }
+    out = s128_from(mid, lo);
+}
+__device__ __forceinline__ void fixed_sum(const u64 w[3], int d, const long long* X, int c, S128& out) {
+    if (d <= 48) {
+        uint32_t l[3], h[3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            l[i] = (uint32_t)w[i] & 0xFFFFFFu;
+            h[i] = (uint32_t)(w[i] >> 24);
+        }
+        S128 a, b;
+        fixed_sum(l, X, c, a);
+        fixed_sum(h, X, c, b);
+        b.hi = (long long)(((u64)b.hi << 24) | (b.lo >> 40));
+        b.lo <<= 24;
+        out = s128_add(a, b);
+        return;
+    }
+    __int128 s = 0;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) s += (__int128)w[i] * (__int128)X[3 * i + c];
+    out = S128{(long long)(s >> 64), (u64)s};
+}
+
+__device__ __forceinline__ void fixed_coord(const float w[3], int d, const long long* X, int c, S128& out) {
+    uint32_t u[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) u[i] = __float2uint_rn(__fmul_rn(w[i], pow2f(d)));
+    fixed_sum(u, X, c, out);
+}
+__device__ __forceinline__ void fixed_coord(const u64 w[3], int d, const long long* X, int c, S128& out) {
+    fixed_sum(w, d, X, c, out);
 }
 
 // ------------------------------------------------------------ displacement
@@ -482,7 +592,10 @@ static __device__ __noinline__ float fbm3(float x0, float x1, float x2, float fr
 // Forms whose vertices the one-launch frame caches from its LOD test for the
 // export (a sphere projection or a displacement costs more to evaluate again
 // than 36 bytes cost to store and load).
-__device__ __forceinline__ bool vc_form(const FrameP& fp) { return fp.precision == 3u || fp.damp != 0.0f; }
+template <int F>
+__device__ __forceinline__ bool vc_form(const FrameP& fp) {
+    return precision_in<F>(fp) == 3u || displaced_in<F>(fp);
+}
 
 // FP32 form: z += amplitude * fbm2 of the world (x, y), the vertex plus the
 // origin rounded to FP32.
@@ -512,12 +625,8 @@ __device__ __forceinline__ void displace_plain(float r[3], const FrameP& fp) {
 // f}, f = radius' y (V: the root triangle's absolute FP64 vertices). It
 // depends on the heap ID, the mesh, the radius and the displacement only.
 template <typename T>
-__device__ __forceinline__ void sphere_point(const T W[9], int v, int d, const FrameP& fp, const double* V,
-                                             double pf[4]) {
-    const double sc = pow2d(-d);
-    const double w0 = __dmul_rn(wdouble(W[3 * v + 0]), sc);
-    const double w1 = __dmul_rn(wdouble(W[3 * v + 1]), sc);
-    const double w2 = __dmul_rn(wdouble(W[3 * v + 2]), sc);
+__device__ __forceinline__ void sphere_point(const T w[3], int d, const FrameP& fp, const double* V, double pf[4]) {
+    const double w0 = weight_f64(w[0], d), w1 = weight_f64(w[1], d), w2 = weight_f64(w[2], d);
     double p[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) p[c] = __fma_rn(w2, V[6 + c], __fma_rn(w1, V[3 + c], __dmul_rn(w0, V[c])));
@@ -546,29 +655,33 @@ __device__ __forceinline__ void sphere_rel(double px, double py, double pz, doub
     r[2] = __double2float_rn(__fma_rn(pz, f, -fp.eye[2]));
 }
 
-template <typename T>
-__device__ __forceinline__ void eval_vertex(const T W[9], int v, int d, const FrameP& fp, const void* rel,
-                                            uint32_t h, float r[3]) {
-    const uint32_t precision = fp.precision;
-    if (precision == 3) {
+// FP32: weights rounded to FP32, root vertices R.
+__device__ __forceinline__ void plain_vertex(const float w[3], const float R[9], float r[3]) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+        r[c] = __fadd_rn(__fadd_rn(__fmul_rn(w[0], R[c]), __fmul_rn(w[1], R[3 + c])), __fmul_rn(w[2], R[6 + c]));
+}
+
+// One vertex with weights w over 2^d (rel: the root tables, h the root).
+template <int F, typename T>
+__device__ __forceinline__ void eval_vertex(const T w[3], int d, const FrameP& fp, const void* rel, uint32_t h,
+                                            float r[3]) {
+    const uint32_t precision = precision_in<F>(fp);
+    if (precision == 3u) {
         double pf[4];
-        sphere_point<T>(W, v, d, fp, static_cast<const double*>(rel) + 9u * h, pf);
+        sphere_point<T>(w, d, fp, static_cast<const double*>(rel) + 9u * h, pf);
         sphere_rel(pf[0], pf[1], pf[2], pf[3], fp, r);
-    } else if (precision == 1) {
+    } else if (precision == 1u) {
         const long long* X = static_cast<const long long*>(rel) + 9u * h;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            __int128 s = (__int128)(unsigned long long)W[3 * v + 0] * (__int128)X[c];
-            s += (__int128)(unsigned long long)W[3 * v + 1] * (__int128)X[3 + c];
-            s += (__int128)(unsigned long long)W[3 * v + 2] * (__int128)X[6 + c];
-            r[c] = __fmul_rn(i128_to_float(s), pow2f(-(d + fp.shift)));
+            S128 s;
+            fixed_coord(w, d, X, c, s);
+            r[c] = __fmul_rn(s128_to_float(s.hi, s.lo), pow2f(-(d + fp.shift)));
         }
-    } else if (precision == 2) {
+    } else if (precision == 2u) {
         const double* Dp = static_cast<const double*>(rel) + 9u * h;
-        const double sc = pow2d(-d);
-        const double w0 = __dmul_rn(wdouble(W[3 * v + 0]), sc);
-        const double w1 = __dmul_rn(wdouble(W[3 * v + 1]), sc);
-        const double w2 = __dmul_rn(wdouble(W[3 * v + 2]), sc);
+        const double w0 = weight_f64(w[0], d), w1 = weight_f64(w[1], d), w2 = weight_f64(w[2], d);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             const double t = __dadd_rn(__dadd_rn(__dmul_rn(w0, Dp[c]), __dmul_rn(w1, Dp[3 + c])),
@@ -577,67 +690,9 @@ __device__ __forceinline__ void eval_vertex(const T W[9], int v, int d, const Fr
         }
     } else {
         const float* R = static_cast<const float*>(rel) + 9u * h;
-        const float sc = pow2f(-d);
-        const float w0 = __fmul_rn(wfloat(W[3 * v + 0]), sc);
-        const float w1 = __fmul_rn(wfloat(W[3 * v + 1]), sc);
-        const float w2 = __fmul_rn(wfloat(W[3 * v + 2]), sc);
-#pragma unroll
-        for (int c = 0; c < 3; ++c)
-            r[c] = __fadd_rn(__fadd_rn(__fmul_rn(w0, R[c]), __fmul_rn(w1, R[3 + c])), __fmul_rn(w2, R[6 + c]));
-        if (fp.damp != 0.0f) displace_plain(r, fp);
-    }
-}
-
-// All three vertices, r[3 v + c] (the same roundings as eval_vertex; the
-// root table is read once for the three).
-template <typename T>
-__device__ __forceinline__ void eval_vertices(const T W[9], int d, const FrameP& fp, const void* rel, uint32_t h,
-                                              float r[9]) {
-    const uint32_t precision = fp.precision;
-    if (precision == 3) {
-#pragma unroll
-        for (int v = 0; v < 3; ++v) eval_vertex<T>(W, v, d, fp, rel, h, r + 3 * v);
-    } else if (precision == 1) {
-        const long long* X = static_cast<const long long*>(rel) + 9u * h;
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                __int128 s = (__int128)(unsigned long long)W[3 * i + 0] * (__int128)X[c];
-                s += (__int128)(unsigned long long)W[3 * i + 1] * (__int128)X[3 + c];
-                s += (__int128)(unsigned long long)W[3 * i + 2] * (__int128)X[6 + c];
-                r[3 * i + c] = __fmul_rn(i128_to_float(s), pow2f(-(d + fp.shift)));
-            }
-    } else if (precision == 2) {
-        const double* Dp = static_cast<const double*>(rel) + 9u * h;
-        const double sc = pow2d(-d);
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            const double w0 = __dmul_rn(wdouble(W[3 * i + 0]), sc);
-            const double w1 = __dmul_rn(wdouble(W[3 * i + 1]), sc);
-            const double w2 = __dmul_rn(wdouble(W[3 * i + 2]), sc);
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                const double t = __dadd_rn(__dadd_rn(__dmul_rn(w0, Dp[c]), __dmul_rn(w1, Dp[3 + c])),
-                                           __dmul_rn(w2, Dp[6 + c]));
-                r[3 * i + c] = __double2float_rn(t);
-            }
-        }
-    } else {
-        const float* R = static_cast<const float*>(rel) + 9u * h;
-        const float sc = pow2f(-d);
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            const float w0 = __fmul_rn(wfloat(W[3 * i + 0]), sc);
-            const float w1 = __fmul_rn(wfloat(W[3 * i + 1]), sc);
-            const float w2 = __fmul_rn(wfloat(W[3 * i + 2]), sc);
-#pragma unroll
-            for (int c = 0; c < 3; ++c)
-                r[3 * i + c] = __fadd_rn(__fadd_rn(__fmul_rn(w0, R[c]), __fmul_rn(w1, R[3 + c])), __fmul_rn(w2, R[6 + c]));
-        }
-        if (fp.damp != 0.0f)
-#pragma unroll
-            for (int i = 0; i < 3; ++i) displace_plain(r + 3 * i, fp);
+        const float wf[3] = {weight_f32(w[0], d), weight_f32(w[1], d), weight_f32(w[2], d)};
+        plain_vertex(wf, R, r);
+        if (displaced_in<F>(fp)) displace_plain(r, fp);
     }
 }
 
@@ -671,14 +726,6 @@ __device__ __forceinline__ bool edge_big(const float* a, const float* b, float q
     const float R2 = __fadd_rn(__fadd_rn(__fmul_rn(mx, mx), __fmul_rn(my, my)), __fmul_rn(mz, mz));
     return __fmul_rn(L2, q) > R2;
 }
-// bit0 visible, bit1 big.
-__device__ __forceinline__ uint32_t lod_test(const float r[9], const FrameP& fp) {
-    uint32_t out = plane_mask(r, fp);
-    if (out) out = plane_mask(r + 3, fp, out);
-    if (out) out = plane_mask(r + 6, fp, out);
-    return (out == 0u ? 1u : 0u) | (edge_big(r, r + 3, fp.q) ? 2u : 0u);
-}
-
 __device__ __forceinline__ bool in_sorted(const uint64_t* a, uint32_t n, uint64_t x) {
     uint32_t lo = 0, hi = n;
     while (lo < hi) {

@@ -20,6 +20,7 @@
 // blocks wrote in an earlier phase follow a barrier whose fences order them.
 // Every wait is bounded: a barrier that runs out sets the batch's abort word,
 // every later wait then returns at once, and the instances report kErrTimeout.
+#pragma once
 #include "cbt_kernels.cuh"
 #include "cbt_phases.cuh"
 
@@ -266,10 +267,11 @@ __device__ __forceinline__ void walk_list(const Inst& I, const uint2* s_list, ui
     }
 }
 
+template <int F>
 __device__ __forceinline__ void classify_one(const Inst& I, const FrameP& fp, uint64_t key, uint32_t i, uint32_t s,
                                              uint64_t j, const uint32_t* s_tab, uint32_t* s_cnt, bool chain,
                                              uint32_t* s_n, uint2* s_list) {
-    const uint32_t cmd = classify_item(I, fp, key, i, s, j, s_tab, s_cnt, vc_form(fp) && fp.vout);
+    const uint32_t cmd = classify_item<F>(I, fp, key, i, s, j, s_tab, s_cnt, vc_form<F>(fp) && fp.vout);
     const bool split = (cmd & kSplitWish) && chain;
     const bool group = (cmd & kMergeWish) && !(cmd & kHeapOdd);
     if (split || group) s_list[atomicAdd(s_n, 1u)] = make_uint2(i | (split ? 0x80000000u : 0u), s);
@@ -282,6 +284,7 @@ constexpr uint32_t kWalkCap = kFBuf / 2;  // uint2 entries of the walk list
 // strides its live list over the whole grid (balanced; the slot and heap ID
 // of the next rounds are loaded while the current item is classified); a
 // batch walks its item tiles.
+template <int F>
 __device__ void phase_classify(const BatchDev& bt, FCtx& c, uint32_t* s_tab, uint32_t* s_cnt, uint32_t* s_n,
                                uint2* s_list) {
     if (bt.B == 1) {
@@ -301,7 +304,7 @@ __device__ void phase_classify(const BatchDev& bt, FCtx& c, uint32_t* s_tab, uin
         for (uint32_t base = blockIdx.x * kFThreads; base < N; base += stride, i += stride) {
             const uint32_t sc = i + 2u * stride < N ? I.live[i + 2u * stride] : 0u;
             const uint64_t jb = i + stride < N ? I.heap[sb] : 0ull;
-            if (i < N) classify_one(I, fp, key, i, sa, ja, s_tab, s_cnt, chain, s_n, s_list);
+            if (i < N) classify_one<F>(I, fp, key, i, sa, ja, s_tab, s_cnt, chain, s_n, s_list);
             sa = sb;
             ja = jb;
             sb = sc;
@@ -348,7 +351,12 @@ __device__ void phase_classify(const BatchDev& bt, FCtx& c, uint32_t* s_tab, uin
 #pragma unroll 1
         for (int k = 0; k < kFPer; ++k) {
             const uint32_t i = lt * kTileItems + (uint32_t)k * kFThreads + threadIdx.x;
-            if (i < N) classify_one(I, fp, key, i, sl[k], hj[k], s_tab, s_cnt, chain, s_n, s_list);
+            if (i < N) classify_one<F>(I, fp, key, i, sl[0], hj[0], s_tab, s_cnt, chain, s_n, s_list);
+#pragma unroll
+            for (int q = 0; q + 1 < kFPer; ++q) {  // constant indices: registers, not local memory
+                sl[q] = sl[q + 1];
+                hj[q] = hj[q + 1];
+            }
         }
         __syncthreads();
         walk_list(I, s_list, *s_n);
@@ -876,6 +884,7 @@ __device__ void phase_reduce(const BatchDev& bt, FCtx& c, uint32_t* s_buf, uint3
 // P8: CachePointers (Alg. 7 for every rank at once) per word tile, and, in a
 // batch, the FP32 vertices of the tile's live bisectors when the frame
 // exports them.
+template <int F>
 __device__ void phase_compact(const BatchDev& bt, FCtx& c, const uint32_t* s_tab, uint32_t* s_buf,
                               uint32_t* s_w) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -931,7 +940,7 @@ __device__ void phase_compact(const BatchDev& bt, FCtx& c, const uint32_t* s_tab
             const uint32_t lim = fp.vcap;
             for (uint32_t k = threadIdx.x; k < tot; k += blockDim.x) {
                 const uint32_t i = before + k;
-                if (i < lim) vertex_item_cached(I, fp, i, s_buf[k], s_tab, fp.vout);
+                if (i < lim) vertex_item_cached<F>(I, fp, i, s_buf[k], s_tab, fp.vout);
             }
         }
         __syncthreads();
@@ -951,16 +960,17 @@ __device__ void phase_compact(const BatchDev& bt, FCtx& c, const uint32_t* s_tab
 // evaluate), and the new ones are listed and evaluated densely by the block
 // (so that no warp idles beside one evaluating lane); otherwise the slot and
 // heap ID of the next round are loaded while the current one is evaluated.
+template <int F>
 __device__ void vertices_of(const Inst& I, const FrameP& fp, const uint32_t* s_tab, uint32_t* s_list,
                             uint32_t* s_n) {
     if (!fp.vout) return;
     const uint32_t n = min(__ldcg(I.sums + 1), fp.vcap);
     const uint32_t stride = gridDim.x * kFThreads;
-    if (vc_form(fp)) {
+    if (vc_form<F>(fp)) {
         auto evaluate = [&](uint32_t cnt) {
             for (uint32_t q = threadIdx.x; q < cnt; q += kFThreads) {
                 const uint32_t i = s_list[q];
-                vertex_item(I, fp, i, I.heap[I.live[i]], s_tab, fp.vout);
+                vertex_item<F>(I, fp, i, I.heap[I.live[i]], s_tab, fp.vout);
             }
         };
         if (threadIdx.x == 0) *s_n = 0;
@@ -1009,13 +1019,20 @@ __device__ void vertices_of(const Inst& I, const FrameP& fp, const uint32_t* s_t
     const uint32_t lane = threadIdx.x & 31u;
     float* stage = reinterpret_cast<float*>(s_list) + 288u * (threadIdx.x >> 5);
     uint32_t w0 = ((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32u;
-    uint64_t j = w0 + lane < n ? I.heap[I.live[w0 + lane]] : 0ull;
+    // the heap ID one round ahead and its slot two, so that no load waits on
+    // one issued in the same round
+    const uint32_t* const live = I.live;
+    const uint64_t* const heap = I.heap;
+    uint64_t j = w0 + lane < n ? heap[live[w0 + lane]] : 0ull;
+    uint32_t sb = w0 + lane + stride < n ? live[w0 + lane + stride] : 0u;
     for (; w0 < n; w0 += stride) {
         const uint32_t i = w0 + lane;
-        const uint64_t jn = i + stride < n ? I.heap[I.live[i + stride]] : 0ull;
+        const uint32_t sc = i + 2u * stride < n ? live[i + 2u * stride] : 0u;
+        const uint64_t jn = i + stride < n ? heap[sb] : 0ull;
+        sb = sc;
         float r[9];
         bool ok = true;
-        if (i < n) ok = vertex_eval(I, fp, j, s_tab, r);
+        if (i < n) ok = vertex_eval<F>(I, fp, j, s_tab, r);
         if (__all_sync(0xFFFFFFFFu, ok)) {
             warp_rows_out(r, stage, fp.vout, w0, min(32u, n - w0));
         } else if (i < n && ok) {  // a row the decode refused stays unwritten
@@ -1026,12 +1043,14 @@ __device__ void vertices_of(const Inst& I, const FrameP& fp, const uint32_t* s_t
         j = jn;
     }
 }
+template <int F>
 __device__ void phase_vertices(const BatchDev& bt, FCtx& c, const uint32_t* s_tab, uint32_t* s_list,
                                uint32_t* s_n) {
     ctx_tile(bt, bt.tile_base, 0, 1, c);
-    vertices_of(c.I, c.fp, s_tab, s_list, s_n);
+    vertices_of<F>(c.I, c.fp, s_tab, s_list, s_n);
 }
 
+template <int F>
 __global__ void __launch_bounds__(kFThreads, CBT_FRAME_MIN_BLOCKS) k_frame(BatchDev bt) {
     __shared__ FCtx s_c;
     __shared__ __align__(16) uint32_t s_tab[kDecTabWords];
@@ -1051,7 +1070,7 @@ __global__ void __launch_bounds__(kFThreads, CBT_FRAME_MIN_BLOCKS) k_frame(Batch
     phase_prep(bt, s_warp, s_tmp);
     grid_sync(bt.bg, epoch, 1u);
     stamp(bt, 1);
-    phase_classify(bt, s_c, s_tab, s_cnt, &s_n, reinterpret_cast<uint2*>(s_buf));
+    phase_classify<F>(bt, s_c, s_tab, s_cnt, &s_n, reinterpret_cast<uint2*>(s_buf));
     grid_sync(bt.bg, epoch, 2u);
     stamp(bt, 2);
     phase_gate_sum(bt, s_c, s_cnt, s_red, &s_n, s_buf);
@@ -1072,11 +1091,11 @@ __global__ void __launch_bounds__(kFThreads, CBT_FRAME_MIN_BLOCKS) k_frame(Batch
     phase_reduce(bt, s_c, s_buf, &s_tmp[0]);
     grid_sync(bt.bg, epoch, 8u);
     stamp(bt, 8);
-    phase_compact(bt, s_c, s_tab, s_buf, s_w);
+    phase_compact<F>(bt, s_c, s_tab, s_buf, s_w);
     if (bt.B == 1) {
         grid_sync(bt.bg, epoch, 9u);
         stamp(bt, 9);
-        phase_vertices(bt, s_c, s_tab, s_buf, &s_n);
+        phase_vertices<F>(bt, s_c, s_tab, s_buf, &s_n);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -1341,6 +1360,7 @@ __device__ __forceinline__ void warp_walks_out(const Inst& I, const uint4* s_wl,
     __syncwarp();
 }
 
+template <int F>
 __device__ void phase_classify1(const BatchDev& bt, FCtx& c, uint32_t* s_tab, uint32_t* s_cnt, uint4* s_list) {
     stats_reset(s_cnt);
     ctx_tile(bt, bt.tile_base, 0, 1, c);
@@ -1350,7 +1370,7 @@ __device__ void phase_classify1(const BatchDev& bt, FCtx& c, uint32_t* s_tab, ui
     const uint32_t S = kFThreads * bt.bg->scan_ipt;
     unsigned long long* wc = wish_counts(bt);
     const uint64_t key = splitmix64(((uint64_t)fp.seed << 32) | (uint64_t)fp.frame);
-    const bool cache = vc_form(fp) && fp.vout;
+    const bool cache = vc_form<F>(fp) && fp.vout;
     const uint32_t lane = threadIdx.x & 31u;
     uint4* s_wl = s_list + kWarpWalks * (threadIdx.x >> 5);  // the warp's walk buffer
     uint32_t nwl = 0;                                           // its entries (warp-uniform)
@@ -1368,7 +1388,7 @@ __device__ void phase_classify1(const BatchDev& bt, FCtx& c, uint32_t* s_tab, ui
         const uint64_t jb = i + stride < N ? I.heap[sb] : 0ull;
         bool split = false, walk = false, interior = false;
         if (i < N) {
-            const uint32_t cmd = classify_item(I, fp, key, i, sa, ja, s_tab, s_cnt, cache);
+            const uint32_t cmd = classify_item<F>(I, fp, key, i, sa, ja, s_tab, s_cnt, cache);
             split = (cmd & kSplitWish) != 0u;
             walk = split || ((cmd & kMergeWish) && !(cmd & kHeapOdd));
             // every bisector under a root whose halfedge has a Twin has one
@@ -1378,17 +1398,15 @@ __device__ void phase_classify1(const BatchDev& bt, FCtx& c, uint32_t* s_tab, ui
             const uint32_t h = d >= 0 ? (uint32_t)((ja >> d) - (1ull << I.ch)) : kNull;
             interior = split && h < I.H && !((__ldg(I.rbnd + (h >> 5)) >> (h & 31u)) & 1u);
         }
-        const unsigned wm = __ballot_sync(0xFFFFFFFFu, walk);
+        const unsigned wm = __ballot_sync(0xFFFFFFFFu, walk), sm = __ballot_sync(0xFFFFFFFFu, split);
         if (walk)
             s_wl[nwl + __popc(wm & ((1u << lane) - 1u))] =
                 make_uint4(i | (split ? kWalkSplit : 0u) | (interior ? kWalkInterior : 0u), sa, (uint32_t)ja,
                            (uint32_t)(ja >> 32));
         nwl += __popc(wm);
-        {  // the split wishes' lower-bound costs per scan tile
-            const uint32_t t = i / S;
-            const unsigned m = __match_any_sync(0xFFFFFFFFu, i < N ? t : kNull);
-            const uint32_t lb = __reduce_add_sync(m, split ? (interior ? 4u : 2u) : 0u);
-            if (lb && lane == (uint32_t)(__ffs(m) - 1)) atomicAdd(&wc[t], (unsigned long long)lb);
+        if (sm) {  // the split wishes' lower-bound costs per scan tile (S is a multiple of 32: one tile per round)
+            const uint32_t lb = 2u * (__popc(sm) + __popc(__ballot_sync(0xFFFFFFFFu, interior)));
+            if (lane == 0u) atomicAdd(&wc[(i - lane) / S], (unsigned long long)lb);
         }
         sa = sb;
         ja = jb;
@@ -1932,6 +1950,7 @@ __device__ void phase_final1(const BatchDev& bt, FCtx& c, uint32_t* s_buf, Pair*
     }
 }
 
+template <int F>
 __global__ void __launch_bounds__(kFThreads, CBT_FRAME_MIN_BLOCKS) k_frame1(BatchDev bt, uint32_t tbits) {
     __shared__ FCtx s_c;
     __shared__ __align__(16) uint32_t s_tab[kDecTabWords];
@@ -1954,14 +1973,14 @@ __global__ void __launch_bounds__(kFThreads, CBT_FRAME_MIN_BLOCKS) k_frame1(Batc
     // the decode tables are fetched now and stored after prep's own loads
     // have gone out
     static_assert(kFThreads == 256, "dec_fetch splits the table over 256 threads");
-    uint4 tab[kDecVecs / 256u + 1u];
+    uint4 tab[kDecVecs];
     dec_fetch(tab);
     if (threadIdx.x == 0) s_c.b = kNull;
     phase_prep1(bt, tbits);
     dec_store(s_tab, tab);
     sync();
     stamp(bt, 1);
-    phase_classify1(bt, s_c, s_tab, s_cnt, reinterpret_cast<uint4*>(s_buf));
+    phase_classify1<F>(bt, s_c, s_tab, s_cnt, reinterpret_cast<uint4*>(s_buf));
     sync();
     stamp(bt, 2);
     phase_walks1(bt, s_c, s_cnt, s_buf, s_warp, s_tmp, &s_n);
@@ -1984,7 +2003,7 @@ __global__ void __launch_bounds__(kFThreads, CBT_FRAME_MIN_BLOCKS) k_frame1(Batc
     if (bt.fp0.vout) {
         sync();
         stamp(bt, 7);
-        vertices_of(bt.inst0, bt.fp0, s_tab, s_buf, &s_n);
+        vertices_of<F>(bt.inst0, bt.fp0, s_tab, s_buf, &s_n);
     } else {
         stamp(bt, 7);
     }
@@ -2000,57 +2019,37 @@ __global__ void __launch_bounds__(kFThreads, CBT_FRAME_MIN_BLOCKS) k_frame1(Batc
 
 }  // namespace
 
-cudaError_t launch_wait_selftest(BatchGlobals* bg, int blocks, int limit, cudaStream_t s) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(blocks));
-    cfg.blockDim = dim3(kFThreads);
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_wait_selftest, bg, limit);
-}
-
-int frame_blocks_per_sm() {
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_frame, kFThreads, 0) != cudaSuccess) return 0;
-    return n;
-}
-
-int frame1_blocks_per_sm() {
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_frame1, kFThreads, 0) != cudaSuccess) return 0;
-    return n;
-}
-
-cudaError_t launch_frame1(const BatchDev& bt, int grid, uint32_t tbits, cudaStream_t s) {
+template <typename... A>
+cudaError_t launch_coop(void (*kernel)(A...), int grid, cudaStream_t s, A... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(grid));
     cfg.blockDim = dim3(kFThreads);
-    cfg.dynamicSmemBytes = 0;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_frame1, bt, tbits);
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-cudaError_t launch_frame(const BatchDev& bt, int grid, cudaStream_t s) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(grid));
-    cfg.blockDim = dim3(kFThreads);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_frame, bt);
+template <int F>
+cudaError_t launch_frame_form(const BatchDev& bt, int grid, cudaStream_t s) {
+    return launch_coop<BatchDev>(k_frame<F>, grid, s, bt);
+}
+template <int F>
+cudaError_t launch_frame1_form(const BatchDev& bt, int grid, uint32_t tbits, cudaStream_t s) {
+    return launch_coop<BatchDev, uint32_t>(k_frame1<F>, grid, s, bt, tbits);
+}
+template <int F>
+int frame_blocks_form() {
+    int n = 0;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_frame<F>, kFThreads, 0) == cudaSuccess ? n : 0;
+}
+template <int F>
+int frame1_blocks_form() {
+    int n = 0;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_frame1<F>, kFThreads, 0) == cudaSuccess ? n : 0;
 }
 
 }  // namespace cbtgpu

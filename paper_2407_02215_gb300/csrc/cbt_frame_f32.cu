@@ -1,0 +1,11 @@
+// The one-launch frames compiled for one vertex form.
+#include "cbt_frame.cuh"
+
+namespace cbtgpu {
+
+template cudaError_t launch_frame_form<kFormF32>(const BatchDev&, int, cudaStream_t);
+template int frame_blocks_form<kFormF32>();
+template cudaError_t launch_frame1_form<kFormF32>(const BatchDev&, int, uint32_t, cudaStream_t);
+template int frame1_blocks_form<kFormF32>();
+
+}  // namespace cbtgpu

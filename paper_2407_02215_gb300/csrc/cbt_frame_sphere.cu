@@ -1,0 +1,9 @@
+// The one-launch frames compiled for one vertex form.
+#include "cbt_frame.cuh"
+
+namespace cbtgpu {
+
+template cudaError_t launch_frame1_form<kFormSphere>(const BatchDev&, int, uint32_t, cudaStream_t);
+template int frame1_blocks_form<kFormSphere>();
+
+}  // namespace cbtgpu

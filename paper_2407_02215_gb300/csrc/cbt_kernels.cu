@@ -124,6 +124,7 @@ __global__ void __launch_bounds__(kThreads) k_walk(BatchDev bt) {
     }
 }
 
+template <int F>
 __global__ void __launch_bounds__(kThreads, 3) k_classify(BatchDev bt) {
     __shared__ uint32_t s_b;
     __shared__ Inst s_I;
@@ -155,7 +156,12 @@ __global__ void __launch_bounds__(kThreads, 3) k_classify(BatchDev bt) {
 #pragma unroll 1
         for (int k = 0; k < kItemsPerThread; ++k) {
             const uint32_t i = lt * kTileItems + (uint32_t)k * kThreads + threadIdx.x;
-            if (i < N) classify_item(I, fp, key, i, sl[k], hj[k], s_tab, s_cnt);
+            if (i < N) classify_item<F>(I, fp, key, i, sl[0], hj[0], s_tab, s_cnt);
+#pragma unroll
+            for (int q = 0; q + 1 < kItemsPerThread; ++q) {  // constant indices: registers, not local memory
+                sl[q] = sl[q + 1];
+                hj[q] = hj[q + 1];
+            }
         }
         __syncthreads();
         stats_flush(s_cnt, I.g, kStSplitWishes);
@@ -639,6 +645,7 @@ __global__ void __launch_bounds__(kThreads) k_leaves(Inst I, uint32_t* slots, ui
 }
 
 // over static tiles of its pool capacity (tiles past the live count exit).
+template <int F>
 __global__ void __launch_bounds__(kThreads, 3) k_vertices(BatchDev bt) {
     __shared__ uint32_t s_b;
     __shared__ Inst s_I;
@@ -667,7 +674,9 @@ __global__ void __launch_bounds__(kThreads, 3) k_vertices(BatchDev bt) {
                 if (w0 >= N) continue;
                 float r[9];
                 bool ok = true;
-                if (i < N) ok = vertex_eval(I, fp, hj[k], s_tab, r);
+                if (i < N) ok = vertex_eval<F>(I, fp, hj[0], s_tab, r);
+#pragma unroll
+                for (int q = 0; q + 1 < kItemsPerThread; ++q) hj[q] = hj[q + 1];  // registers, not local memory
                 if (__all_sync(0xFFFFFFFFu, ok)) {
                     warp_rows_out(r, s_stage[threadIdx.x >> 5], fp.vout, w0, min(32u, N - w0));
                 } else if (i < N && ok) {  // a row the decode refused stays unwritten
@@ -686,7 +695,13 @@ __global__ void __launch_bounds__(kThreads, 3) k_vertices(BatchDev bt) {
 void launch_prep(const BatchDev& bt, bool frame_start, int grid, cudaStream_t s) {
     k_prep<<<grid, kThreads, 0, s>>>(bt, frame_start ? 1 : 0);
 }
-void launch_classify(const BatchDev& bt, int grid, cudaStream_t s) { k_classify<<<grid, kThreads, 0, s>>>(bt); }
+void launch_classify(const BatchDev& bt, int form, int grid, cudaStream_t s) {
+    switch (form) {
+        case kFormF32: k_classify<kFormF32><<<grid, kThreads, 0, s>>>(bt); break;
+        case kFormFixed: k_classify<kFormFixed><<<grid, kThreads, 0, s>>>(bt); break;
+        default: k_classify<kFormAny><<<grid, kThreads, 0, s>>>(bt); break;
+    }
+}
 void launch_walk(const BatchDev& bt, int grid, cudaStream_t s) { k_walk<<<grid, kThreads, 0, s>>>(bt); }
 void launch_gate(const BatchDev& bt, int grid, cudaStream_t s) { k_gate<<<grid, kScanThreads, 0, s>>>(bt); }
 void launch_scatter(const BatchDev& bt, int grid, cudaStream_t s) { k_scatter<<<grid, kThreads, 0, s>>>(bt); }
@@ -697,7 +712,13 @@ void launch_cbt(const BatchDev& bt, int grid, cudaStream_t s) {
     k_cbt<<<grid, bt.tw, 0, s>>>(bt);
     k_compact<<<grid, bt.tw, 0, s>>>(bt);
 }
-void launch_vertices(const BatchDev& bt, int grid, cudaStream_t s) { k_vertices<<<grid, kThreads, 0, s>>>(bt); }
+void launch_vertices(const BatchDev& bt, int form, int grid, cudaStream_t s) {
+    switch (form) {
+        case kFormF32: k_vertices<kFormF32><<<grid, kThreads, 0, s>>>(bt); break;
+        case kFormFixed: k_vertices<kFormFixed><<<grid, kThreads, 0, s>>>(bt); break;
+        default: k_vertices<kFormAny><<<grid, kThreads, 0, s>>>(bt); break;
+    }
+}
 void launch_init(const Inst& I, const int32_t* twin, const int32_t* next, const int32_t* prev,
                  const double* hpos, int grid, cudaStream_t s) {
     k_init<<<grid, kThreads, 0, s>>>(I, twin, next, prev, hpos);

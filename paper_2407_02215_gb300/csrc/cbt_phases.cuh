@@ -1,8 +1,10 @@
 // Device functions shared by the per-step kernels (cbt_kernels.cu) and the
-// persistent one-launch-per-frame kernel (cbt_fused.cu): tile bookkeeping,
+// persistent one-launch-per-frame kernel (cbt_frame.cuh): tile bookkeeping,
 // block scans, the item-level steps of the frame and the word-tile steps
 // of the CBT.
 #pragma once
+#include <type_traits>
+
 #include "cbt_device.cuh"
 
 namespace cbtgpu {
@@ -312,20 +314,27 @@ static __device__ bool find_group(const Inst& I, uint32_t s1, Group& g) {
 
 // -------------------------------------------------------------- classify
 
-// The wishes from the bisector's camera-relative vertices r (R8 reading):
-// split = visible, big and below the maximum depth; merge = no split, depth
-// >= 1 and the parent not (visible and big). The parent's vertices are
-// {nv, r0, r1} (nv its new vertex, from new_vertex() only when needed), its
-// refinement edge (nv, r1) for an odd heap ID and (r0, nv) for an even one;
-// its plane masks for r0 and r1 are the child's.
-template <typename NV>
-__device__ __forceinline__ void wishes_from(const float r[9], bool odd, int d, uint32_t max_depth, const FrameP& fp,
-                                            NV new_vertex, bool& split, bool& merge) {
+// The wishes from the bisector's camera-relative vertices r0, r1 (R8
+// reading): split = visible, big and below the maximum depth; merge = no
+// split, depth >= 1 and the parent not (visible and big). The third vertex
+// (third(v)) and the parent's one that the bisector does not share
+// (new_vertex(v)) are asked for only when the answer needs them: a plane
+// culls only when r0 and r1 are both behind it. The parent's refinement edge
+// is (nv, r1) for an odd heap ID and (r0, nv) for an even one; its plane
+// masks for r0 and r1 are the child's.
+template <typename V2, typename NV>
+__device__ __forceinline__ void wishes_from(const float r[6], bool odd, int d, uint32_t max_depth, const FrameP& fp,
+                                            V2 third, NV new_vertex, bool& split, bool& merge) {
     // m01: the planes both r0 and r1 are behind (the parent's culling
     // candidates too); r2 and the parent's new vertex are tested only there
     const uint32_t m0 = plane_mask(r, fp);
     const uint32_t m01 = m0 ? plane_mask(r + 3, fp, m0) : 0u;
-    const uint32_t m012 = m01 ? plane_mask(r + 6, fp, m01) : 0u;
+    uint32_t m012 = 0u;
+    if (m01) {
+        float r2[3];
+        third(r2);
+        m012 = plane_mask(r2, fp, m01);
+    }
     const bool big = edge_big(r, r + 3, fp.q);
     split = m012 == 0u && big && d < (int)max_depth;
     merge = false;
@@ -343,30 +352,112 @@ __device__ __forceinline__ void wishes_from(const float r[9], bool odd, int d, u
     }
 }
 
-template <typename T>
-__device__ __forceinline__ void lod_wishes(const Inst& I, const FrameP& fp, uint64_t j, int d,
-                                           uint32_t h, const uint32_t* tab, bool& split, bool& merge,
-                                           float* keep) {
-    T W[9], Wp[9];
-    decode_weights<T>(j, d, W, Wp, tab);
-    float r[9];
-    eval_vertices<T>(W, d, fp, I.rel, h, r);
+// Which weights a bisector at depth d is decoded to: FP32 ones while they are
+// exact, else 64-bit integers. Outside FP32, whose evaluation is the same for
+// both, a warp with both kinds takes the integer path once rather than
+// running the evaluation twice (on the projected planet, with most warps
+// mixed, the two-path form made classify 62 us against 43 us).
+__device__ __forceinline__ bool float_weights(int d) { return !__any_sync(__activemask(), d > kFloatDepth); }
+
+// Rows of points to evaluate: the bisector's vertices 0 to 2, and (kRowParent)
+// the parent's vertex that it does not share.
+constexpr int kRowParent = 3;
+
+// The points of up to four rows of bisector j (the bits of `rows`, a compile-
+// time constant at the call) into r[3 row ..]. The root's data is read once
+// for all of them; FP32 weights come from one code path per decode only.
+template <int F>
+__device__ __forceinline__ void eval_rows(const FrameP& fp, const void* rel, uint64_t j, int d, uint32_t h,
+                                          const uint32_t* tab, const int rows, float r[12]) {
+    const bool odd = (j & 1ull) != 0ull;
+    if (F == kFormF32 || F == kFormF32Disp) {
+        const float* Rp = static_cast<const float*>(rel) + 9u * h;
+        float R[9], w[4][3];
+#pragma unroll
+        for (int k = 0; k < 9; ++k) R[k] = Rp[k];
+        if (d <= kFloatDepth) {
+            float a[6];
+            decode_cols(j, d, tab, a);
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                if (!((rows >> v) & 1)) continue;
+                if (v < 3)
+                    weight_row<float>(a, v, d, w[v]);
+                else
+                    parent_row<float>(a, odd, d, w[v]);
+            }
+        } else {
+            u64 a[6], u[3];
+            decode_cols(j, d, tab, a);
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                if (!((rows >> v) & 1)) continue;
+                if (v < 3)
+                    weight_row<u64>(a, v, d, u);
+                else
+                    parent_row<u64>(a, odd, d, u);
+#pragma unroll
+                for (int k = 0; k < 3; ++k) w[v][k] = weight_f32(u[k], d);
+            }
+        }
+#pragma unroll
+        for (int v = 0; v < 4; ++v)
+            if ((rows >> v) & 1) {
+                plain_vertex(w[v], R, r + 3 * v);
+                if (F == kFormF32Disp) displace_plain(r + 3 * v, fp);
+            }
+        return;
+    }
+    auto eval = [&](auto a) {
+        typedef typename std::remove_pointer<decltype(a)>::type T;
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            if (!((rows >> v) & 1)) continue;
+            T w[3];
+            if (v < 3)
+                weight_row<T>(a, v, d, w);
+            else
+                parent_row<T>(a, odd, d, w);
+            eval_vertex<F, T>(w, d, fp, rel, h, r + 3 * v);
+        }
+    };
+    if (float_weights(d)) {
+        float a[6];
+        decode_cols(j, d, tab, a);
+        eval(a);
+    } else {
+        u64 a[6];
+        decode_cols(j, d, tab, a);
+        eval(a);
+    }
+}
+
+// The wishes of bisector j by the LOD test; the vertices go to keep when it
+// is given (the forms whose export copies them). Two vertices of the parent
+// are the child's, and a weight row over 2^d evaluates to the same value as
+// its half over 2^(d - 1) in every precision form. The parent's third is
+// evaluated with the bisector's own (only the few split wishes do without
+// it). The bisector's third is rarely needed: the fixed-point and FP64 forms,
+// where it is not cheap, decode again where it is.
+template <int F>
+__device__ __forceinline__ void lod_wishes(const Inst& I, const FrameP& fp, uint64_t j, int d, uint32_t h,
+                                           const uint32_t* tab, bool& split, bool& merge, float* keep) {
+    constexpr bool kLazy = F == kFormFixed || F == kFormF64;
+    float r[12];
+    const bool odd = (j & 1ull) != 0ull;
+    eval_rows<F>(fp, I.rel, j, d, h, tab, kLazy ? 11 : 15, r);
     if (keep)
 #pragma unroll
         for (int k = 0; k < 9; ++k) keep[k] = r[k];
-    // Two vertices of the parent are the child's: a 0 bit makes the child's
-    // rows (2 r0, 2 r2, r0 + r1) of the parent's, a 1 bit (2 r2, 2 r1,
-    // r0 + r1) (Eq. 1), and a row doubled over a doubled denominator
-    // evaluates to the same value in every precision form. The new vertex is
-    // the parent's v0 (1 bit) or v1 (0 bit); the row is picked by selects so
-    // that every lane takes the same path.
-    const bool odd = (j & 1ull) != 0ull;
     wishes_from(r, odd, d, I.max_depth, fp,
-                [&](float nv[3]) {
-                    T row[9];
+                [&](float r2[3]) {
+                    if (kLazy) eval_rows<F>(fp, I.rel, j, d, h, tab, 4, r);
 #pragma unroll
-                    for (int k = 0; k < 3; ++k) row[k] = odd ? Wp[k] : Wp[3 + k];
-                    eval_vertex<T>(row, 0, d - 1, fp, I.rel, h, nv);
+                    for (int k = 0; k < 3; ++k) r2[k] = r[6 + k];
+                },
+                [&](float nv[3]) {
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) nv[k] = r[9 + k];
                 },
                 split, merge);
 }
@@ -383,30 +474,23 @@ __device__ __forceinline__ void lod_wishes(const Inst& I, const FrameP& fp, uint
 template <typename T>
 __device__ __forceinline__ void sphere_points(const Inst& I, const FrameP& fp, uint64_t j, int d, uint32_t h,
                                            const uint32_t* tab, uint32_t s) {
-    T W[9], Wp[9];
-    decode_weights<T>(j, d, W, Wp, tab);
+    T a[6];
+    decode_cols(j, d, tab, a);
     const double* V = static_cast<const double*>(I.rel) + 9u * h;
     const size_t cap = I.cap;
     double* pc = I.pc + s;
-#pragma unroll 1
-    for (int v = 0; v < 3; ++v) {
-        double pf[4];
-        sphere_point<T>(W, v, d, fp, V, pf);
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+        double pf[4] = {0.0, 0.0, 0.0, 0.0};  // a root has no parent (never read)
+        T w[3];
+        if (v < 3)
+            weight_row<T>(a, v, d, w);
+        else
+            parent_row<T>(a, (j & 1ull) != 0ull, d, w);
+        if (v < 3 || d >= 1) sphere_point<T>(w, d, fp, V, pf);
 #pragma unroll
         for (int k = 0; k < 4; ++k) pc[(size_t)(4 * v + k) * cap] = pf[k];
     }
-    double pf[4] = {0.0, 0.0, 0.0, 0.0};  // a root has no parent (never read)
-    if (d >= 1) {
-        // the parent's new vertex: its v0 (odd heap ID) or v1 (even), as in
-        // lod_wishes
-        const bool odd = (j & 1ull) != 0ull;
-        T row[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) row[k] = odd ? Wp[k] : Wp[3 + k];
-        sphere_point<T>(row, 0, d - 1, fp, V, pf);
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) pc[(size_t)(12 + k) * cap] = pf[k];
 }
 
 __device__ __forceinline__ void sphere_wishes(const Inst& I, const FrameP& fp, uint32_t s, uint64_t j, int d,
@@ -415,10 +499,10 @@ __device__ __forceinline__ void sphere_wishes(const Inst& I, const FrameP& fp, u
     const unsigned long long gen = I.g->pc_gen;
     const ulonglong2 tag = I.pct[s];
     if (tag.x != j || tag.y != gen) {
-        if (d <= 31)
-            sphere_points<uint32_t>(I, fp, j, d, h, tab, s);
+        if (float_weights(d))
+            sphere_points<float>(I, fp, j, d, h, tab, s);
         else
-            sphere_points<unsigned long long>(I, fp, j, d, h, tab, s);
+            sphere_points<u64>(I, fp, j, d, h, tab, s);
         I.pct[s] = make_ulonglong2(j, gen);
     }
     const size_t cap = I.cap;
@@ -432,6 +516,10 @@ __device__ __forceinline__ void sphere_wishes(const Inst& I, const FrameP& fp, u
 #pragma unroll
         for (int k = 0; k < 9; ++k) keep[k] = r[k];
     wishes_from(r, (j & 1ull) != 0ull, d, I.max_depth, fp,
+                [&](float r2[3]) {
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) r2[k] = r[6 + k];
+                },
                 [&](float nv[3]) { sphere_rel(pc[12 * cap], pc[13 * cap], pc[14 * cap], pc[15 * cap], fp, nv); },
                 split, merge);
 }
@@ -535,6 +623,7 @@ static __device__ uint32_t chain_walk(const Inst& I, uint32_t b, int d, bool sca
 //
 // keep (optional): where the LOD test's vertices of j are stored (only the
 // LOD mode evaluates them; `kept` says whether it did).
+template <int F>
 __device__ __forceinline__ bool item_wishes(const Inst& I, const FrameP& fp, uint64_t key, uint32_t s, uint64_t j,
                                             const uint32_t* tab, bool& split, bool& merge, float* keep = nullptr,
                                             bool* kept = nullptr) {
@@ -545,12 +634,10 @@ __device__ __forceinline__ bool item_wishes(const Inst& I, const FrameP& fp, uin
     if (d < 0 || h >= I.H) return false;
     switch (fp.mode) {
         case 0:
-            if (fp.precision == 3u && I.pc)
+            if (precision_in<F>(fp) == 3u && I.pc)
                 sphere_wishes(I, fp, s, j, d, h, tab, split, merge, keep);
-            else if (d <= 31)
-                lod_wishes<uint32_t>(I, fp, j, d, h, tab, split, merge, keep);
             else
-                lod_wishes<unsigned long long>(I, fp, j, d, h, tab, split, merge, keep);
+                lod_wishes<F>(I, fp, j, d, h, tab, split, merge, keep);
             if (kept) *kept = keep != nullptr;
             break;
         case 1:
@@ -576,11 +663,12 @@ __device__ __forceinline__ bool item_wishes(const Inst& I, const FrameP& fp, uin
 // (kVcValid): the export then copies them instead of evaluating them again.
 // With `merge_in` the word is ORed in: it was cleared before the phase and
 // other bisectors' chain walks may mark it while this one classifies.
+template <int F>
 __device__ __forceinline__ uint32_t classify_item(const Inst& I, const FrameP& fp, uint64_t key, uint32_t i,
                                                   uint32_t s, uint64_t j, const uint32_t* tab, uint32_t* s_cnt,
                                                   bool cache = false, bool merge_in = false) {
     bool split, merge, kept;
-    if (!item_wishes(I, fp, key, s, j, tab, split, merge, cache ? I.vc + 9ull * s : nullptr, &kept)) {
+    if (!item_wishes<F>(I, fp, key, s, j, tab, split, merge, cache ? I.vc + 9ull * s : nullptr, &kept)) {
         set_err(I.g, kErrLink);
         if (!merge_in) *cmd_ptr(I, s) = 0u;
         I.scan[i] = 0u;
@@ -1074,6 +1162,7 @@ static __device__ uint32_t fill_merge(const Inst& I, uint32_t dest, const uint4 
 
 // The three vertices of bisector j into r; false (error word set, r not
 // written) when j does not decode to a root of this mesh.
+template <int F>
 __device__ __forceinline__ bool vertex_eval(const Inst& I, const FrameP& fp, uint64_t j, const uint32_t* tab,
                                             float r[9]) {
     const int d = depth_of(j, I.ch);
@@ -1082,22 +1171,18 @@ __device__ __forceinline__ bool vertex_eval(const Inst& I, const FrameP& fp, uin
         set_err(I.g, kErrLink);
         return false;
     }
-    if (d <= 31) {
-        uint32_t W[9], Wp[9];
-        decode_weights<uint32_t>(j, d, W, Wp, tab);
-        eval_vertices<uint32_t>(W, d, fp, I.rel, h, r);
-    } else {
-        unsigned long long W[9], Wp[9];
-        decode_weights<unsigned long long>(j, d, W, Wp, tab);
-        eval_vertices<unsigned long long>(W, d, fp, I.rel, h, r);
-    }
+    float q[12];
+    eval_rows<F>(fp, I.rel, j, d, h, tab, 7, q);
+#pragma unroll
+    for (int k = 0; k < 9; ++k) r[k] = q[k];
     return true;
 }
 
+template <int F>
 __device__ __forceinline__ void vertex_item(const Inst& I, const FrameP& fp, uint32_t i, uint64_t j,
                                             const uint32_t* tab, float* out) {
     float r[9];
-    if (!vertex_eval(I, fp, j, tab, r)) return;
+    if (!vertex_eval<F>(I, fp, j, tab, r)) return;
     float* o = out + 9ull * i;
 #pragma unroll
     for (int k = 0; k < 9; ++k) o[k] = r[k];
@@ -1132,15 +1217,16 @@ __device__ __forceinline__ void warp_rows_out(const float r[9], float* stage, fl
 // Vertices of the live bisector in slot s at output row i: in the sphere
 // and displaced forms copied from the frame's cache when the LOD test stored
 // them, else evaluated.
+template <int F>
 __device__ __forceinline__ void vertex_item_cached(const Inst& I, const FrameP& fp, uint32_t i, uint32_t s,
                                                    const uint32_t* tab, float* out) {
-    if (vc_form(fp) && (*cmd_ptr(I, s) & kVcValid)) {
+    if (vc_form<F>(fp) && (*cmd_ptr(I, s) & kVcValid)) {
         const float* src = I.vc + 9ull * s;
         float* o = out + 9ull * i;
 #pragma unroll
         for (int k = 0; k < 9; ++k) o[k] = src[k];
     } else {
-        vertex_item(I, fp, i, I.heap[s], tab, out);
+        vertex_item<F>(I, fp, i, I.heap[s], tab, out);
     }
 }
 
