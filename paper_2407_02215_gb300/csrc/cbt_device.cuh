@@ -368,19 +368,38 @@ __device__ __forceinline__ void decode_cols(uint64_t j, int d, const uint32_t* t
     decode_levels((uint32_t)j & ((1u << d) - 1u), d, tab, a);
 }
 // The levels in runs of at most 24, each decoded in FP32 and applied to the
-// integer weights so far: 2^24 a2 + b0 (a0 - a2) + b1 (a1 - a2), b = 2^24 P.
+// integer weights so far: 2^24 a2 + b0 (a0 - a2) + b1 (a1 - a2), b = 2^24 P
+// (32 x 32 -> 64 bit products while the weights so far fit 25 bits).
 __device__ __forceinline__ void decode_cols(uint64_t j, int d, const uint32_t* tab, u64 a[6]) {
     const int first = d > 0 ? (d - 1) % 24 + 1 : 0;
     float p[6];
     decode_levels((uint32_t)(j >> (d - first)) & ((1u << first) - 1u), first, tab, p);
+    int s[6];
 #pragma unroll
-    for (int k = 0; k < 6; ++k) a[k] = __float2uint_rn(__fmul_rn(p[k], pow2f(first)));
-#pragma unroll 1
-    for (int lo = d - first - 24; lo >= 0; lo -= 24) {
+    for (int k = 0; k < 6; ++k) {
+        s[k] = __float2int_rn(__fmul_rn(p[k], pow2f(first)));
+        a[k] = (u64)s[k];
+    }
+    int lo = d - first - 24;
+    if (lo >= 0) {
         decode_levels((uint32_t)(j >> lo) & 0xFFFFFFu, 24, tab, p);
-        uint32_t b[6];
+        int b[6];
 #pragma unroll
-        for (int k = 0; k < 6; ++k) b[k] = __float2uint_rn(__fmul_rn(p[k], 0x1p24f));
+        for (int k = 0; k < 6; ++k) b[k] = __float2int_rn(__fmul_rn(p[k], 0x1p24f));
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const long long e = s[c] - s[4 + c], f = s[2 + c] - s[4 + c], a2 = (long long)s[4 + c] << 24;
+#pragma unroll
+            for (int r = 0; r < 3; ++r) a[2 * r + c] = (u64)(a2 + (long long)b[2 * r] * e + (long long)b[2 * r + 1] * f);
+        }
+        lo -= 24;
+    }
+#pragma unroll 1
+    for (; lo >= 0; lo -= 24) {
+        decode_levels((uint32_t)(j >> lo) & 0xFFFFFFu, 24, tab, p);
+        int b[6];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) b[k] = __float2int_rn(__fmul_rn(p[k], 0x1p24f));
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
             const long long e = (long long)(a[c] - a[4 + c]), f = (long long)(a[2 + c] - a[4 + c]);
@@ -429,10 +448,13 @@ __device__ __forceinline__ double weight_f64(u64 w, int d) {
     return __dsub_rn(__longlong_as_double(__double_as_longlong(one) | (long long)w), one);
 }
 
-// Correctly rounded signed 128-bit integer (hi 2^64 + lo) -> float: the
-// magnitude's top 32 bits with a sticky bit for the rest, one RN conversion,
-// one exact scaling.
-__device__ __forceinline__ float s128_to_float(long long hi, u64 lo) {
+// Correctly rounded signed 128-bit integer (hi 2^64 + lo) -> float. Below
+// 2^63 in magnitude one 64-bit conversion; below 2^95 one of the value over
+// 2^32 rounded to odd (its lowest bit set when bits were cut off: more than
+// two bits below an FP32's last place, so the second rounding is as the
+// first would have been). Beyond (never with camera-relative coordinates of
+// a scene, but legal) the magnitude's top 32 bits with a sticky bit.
+static __device__ __noinline__ float s128_to_float_any(long long hi, u64 lo) {
     const bool neg = hi < 0;
     u64 h = (u64)hi;
     if (neg) {
@@ -453,66 +475,63 @@ __device__ __forceinline__ float s128_to_float(long long hi, u64 lo) {
     const float m = __fmul_rn(f, pow2f(e - lz));
     return neg ? -m : m;
 }
+__device__ __forceinline__ float s128_to_float(long long hi, u64 lo) {
+    if ((hi >> 31) != (hi >> 63)) return s128_to_float_any(hi, lo);
+    const bool small = hi == (long long)lo >> 63;
+    const long long over = (long long)(((u64)hi << 32) | (lo >> 32)) | ((uint32_t)lo != 0u ? 1ll : 0ll);
+    const float f = __ll2float_rn(small ? (long long)lo : over);
+    return small ? f : __fmul_rn(f, 0x1p32f);
+}
 
-// Fixed point: the exact sum over the root's vertices of weight times
-// coordinate. Weights below 2^25 (float ones, d <= 24) take six 32 x 32 -> 64
-// multiply-adds per coordinate, sum = mid 2^32 + lo; wider ones (d <= 48) are
-// split into two 24-bit parts, so that no partial sum overflows either;
-// beyond, the general 128-bit product.
+// Fixed point: exact sums over the root's vertices of weight times
+// coordinate. A coordinate x (|x| < 2^62) is split as xh 2^32 + xl with both
+// halves signed 32 bits, so that every product is one signed 32 x 32 -> 64
+// multiply-add and no partial sum overflows.
 struct S128 {
     long long hi;
     u64 lo;
 };
-__device__ __forceinline__ S128 s128_from(long long mid, u64 lo) {  // mid 2^32 + lo
-    const u64 l = lo + ((u64)mid << 32);
-    return S128{(mid >> 32) + (l < lo ? 1ll : 0ll), l};
-}
 __device__ __forceinline__ S128 s128_add(S128 a, S128 b) {
     const u64 l = a.lo + b.lo;
     return S128{a.hi + b.hi + (l < a.lo ? 1ll : 0ll), l};
 }
-__device__ __forceinline__ void fixed_sum(const uint32_t w[3], const long long* X, int c, S128& out) {
-    u64 lo = 0ull;
-    long long mid = 0;
+// (m 2^32 + l) 2^k, k = 0 or 24, l the low half's sum (signed).
+__device__ __forceinline__ S128 s128_parts(long long m, long long l) {
+    m += l >> 32;
+    return S128{m >> 32, ((u64)m << 32) | (uint32_t)l};
+}
+__device__ __forceinline__ S128 s128_shl24(S128 a) {
+    return S128{(long long)(((u64)a.hi << 24) | (a.lo >> 40)), a.lo << 24};
+}
+__device__ __forceinline__ void split_coord(long long x, int& xl, int& xh) {
+    xl = (int)x;
+    xh = (int)(x >> 32) + (xl < 0 ? 1 : 0);
+}
+// Signed weights below 2^26 in magnitude.
+__device__ __forceinline__ S128 fixed_narrow(const int w[3], const int xl[3], const int xh[3]) {
+    long long l = 0, m = 0;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        const long long x = X[3 * i + c];
-        lo += (u64)w[i] * (u64)(uint32_t)x;
-        mid += (long long)(int)w[i] * (long long)(int)(x >> 32);
+        l += (long long)w[i] * (long long)xl[i];
+        m += (long long)w[i] * (long long)xh[i];
     }
-    out = s128_from(mid, lo);
+    return s128_parts(m, l);
 }
-__device__ __forceinline__ void fixed_sum(const u64 w[3], int d, const long long* X, int c, S128& out) {
-    if (d <= 48) {
-        uint32_t l[3], h[3];
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            l[i] = (uint32_t)w[i] & 0xFFFFFFu;
-            h[i] = (uint32_t)(w[i] >> 24);
-        }
-        S128 a, b;
-        fixed_sum(l, X, c, a);
-        fixed_sum(h, X, c, b);
-        b.hi = (long long)(((u64)b.hi << 24) | (b.lo >> 40));
-        b.lo <<= 24;
-        out = s128_add(a, b);
-        return;
-    }
+// Weights up to 2^48, in two 24-bit parts (the upper ones all 0: `wide` false).
+__device__ __forceinline__ S128 fixed_wide(const int wl[3], const int wh[3], bool wide, const int xl[3],
+                                           const int xh[3]) {
+    const S128 a = fixed_narrow(wl, xl, xh);
+    return wide ? s128_add(a, s128_shl24(fixed_narrow(wh, xl, xh))) : a;
+}
+// Any weights (one coordinate; X points at the root's first vertex's).
+__device__ __forceinline__ S128 fixed_any(const u64 w[3], const long long* X) {
     __int128 s = 0;
 #pragma unroll
-    for (int i = 0; i < 3; ++i) s += (__int128)w[i] * (__int128)X[3 * i + c];
-    out = S128{(long long)(s >> 64), (u64)s};
+    for (int i = 0; i < 3; ++i) s += (__int128)w[i] * (__int128)X[3 * i];
+    return S128{(long long)(s >> 64), (u64)s};
 }
-
-__device__ __forceinline__ void fixed_coord(const float w[3], int d, const long long* X, int c, S128& out) {
-    uint32_t u[3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) u[i] = __float2uint_rn(__fmul_rn(w[i], pow2f(d)));
-    fixed_sum(u, X, c, out);
-}
-__device__ __forceinline__ void fixed_coord(const u64 w[3], int d, const long long* X, int c, S128& out) {
-    fixed_sum(w, d, X, c, out);
-}
+__device__ __forceinline__ u64 weight_int(u64 w, int) { return w; }
+__device__ __forceinline__ u64 weight_int(float w, int d) { return (u64)__float2int_rn(__fmul_rn(w, pow2f(d))); }
 
 // ------------------------------------------------------------ displacement
 
@@ -673,10 +692,10 @@ __device__ __forceinline__ void eval_vertex(const T w[3], int d, const FrameP& f
         sphere_rel(pf[0], pf[1], pf[2], pf[3], fp, r);
     } else if (precision == 1u) {
         const long long* X = static_cast<const long long*>(rel) + 9u * h;
+        const u64 wi[3] = {weight_int(w[0], d), weight_int(w[1], d), weight_int(w[2], d)};
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            S128 s;
-            fixed_coord(w, d, X, c, s);
+            const S128 s = fixed_any(wi, X + c);
             r[c] = __fmul_rn(s128_to_float(s.hi, s.lo), pow2f(-(d + fp.shift)));
         }
     } else if (precision == 2u) {

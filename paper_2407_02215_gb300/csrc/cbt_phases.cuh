@@ -408,6 +408,54 @@ __device__ __forceinline__ void eval_rows(const FrameP& fp, const void* rel, uin
             }
         return;
     }
+    if (F == kFormFixed && d <= 48) {
+        // The first row's sum from its weights; the others' add the exact sum
+        // over their weights' differences from it, which are small: a vertex
+        // of the bisector (or its parent) at depth d differs from another in
+        // barycentric coordinates by at most 2^(1 - floor(d / 2)), i.e. 2^26
+        // over 2^48, so one 32-bit product per half coordinate will do. (With
+        // 64-bit weights and 128-bit products for every vertex, classify of
+        // 2.2M bisectors took 195 us and the export 119; so 129 and 83.)
+        u64 a[6];
+        decode_cols(j, d, tab, a);
+        const int base = (rows & 1) ? 0 : (rows & 2) ? 1 : 2;
+        u64 w0[3];
+        weight_row<u64>(a, base, d, w0);
+        int wl[3], wh[3], dw[4][3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            wl[k] = (int)((uint32_t)w0[k] & 0xFFFFFFu);
+            wh[k] = (int)(w0[k] >> 24);
+        }
+        const bool wide = __any_sync(__activemask(), (wh[0] | wh[1] | wh[2]) != 0);
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            if (!((rows >> v) & 1) || v == base) continue;
+            u64 w[3];
+            if (v < 3)
+                weight_row<u64>(a, v, d, w);
+            else
+                parent_row<u64>(a, odd, d, w);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) dw[v][k] = (int)(uint32_t)(w[k] - w0[k]);
+        }
+        const long long* X = static_cast<const long long*>(rel) + 9u * h;
+        const float sc = pow2f(-(d + fp.shift));
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            int xl[3], xh[3];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) split_coord(X[3 * i + c], xl[i], xh[i]);
+            const S128 s0 = fixed_wide(wl, wh, wide, xl, xh);
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                if (!((rows >> v) & 1)) continue;
+                const S128 s = v == base ? s0 : s128_add(s0, fixed_narrow(dw[v], xl, xh));
+                r[3 * v + c] = __fmul_rn(s128_to_float(s.hi, s.lo), sc);
+            }
+        }
+        return;
+    }
     auto eval = [&](auto a) {
         typedef typename std::remove_pointer<decltype(a)>::type T;
 #pragma unroll
