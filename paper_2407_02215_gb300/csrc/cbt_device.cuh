@@ -643,9 +643,8 @@ __device__ __forceinline__ void displace_plain(float r[3], const FrameP& fp) {
 // The sphere form's frame-independent part of vertex v: pf = {p_x, p_y, p_z,
 // f}, f = radius' y (V: the root triangle's absolute FP64 vertices). It
 // depends on the heap ID, the mesh, the radius and the displacement only.
-template <typename T>
-__device__ __forceinline__ void sphere_point(const T w[3], int d, const FrameP& fp, const double* V, double pf[4]) {
-    const double w0 = weight_f64(w[0], d), w1 = weight_f64(w[1], d), w2 = weight_f64(w[2], d);
+__device__ __forceinline__ void sphere_point(const double w[3], const FrameP& fp, const double* V, double pf[4]) {
+    const double w0 = w[0], w1 = w[1], w2 = w[2];
     double p[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) p[c] = __fma_rn(w2, V[6 + c], __fma_rn(w1, V[3 + c], __dmul_rn(w0, V[c])));
@@ -688,7 +687,8 @@ __device__ __forceinline__ void eval_vertex(const T w[3], int d, const FrameP& f
     const uint32_t precision = precision_in<F>(fp);
     if (precision == 3u) {
         double pf[4];
-        sphere_point<T>(w, d, fp, static_cast<const double*>(rel) + 9u * h, pf);
+        const double wd[3] = {weight_f64(w[0], d), weight_f64(w[1], d), weight_f64(w[2], d)};
+        sphere_point(wd, fp, static_cast<const double*>(rel) + 9u * h, pf);
         sphere_rel(pf[0], pf[1], pf[2], pf[3], fp, r);
     } else if (precision == 1u) {
         const long long* X = static_cast<const long long*>(rel) + 9u * h;

@@ -535,7 +535,8 @@ __device__ __forceinline__ void sphere_points(const Inst& I, const FrameP& fp, u
             weight_row<T>(a, v, d, w);
         else
             parent_row<T>(a, (j & 1ull) != 0ull, d, w);
-        if (v < 3 || d >= 1) sphere_point<T>(w, d, fp, V, pf);
+        const double wd[3] = {weight_f64(w[0], d), weight_f64(w[1], d), weight_f64(w[2], d)};
+        if (v < 3 || d >= 1) sphere_point(wd, fp, V, pf);
 #pragma unroll
         for (int k = 0; k < 4; ++k) pc[(size_t)(4 * v + k) * cap] = pf[k];
     }
@@ -706,6 +707,24 @@ __device__ __forceinline__ bool item_wishes(const Inst& I, const FrameP& fp, uin
     return true;
 }
 
+// The command word of slot s (live index i, heap ID j) and its scan word.
+__device__ __forceinline__ uint32_t store_command(const Inst& I, const FrameP& fp, uint32_t i, uint32_t s, uint64_t j,
+                                                  bool split, bool merge, bool kept, uint32_t* s_cnt,
+                                                  bool merge_in = false) {
+    const int d = depth_of(j, I.ch);
+    const uint32_t cmd = (split ? kSplitWish : 0u) | (merge ? kMergeWish : 0u) |
+                         ((d & 1) ? kDepthOdd : 0u) | ((j & 1ull) ? kHeapOdd : 0u) | (kept ? kVcValid : 0u);
+    if (merge_in)
+        atomicOr(cmd_ptr(I, s), cmd);
+    else
+        *cmd_ptr(I, s) = cmd;
+    // the paper's gate charges 3d + 4 without walking the chain (k_walk
+    // computes the exact chain cost otherwise)
+    I.scan[i] = (split && fp.gate == 1) ? 3u * (uint32_t)d + 4u : 0u;
+    count_stat(s_cnt, 0, split);
+    return cmd;
+}
+
 // With `cache` (the one-launch frame exporting sphere-form or displaced
 // vertices) the LOD test's vertices go to vc[s] and the command word says so
 // (kVcValid): the export then copies them instead of evaluating them again.
@@ -722,18 +741,7 @@ __device__ __forceinline__ uint32_t classify_item(const Inst& I, const FrameP& f
         I.scan[i] = 0u;
         return 0u;
     }
-    const int d = depth_of(j, I.ch);
-    const uint32_t cmd = (split ? kSplitWish : 0u) | (merge ? kMergeWish : 0u) |
-                         ((d & 1) ? kDepthOdd : 0u) | ((j & 1ull) ? kHeapOdd : 0u) | (kept ? kVcValid : 0u);
-    if (merge_in)
-        atomicOr(cmd_ptr(I, s), cmd);
-    else
-        *cmd_ptr(I, s) = cmd;
-    // the paper's gate charges 3d + 4 without walking the chain (k_walk
-    // computes the exact chain cost otherwise)
-    I.scan[i] = (split && fp.gate == 1) ? 3u * (uint32_t)d + 4u : 0u;
-    count_stat(s_cnt, 0, split);
-    return cmd;
+    return store_command(I, fp, i, s, j, split, merge, kept, s_cnt, merge_in);
 }
 
 // Pointer chases of the frame, after classify: the compatibility-chain cost
@@ -1234,6 +1242,27 @@ __device__ __forceinline__ void vertex_item(const Inst& I, const FrameP& fp, uin
     float* o = out + 9ull * i;
 #pragma unroll
     for (int k = 0; k < 9; ++k) o[k] = r[k];
+}
+
+// Vertex v of bisector j alone (nothing written when vertex_eval refuses j).
+template <int F>
+__device__ __forceinline__ void vertex_point(const Inst& I, const FrameP& fp, uint64_t j, int v, const uint32_t* tab,
+                                             float* out) {
+    const int d = depth_of(j, I.ch);
+    const uint32_t h = (uint32_t)((j >> d) - (1ull << I.ch));
+    if (d < 0 || h >= I.H) {
+        set_err(I.g, kErrLink);
+        return;
+    }
+    u64 a[6], w[3];
+    decode_cols(j, d, tab, a);
+    w[0] = v == 0 ? a[0] : v == 1 ? a[2] : a[4];
+    w[1] = v == 0 ? a[1] : v == 1 ? a[3] : a[5];
+    w[2] = (1ull << d) - w[0] - w[1];
+    float r[3];
+    eval_vertex<F, u64>(w, d, fp, I.rel, h, r);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) out[c] = r[c];
 }
 
 // A warp's 32 consecutive output rows of 9 floats (rows row0 .. row0 + 31,
