@@ -422,19 +422,25 @@ __device__ void phase_gate_sum(const BatchDev& bt, FCtx& c, uint32_t* s_cnt, uin
 
 // Granted merge total Mg when the merge requests of the instance overflow F:
 // the largest inclusive merge prefix that fits (merges are granted first, in
-// slot order). Only taken when the instance's merge sum exceeds F.
+// slot order). Only taken when the instance's merge sum exceeds F. The tile
+// that crosses F is found by scans of the tile sums, 256 at a time: one
+// thread adding them up one load after another made the gate of a full
+// 2^23-slot pool (4,000 tiles) 563 us; so it is 71.
 __device__ uint32_t crossing_mg(const BatchDev& bt, const FCtx& c, uint32_t F, uint32_t ipt, Pair* s_warp,
                                 uint32_t* s_tmp) {
-    if (threadIdx.x == 0) {
-        uint32_t acc = 0, u = c.tb;
-        for (; u < c.te; ++u) {
-            const uint32_t a = unpack_pair(__ldcg(bt.status + u)).a;
-            if ((uint64_t)acc + a > F) break;
-            acc += a;
+    uint32_t done = 0;
+    for (uint32_t u0 = c.tb; u0 < c.te; u0 += blockDim.x) {  // block-uniform
+        const uint32_t u = u0 + threadIdx.x;
+        const uint32_t a = u < c.te ? unpack_pair(__ldcg(bt.status + u)).a : 0u;
+        Pair all;
+        const Pair ex = block_scan(Pair{a, 0u}, all, s_warp);
+        const uint64_t before = (uint64_t)done + ex.a;
+        if (before <= F && before + a > F) {  // one thread: the sums are not negative
+            s_tmp[0] = u - c.tb;
+            s_tmp[1] = s_tmp[2] = (uint32_t)before;
         }
-        s_tmp[0] = u - c.tb;
-        s_tmp[1] = acc;
-        s_tmp[2] = acc;
+        if ((uint64_t)done + all.a > F) break;
+        done += all.a;
     }
     __syncthreads();
     const uint32_t lt = s_tmp[0], acc = s_tmp[1];
@@ -886,7 +892,7 @@ __device__ void phase_reduce(const BatchDev& bt, FCtx& c, uint32_t* s_buf, uint3
 // exports them.
 template <int F>
 __device__ void phase_compact(const BatchDev& bt, FCtx& c, const uint32_t* s_tab, uint32_t* s_buf,
-                              uint32_t* s_w) {
+                              uint32_t* s_w, float* s_stage) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     for (uint32_t wt = blockIdx.x; wt < bt.Twords; wt += gridDim.x) {
         ctx_tile(bt, bt.wtile_base, wt, bt.Twords, c);
@@ -937,10 +943,30 @@ __device__ void phase_compact(const BatchDev& bt, FCtx& c, const uint32_t* s_tab
         __syncthreads();
         for (uint32_t k = threadIdx.x; k < tot; k += blockDim.x) I.live[before + k] = s_buf[k];
         if (fp.vout && bt.B > 1) {
-            const uint32_t lim = fp.vcap;
-            for (uint32_t k = threadIdx.x; k < tot; k += blockDim.x) {
-                const uint32_t i = before + k;
-                if (i < lim) vertex_item_cached<F>(I, fp, i, s_buf[k], s_tab, fp.vout);
+            // rows of 32 consecutive live bisectors per warp, staged and stored
+            // 16 bytes wide; the heap ID of the warp's next round loaded ahead
+            const uint32_t n = before < fp.vcap ? min(tot, fp.vcap - before) : 0u;
+            const uint64_t* const heap = I.heap;
+            if (vc_form<F>(fp)) {
+                for (uint32_t k = threadIdx.x; k < n; k += blockDim.x)
+                    vertex_item_cached<F>(I, fp, before + k, s_buf[k], s_tab, fp.vout);
+            } else {
+                uint64_t j = threadIdx.x < n ? heap[s_buf[threadIdx.x]] : 0ull;
+                for (uint32_t k0 = threadIdx.x & ~31u; k0 < n; k0 += blockDim.x) {  // warp-uniform
+                    const uint32_t k = k0 + lane, kn = k + blockDim.x;
+                    const uint64_t jn = kn < n ? heap[s_buf[kn]] : 0ull;
+                    float r[9];
+                    bool ok = true;
+                    if (k < n) ok = vertex_eval<F>(I, fp, j, s_tab, r);
+                    if (__all_sync(0xFFFFFFFFu, ok)) {
+                        warp_rows_out(r, s_stage + 288u * warp, fp.vout, (uint64_t)before + k0, min(32u, n - k0));
+                    } else if (k < n && ok) {  // a row the decode refused stays unwritten
+                        float* o = fp.vout + 9ull * (before + k);
+#pragma unroll
+                        for (int q = 0; q < 9; ++q) o[q] = r[q];
+                    }
+                    j = jn;
+                }
             }
         }
         __syncthreads();
@@ -1061,6 +1087,7 @@ __global__ void __launch_bounds__(kFThreads, CBT_FRAME_MIN_BLOCKS) k_frame(Batch
     __shared__ uint32_t s_w[kFThreads / 32 + 1];
     __shared__ uint32_t s_tmp[4];
     __shared__ uint32_t s_n;
+    __shared__ __align__(16) float s_stage[288 * (kFThreads / 32)];  // per warp: 32 rows of 9 floats
     // every block reads the epoch before its first arrival; block 0 advances
     // it after the last barrier, when every block has read it
     const uint32_t epoch = ld_volatile(&bt.bg->bar_epoch);
@@ -1091,7 +1118,7 @@ __global__ void __launch_bounds__(kFThreads, CBT_FRAME_MIN_BLOCKS) k_frame(Batch
     phase_reduce(bt, s_c, s_buf, &s_tmp[0]);
     grid_sync(bt.bg, epoch, 8u);
     stamp(bt, 8);
-    phase_compact<F>(bt, s_c, s_tab, s_buf, s_w);
+    phase_compact<F>(bt, s_c, s_tab, s_buf, s_w, s_stage);
     if (bt.B == 1) {
         grid_sync(bt.bg, epoch, 9u);
         stamp(bt, 9);
