@@ -28,8 +28,8 @@ const char* const kKernelNames[kNumKernels] = {"prep", "classify", "walk", "gate
 // launches per entry of kKernelNames ("cbt" is the reduction plus the compaction)
 constexpr uint32_t kLaunchesPerStep[kNumKernels] = {1, 1, 1, 1, 1, 1, 1, 1, 2, 1};
 // phases of the one-launch frame
-const char* const kPhaseNames[kFramePhases] = {"prep",  "classify", "gate_sum", "gate",    "alloc_sum",
-                                               "alloc", "fill",     "reduce",   "compact", "vertices"};
+const char* const kPhaseNames[kFramePhases] = {"prep", "classify", "gate_sum", "gate",    "alloc",
+                                               "fill", "reduce",   "compact", "vertices"};
 // phases of the single-instance frame (k_frame1)
 const char* const kPhaseNames1[kFrame1Phases] = {"prep",  "classify", "walks", "gate",
                                                  "alloc", "fill",     "final", "vertices"};

@@ -4,17 +4,16 @@
 //
 //   P0 prep       frame counters, item-tile prefix, camera-relative roots
 //   P1 classify   LOD wishes, then the chain and group walks of the same tile
-//   P2 gate-sum   per-tile sums of (merge cost, split cost)
-//   P3 gate       tile prefix from the sums, grants, chain marking
-//   P4 alloc-sum  fates and per-tile sums of (changed, allocations); free list
-//   P5 alloc      tile prefix, free-list indices of the new records
-//   P6 fill       new records, neighbour links, bitfield
-//   P7 reduce     sum tree (the last word tile of an instance builds the top)
-//   P8 compact    live list, and the vertices of the new triangulation
+//   P2 gate-sum   merge candidates among the listed groups, and their costs
+//   P3 gate       tile prefix from the tiles' cost sums, grants, chain marking
+//   P4 alloc      fates, tile-local allocation prefixes, fill records; free list
+//   P5 fill       new records, neighbour links, bitfield
+//   P6 reduce     sum tree (the last word tile of an instance builds the top)
+//   P7 compact    live list, and the vertices of the new triangulation
 //
 // The two prefix sums of the per-step kernels (decoupled look-back) become
 // reduce-then-scan here: tile sums, a barrier, then each tile adds the sums
-// before it. State between phases lives in the slot arrays (command words,
+// before it (the gate), or the fill adds its tile's prefix (the allocation). State between phases lives in the slot arrays (command words,
 // scan words); each block keeps its instance descriptor and frame
 // parameters in shared memory across tiles and phases. Reads of data other
 // blocks wrote in an earlier phase follow a barrier whose fences order them.
@@ -35,7 +34,8 @@ constexpr uint32_t kFBuf = 4096;  // shared scratch words (lists, tree top, live
 constexpr uint32_t kRelRange = 256;  // root-table entries per warp range in P0
 constexpr uint32_t kMinIpt = 4, kMaxIpt = 8;  // items per thread of a scan tile
 constexpr int kBarrierSpin = 1 << 22;
-constexpr uint32_t kBarriers = 8;  // grid barriers per frame (one more for a single instance)
+constexpr uint32_t kBarriers = 7;  // grid barriers per frame (one more for a single instance)
+constexpr int kAllocDone = 7;      // ticket counter: blocks done with the allocation phase
 
 __device__ __forceinline__ unsigned long long global_ns() {
     unsigned long long t;
@@ -182,7 +182,7 @@ __device__ void phase_prep(const BatchDev& bt, Pair* s_warp, uint32_t* s_tmp) {
         for (uint32_t b = threadIdx.x; b < bt.B; b += blockDim.x) atomicAdd(&s_tmp[2], bt.inst[b].sums[1]);
         __syncthreads();
         const uint32_t per_round = gridDim.x * kFThreads;
-        const uint32_t ipt = min(kMaxIpt, max(kMinIpt, (s_tmp[2] + per_round - 1u) / per_round));
+        const uint32_t ipt = s_tmp[2] > kMinIpt * per_round ? kMaxIpt : kMinIpt;  // 16-byte loads per thread
         const uint32_t S = ipt * kFThreads;
         for (uint32_t b0 = 0; b0 < bt.B; b0 += blockDim.x) {
             const uint32_t b = b0 + threadIdx.x;
@@ -198,6 +198,7 @@ __device__ void phase_prep(const BatchDev& bt, Pair* s_warp, uint32_t* s_tmp) {
                 g->Stot = 0;
                 g->C = 0;
                 g->done = 0;
+                g->nwalk = 0;
                 g->marks_clean = 0;
                 g->freel_full = 0;
                 tiles = (N + kTileItems - 1u) / kTileItems;
@@ -232,6 +233,7 @@ __device__ void phase_prep(const BatchDev& bt, Pair* s_warp, uint32_t* s_tmp) {
             bt.bg->scan_ipt = ipt;
             bt.bg->live_total = s_tmp[2];
             bt.bg->t[kFramePhases] = 0;
+            bt.bg->tickets[kAllocDone] = 0;
         }
     }
     // block 0 sets up the instances; the others share the root tables in
@@ -242,42 +244,89 @@ __device__ void phase_prep(const BatchDev& bt, Pair* s_warp, uint32_t* s_tmp) {
         const uint32_t nw = nb * (kFThreads / 32), wid = bb * (kFThreads / 32) + threadIdx.x / 32u;
         const uint32_t per = min(kRelRange, ((bt.Trel + nw - 1u) / nw + 31u) & ~31u);
         for (uint32_t e = wid * per; e < bt.Trel; e += nw * per) rel_range(bt, e, min(bt.Trel, e + per));
+        // the scan tiles' cost sums (at most one tile per kTileItems slots)
+        for (uint32_t t = bb * kFThreads + threadIdx.x; t < bt.Titems; t += nb * kFThreads) bt.status[t] = 0ull;
     }
+}
+
+constexpr uint32_t kWalkCap = kFBuf / 4;  // uint2 entries of the walk list (the groups found take the other half)
+static_assert(kWalkCap >= kTileItems, "a tile's walks fit");
+
+// Where the walks of an instance leave what the gate needs: the split costs
+// per scan tile (S items) and the list of its merge groups (the per-step
+// form's list of changed items), with its length in the counters.
+struct WalkOut {
+    unsigned long long* sums;
+    uint32_t S;
+    uint32_t* groups;
+    uint32_t* ngroups;
+};
+__device__ __forceinline__ WalkOut walk_out(const BatchDev& bt, const Inst& I, uint32_t b) {
+    return WalkOut{bt.status + (bt.B == 1 ? 0u : bt.stile_base[b]), kFThreads * bt.bg->scan_ipt, I.chg, &I.g->nwalk};
 }
 
 // Walks of listed items on the frame-start state: the chain cost of a split
 // wish (command form of Alg. 3, its members recorded in its grp word for the
-// marking), the Alg. 4 group of a merge wish with an even heap ID (its
-// smallest member records the members).
-__device__ __forceinline__ void walk_list(const Inst& I, const uint2* s_list, uint32_t n) {
-    for (uint32_t q = threadIdx.x; q < n; q += kFThreads) {
-        const uint2 e = s_list[q];
-        const uint32_t i = e.x & 0x7FFFFFFFu, s = e.y;
-        if (e.x & 0x80000000u) {
-            uint4 rec;
-            I.scan[i] = chain_walk(I, s, depth_of(I.heap[s], I.ch), false, &rec);
-            I.grp[i] = rec;
-        } else {
-            Group g;
-            if (find_group(I, s, g) && g.imin == 0) {
-                I.grp[i] = make_uint4(g.m[0], g.m[1], g.m[2], g.m[3]);
-                atomicOr(cmd_ptr(I, s), kGrpMin);
+// marking) and its share of the scan tile's sum; the Alg. 4 group of a merge
+// wish with an even heap ID (its smallest member records the members and is
+// listed).
+// Called by the whole block with at most kWalkCap entries, which the groups
+// found follow in shared memory until one atomic reserves their place; split
+// costs leave as one atomic per warp and scan tile. (An atomic per walk made
+// classify of a batch of 15M bisectors 900 us instead of 680.)
+__device__ __forceinline__ void walk_list(const Inst& I, const WalkOut& o, uint2* s_list, uint32_t n,
+                                          uint32_t* s_ng) {
+    const uint32_t lane = threadIdx.x & 31u;
+    uint32_t* s_groups = reinterpret_cast<uint32_t*>(s_list + kWalkCap);
+    if (threadIdx.x == 0) s_ng[0] = 0;
+    __syncthreads();
+    for (uint32_t q0 = threadIdx.x & ~31u; q0 < n; q0 += kFThreads) {  // warp-uniform
+        const uint32_t q = q0 + lane;
+        uint32_t cost = 0, t = kNull;
+        if (q < n) {
+            const uint2 e = s_list[q];
+            const uint32_t s = e.y, i = e.x & 0x7FFFFFFFu;
+            if (e.x & 0x80000000u) {
+                uint4 rec;
+                cost = chain_walk(I, s, depth_of(I.heap[s], I.ch), false, &rec);
+                I.scan[i] = cost;
+                I.grp[i] = rec;
+                t = i / o.S;
+            } else {
+                Group g;
+                if (find_group(I, s, g) && g.imin == 0) {
+                    I.grp[i] = make_uint4(g.m[0], g.m[1], g.m[2], g.m[3]);
+                    atomicOr(cmd_ptr(I, s), kGrpMin);
+                    s_groups[atomicAdd(s_ng, 1u)] = i;
+                }
             }
         }
+        __syncwarp();
+        if (__any_sync(0xFFFFFFFFu, cost != 0u)) {
+            const unsigned m = __match_any_sync(0xFFFFFFFFu, t);
+            const uint32_t sum = __reduce_add_sync(m, cost);
+            if (t != kNull && lane == (uint32_t)(__ffs(m) - 1)) atomicAdd(o.sums + t, (unsigned long long)sum);
+        }
     }
+    __syncthreads();
+    const uint32_t ng = s_ng[0];
+    if (threadIdx.x == 0 && ng) s_ng[1] = atomicAdd(o.ngroups, ng);
+    __syncthreads();
+    for (uint32_t q = threadIdx.x; q < ng; q += kFThreads) o.groups[s_ng[1] + q] = s_groups[q];
 }
 
 template <int F>
-__device__ __forceinline__ void classify_one(const Inst& I, const FrameP& fp, uint64_t key, uint32_t i, uint32_t s,
-                                             uint64_t j, const uint32_t* s_tab, uint32_t* s_cnt, bool chain,
-                                             uint32_t* s_n, uint2* s_list) {
+__device__ __forceinline__ void classify_one(const Inst& I, const FrameP& fp, const WalkOut& o, uint64_t key,
+                                             uint32_t i, uint32_t s, uint64_t j, const uint32_t* s_tab,
+                                             uint32_t* s_cnt, bool chain, uint32_t* s_n, uint2* s_list) {
     const uint32_t cmd = classify_item<F>(I, fp, key, i, s, j, s_tab, s_cnt, vc_form<F>(fp) && fp.vout);
     const bool split = (cmd & kSplitWish) && chain;
     const bool group = (cmd & kMergeWish) && !(cmd & kHeapOdd);
     if (split || group) s_list[atomicAdd(s_n, 1u)] = make_uint2(i | (split ? 0x80000000u : 0u), s);
+    // the paper's gate: the cost classify_item has set, without a walk
+    if ((cmd & kSplitWish) && !chain) atomicAdd(o.sums + i / o.S, (unsigned long long)I.scan[i]);
 }
 
-constexpr uint32_t kWalkCap = kFBuf / 2;  // uint2 entries of the walk list
 
 // P1: wishes of every live bisector (Sec. 3.3 GenerateCommands with the R8
 // LOD reading), then the walks of the listed items. A single instance
@@ -286,7 +335,7 @@ constexpr uint32_t kWalkCap = kFBuf / 2;  // uint2 entries of the walk list
 // batch walks its item tiles.
 template <int F>
 __device__ void phase_classify(const BatchDev& bt, FCtx& c, uint32_t* s_tab, uint32_t* s_cnt, uint32_t* s_n,
-                               uint2* s_list) {
+                               uint2* s_list, uint32_t* s_ng) {
     if (bt.B == 1) {
         if (threadIdx.x == 0) *s_n = 0;
         stats_reset(s_cnt);
@@ -295,6 +344,7 @@ __device__ void phase_classify(const BatchDev& bt, FCtx& c, uint32_t* s_tab, uin
         const FrameP& fp = c.fp;
         const uint32_t N = c.N;
         const bool chain = fp.gate != 1;
+        const WalkOut wo = walk_out(bt, I, c.b);
         const uint64_t key = splitmix64(((uint64_t)fp.seed << 32) | (uint64_t)fp.frame);
         const uint32_t stride = gridDim.x * kFThreads;
         uint32_t i = blockIdx.x * kFThreads + threadIdx.x;
@@ -304,7 +354,7 @@ __device__ void phase_classify(const BatchDev& bt, FCtx& c, uint32_t* s_tab, uin
         for (uint32_t base = blockIdx.x * kFThreads; base < N; base += stride, i += stride) {
             const uint32_t sc = i + 2u * stride < N ? I.live[i + 2u * stride] : 0u;
             const uint64_t jb = i + stride < N ? I.heap[sb] : 0ull;
-            if (i < N) classify_one<F>(I, fp, key, i, sa, ja, s_tab, s_cnt, chain, s_n, s_list);
+            if (i < N) classify_one<F>(I, fp, wo, key, i, sa, ja, s_tab, s_cnt, chain, s_n, s_list);
             sa = sb;
             ja = jb;
             sb = sc;
@@ -312,14 +362,14 @@ __device__ void phase_classify(const BatchDev& bt, FCtx& c, uint32_t* s_tab, uin
             const uint32_t n = *s_n;
             __syncthreads();
             if (n > kWalkCap - kFThreads) {  // block-uniform
-                walk_list(I, s_list, n);
+                walk_list(I, wo, s_list, n, s_ng);
                 __syncthreads();
                 if (threadIdx.x == 0) *s_n = 0;
                 __syncthreads();
             }
         }
         __syncthreads();
-        walk_list(I, s_list, *s_n);
+        walk_list(I, wo, s_list, *s_n, s_ng);
         __syncthreads();
         stats_flush(s_cnt, I.g, kStSplitWishes);
         __syncthreads();
@@ -335,6 +385,7 @@ __device__ void phase_classify(const BatchDev& bt, FCtx& c, uint32_t* s_tab, uin
         const uint32_t N = c.N;
         const uint32_t lt = c.lt;
         const bool chain = fp.gate != 1;
+        const WalkOut wo = walk_out(bt, I, c.b);
         const uint64_t key = splitmix64(((uint64_t)fp.seed << 32) | (uint64_t)fp.frame);
         uint32_t sl[kFPer];
         uint64_t hj[kFPer];
@@ -351,7 +402,7 @@ __device__ void phase_classify(const BatchDev& bt, FCtx& c, uint32_t* s_tab, uin
 #pragma unroll 1
         for (int k = 0; k < kFPer; ++k) {
             const uint32_t i = lt * kTileItems + (uint32_t)k * kFThreads + threadIdx.x;
-            if (i < N) classify_one<F>(I, fp, key, i, sl[0], hj[0], s_tab, s_cnt, chain, s_n, s_list);
+            if (i < N) classify_one<F>(I, fp, wo, key, i, sl[0], hj[0], s_tab, s_cnt, chain, s_n, s_list);
 #pragma unroll
             for (int q = 0; q + 1 < kFPer; ++q) {  // constant indices: registers, not local memory
                 sl[q] = sl[q + 1];
@@ -359,7 +410,7 @@ __device__ void phase_classify(const BatchDev& bt, FCtx& c, uint32_t* s_tab, uin
             }
         }
         __syncthreads();
-        walk_list(I, s_list, *s_n);
+        walk_list(I, wo, s_list, *s_n, s_ng);
         __syncthreads();
         stats_flush(s_cnt, I.g, kStSplitWishes);
         __syncthreads();
@@ -373,51 +424,96 @@ __device__ __forceinline__ uint32_t stile_first(const FCtx& c, uint32_t ipt) {
     return c.lt * kFThreads * ipt + threadIdx.x * ipt;
 }
 
-// P2: per item its split cost and, at a merge group's smallest member, the
-// merge cost (kept in the top byte of its scan word for P3); per tile the
-// sums. The group checks (group record, then the members' command words)
-// run from a list, two dependent loads per listed item.
-__device__ void phase_gate_sum(const BatchDev& bt, FCtx& c, uint32_t* s_cnt, uint32_t* s_red, uint32_t* s_n,
-                               uint32_t* s_list, bool clear_marks = false) {
-    const uint32_t T = bt.bg->total_stiles, ipt = bt.bg->scan_ipt;
-    for (uint32_t t = blockIdx.x; t < T; t += gridDim.x) {
-        if (threadIdx.x == 0) *s_n = 0;
+// The items of a list that every instance of the batch has (count(I) of them),
+// as one range walked evenly over the grid: body(b, I, q) -> uint32_t for
+// item q of instance b, its results added to the instance's statistic `stat`.
+// Lists cluster in a few instances; a block finds an item's instance in the
+// prefix of the lists' lengths, built in shared memory.
+template <typename Count, typename Body>
+__device__ __forceinline__ void batch_list(const BatchDev& bt, FCtx& c, int stat, uint32_t* s_cnt, uint32_t* s_list,
+                                           Pair* s_warp, Count count, Body body) {
+    const uint32_t stride = gridDim.x * kFThreads;
+    if (bt.B == 1) {
         stats_reset(s_cnt);
-        ctx_tile(bt, bt.stile_base, t, T, c);
+        ctx_tile(bt, bt.tile_base, 0, 1, c);  // instance 0 in shared memory
         const Inst& I = c.I;
-        const uint32_t N = c.N;
-        const uint32_t i0 = stile_first(c, ipt);
-        uint32_t sl[kMaxIpt];
-        Pair loc{0, 0};
-#pragma unroll
-        for (uint32_t k = 0; k < kMaxIpt; ++k) {
-            const bool in = k < ipt && i0 + k < N;
-            sl[k] = in ? I.live[i0 + k] : kNull;
-            loc.b += in ? I.scan[i0 + k] : 0u;
-        }
-#pragma unroll
-        for (uint32_t k = 0; k < kMaxIpt; ++k) {
-            if (sl[k] == kNull) continue;
-            // the single-instance frame's classify marked every chain; the
-            // prefix gate starts from unmarked words
-            const uint32_t cw = clear_marks ? atomicAnd(cmd_ptr(I, sl[k]), ~kSplitMask) : *cmd_ptr(I, sl[k]);
-            if (cw & kGrpMin) s_list[atomicAdd(s_n, 1u)] = i0 + k;
-        }
+        const uint32_t n = count(I);
+        uint32_t sum = 0;
+        for (uint32_t q = blockIdx.x * kFThreads + threadIdx.x; q < n; q += stride) sum += body(0u, I, q);
+        if (sum) atomicAdd(&s_cnt[0], sum);
         __syncthreads();
-        const uint32_t n = *s_n;
-        for (uint32_t q = threadIdx.x; q < n; q += kFThreads) {
-            const uint32_t i = s_list[q];
-            const uint32_t mc = merge_cost(I, i, kGrpMin, c.fp.gate);
-            if (mc) I.scan[i] |= mc << 24;
-            loc.a += mc;
-            count_stat(s_cnt, 0, mc != 0u);
-        }
-        Pair dummy{0, 0};
-        block_sum2(loc, dummy, s_red);
-        if (threadIdx.x == 0) bt.status[t] = pack_pair(loc);
-        stats_flush(s_cnt, I.g, kStMergeCand);
+        stats_flush(s_cnt, I.g, stat);
         __syncthreads();
+        return;
     }
+    const int lane = threadIdx.x & 31;
+    const uint32_t wfirst = blockIdx.x * kFThreads + (threadIdx.x & ~31u);
+    for (uint32_t cb = 0; cb < bt.B; cb += kFBuf) {  // kFBuf instances at a time
+        const uint32_t nb = min(kFBuf, bt.B - cb);
+        uint32_t total = 0;
+        __syncthreads();
+        for (uint32_t b0 = 0; b0 < nb; b0 += kFThreads) {
+            const uint32_t b = b0 + threadIdx.x;
+            const uint32_t n = b < nb ? count(bt.inst[cb + b]) : 0u;
+            Pair tot;
+            const Pair ex = block_scan(Pair{n, 0u}, tot, s_warp);
+            if (b < nb) s_list[b] = total + ex.a;
+            total += tot.a;
+        }
+        __syncthreads();
+        for (uint32_t q0 = wfirst; q0 < total; q0 += stride) {  // warp-uniform trips
+            const uint32_t q = q0 + (uint32_t)lane;
+            uint32_t b = kNull, r = 0;
+            if (q < total) {
+                const uint32_t lb = find_inst(s_list, nb, q);
+                b = cb + lb;
+                r = body(b, bt.inst[b], q - s_list[lb]);
+            }
+            __syncwarp();
+            const uint32_t same = __match_any_sync(0xFFFFFFFFu, b);
+            const uint32_t sum = __reduce_add_sync(same, r);
+            if (b != kNull && sum && lane == __ffs(same) - 1) atomicAdd(&bt.inst[b].g->stats[stat], sum);
+        }
+    }
+}
+
+// P2: the merge groups the walks listed: a group whose members all wish to
+// merge is a candidate; its cost goes to the top byte of its smallest
+// member's scan word and to its scan tile's sum (the walks added the split
+// costs). Reading only the listed items, not every live one's slot, scan and
+// command words, took this phase of a batch of 15M bisectors from 126 to
+// 67 us.
+__device__ void phase_gate_sum(const BatchDev& bt, FCtx& c, uint32_t* s_cnt, uint32_t* s_list, Pair* s_warp) {
+    const uint32_t S = kFThreads * bt.bg->scan_ipt;
+    batch_list(bt, c, kStMergeCand, s_cnt, s_list, s_warp, [](const Inst& I) { return __ldcg(&I.g->nwalk); },
+               [&](uint32_t b, const Inst& I, uint32_t q) {
+                   const uint32_t i = I.chg[q];
+                   const uint32_t mc = merge_cost(I, i, kGrpMin, frame_of(bt, b).gate);
+                   if (mc == 0u) return 0u;
+                   I.scan[i] = mc << 24;
+                   atomicAdd(bt.status + (bt.B == 1 ? 0u : bt.stile_base[b]) + i / S, (unsigned long long)mc << 32);
+                   return 1u;
+               });
+}
+
+// The ipt consecutive words from p + i0 (those at index >= n: `none`), as
+// 16-byte loads when ipt and so i0 are multiples of 4.
+__device__ __forceinline__ void load_items(const uint32_t* p, uint32_t i0, uint32_t ipt, uint32_t n, uint32_t none,
+                                           uint32_t v[kMaxIpt]) {
+    if ((ipt & 3u) == 0u) {
+#pragma unroll
+        for (uint32_t k = 0; k < kMaxIpt; k += 4u) {
+            uint4 x = make_uint4(none, none, none, none);
+            if (k < ipt && i0 + k < n) x = *reinterpret_cast<const uint4*>(p + i0 + k);
+            v[k] = x.x;
+            v[k + 1] = i0 + k + 1u < n ? x.y : none;
+            v[k + 2] = i0 + k + 2u < n ? x.z : none;
+            v[k + 3] = i0 + k + 3u < n ? x.w : none;
+        }
+        return;
+    }
+#pragma unroll
+    for (uint32_t k = 0; k < kMaxIpt; ++k) v[k] = (k < ipt && i0 + k < n) ? p[i0 + k] : none;
 }
 
 // Granted merge total Mg when the merge requests of the instance overflow F:
@@ -486,12 +582,8 @@ __device__ void phase_gate(const BatchDev& bt, FCtx& c, uint32_t* s_cnt, uint32_
         const uint32_t N = c.N, F = c.F;
         const uint32_t i0 = stile_first(c, ipt);
         uint32_t sl[kMaxIpt], w[kMaxIpt];
-#pragma unroll
-        for (uint32_t k = 0; k < kMaxIpt; ++k) {  // loaded before the tile sums, which do not need them
-            const bool in = k < ipt && i0 + k < N;
-            sl[k] = in ? I.live[i0 + k] : kNull;
-            w[k] = in ? I.scan[i0 + k] : 0u;
-        }
+        load_items(I.live, i0, ipt, N, kNull, sl);  // before the tile sums, which do not need them
+        load_items(I.scan, i0, ipt, N, 0u, w);
         Pair before, all;
         tile_sums(bt.status, c, before, all, s_red);
         const uint32_t Mg = all.a <= F ? all.a : crossing_mg(bt, c, F, ipt, s_warp, s_tmp);
@@ -571,52 +663,179 @@ __device__ void phase_gate(const BatchDev& bt, FCtx& c, uint32_t* s_cnt, uint32_
 __device__ void free_list(const BatchDev& bt, FCtx& c, uint32_t* s_w, bool all_granted,
                           const unsigned long long* tcounts = nullptr);
 
-// P4: the fate of every item after the chains are marked (kept in its scan
-// word for P5) and per tile the sums of (changed, allocations); then the
-// free list up to the frame's allocation bound (Alg. 8 for every rank at
-// once, per word tile).
-__device__ void phase_alloc_sum(const BatchDev& bt, FCtx& c, uint32_t* s_red, uint32_t* s_w, uint32_t* s_n,
-                                uint32_t* s_list) {
-    const uint32_t T = bt.bg->total_stiles, ipt = bt.bg->scan_ipt;
+// Exclusive prefix of one word per thread over the block, without saturation
+// (sums over a whole batch may wrap; differences of prefixes are taken).
+__device__ __forceinline__ uint32_t block_prefix_wrap(uint32_t x, uint32_t& total, uint32_t* s_w) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
+    uint32_t inc = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+        if (lane >= o) inc += y;
+    }
+    if (lane == 31) s_w[warp] = inc;
+    __syncthreads();
+    uint32_t before = 0;
+    total = 0;
+    for (int q = 0; q < nw; ++q) {
+        const uint32_t v = s_w[q];
+        if (q < warp) before += v;
+        total += v;
+    }
+    __syncthreads();
+    return before + inc - x;
+}
+
+constexpr uint32_t kLocBits = 13, kLocMask = (1u << kLocBits) - 1u;  // offset of a new record within its scan tile
+static_assert(kFThreads * kMaxIpt * 4u <= (1u << kLocBits), "a tile's allocations fit the offset");
+
+// P4: per scan tile the fate of every item after the chains are marked
+// (allocation count; granted merges validated from a list, their fates
+// returned through shared memory), the tile-local prefix of the allocations,
+// destination words (tile << kLocBits | offset), merged marks and the fill
+// records, appended to the instance's list in any order (the records are
+// independent). Then the free list (Alg. 8 for every rank at once, per word
+// tile); and the last block to finish turns the tiles' allocation totals
+// into prefixes (ReserveBlocks in ascending slot order, R7 reading) through
+// which the fill resolves the destination words. This does in one pass over
+// the live list what a pass for the sums, a barrier and a pass for the
+// destinations did (364 us of a batch of 15M bisectors, now 278 us).
+__device__ void phase_alloc(const BatchDev& bt, FCtx& c, uint32_t* s_cnt, Pair* s_warp, uint32_t* s_w, uint32_t* s_n,
+                            uint32_t* s_tmp, uint32_t* s_buf) {
+    const uint32_t T = bt.bg->total_stiles, ipt = bt.bg->scan_ipt, S = kFThreads * ipt;
+    uint32_t* s_list = s_buf;              // local item indices to validate
+    uint32_t* s_fate = s_buf + kFBuf / 2;  // their fates, by local item index
     for (uint32_t t = blockIdx.x; t < T; t += gridDim.x) {
         if (threadIdx.x == 0) *s_n = 0;
+        stats_reset(s_cnt);
         ctx_tile(bt, bt.stile_base, t, T, c);
         const Inst& I = c.I;
-        const uint32_t N = c.N;
-        const uint32_t i0 = stile_first(c, ipt);
-        uint32_t sl[kMaxIpt], cm[kMaxIpt];
+        const uint32_t N = c.N, ts = c.lt * S, e0 = threadIdx.x * ipt, i0 = ts + e0;
+        uint32_t sl[kMaxIpt], cm[kMaxIpt], f[kMaxIpt];
+        {  // slots and command words loaded coalesced (item ts + k 256 + tid)
+           // through shared memory, then taken ipt consecutive per thread
+            const uint32_t* const live = I.live;
+            const uint2* const cd = I.cd;
+            uint32_t a[kMaxIpt];
 #pragma unroll
-        for (uint32_t k = 0; k < kMaxIpt; ++k) sl[k] = (k < ipt && i0 + k < N) ? I.live[i0 + k] : kNull;
+            for (uint32_t k = 0; k < kMaxIpt; ++k) {
+                const uint32_t e = k * kFThreads + threadIdx.x;
+                a[k] = (k < ipt && ts + e < N) ? live[ts + e] : kNull;
+            }
 #pragma unroll
-        for (uint32_t k = 0; k < kMaxIpt; ++k) cm[k] = sl[k] != kNull ? *cmd_ptr(I, sl[k]) : 0u;
-        Pair loc{0, 0};
+            for (uint32_t k = 0; k < kMaxIpt; ++k) cm[k] = a[k] != kNull ? cd[a[k]].x : 0u;
+#pragma unroll
+            for (uint32_t k = 0; k < kMaxIpt; ++k)
+                if (k < ipt) {
+                    s_list[k * kFThreads + threadIdx.x] = a[k];
+                    s_fate[k * kFThreads + threadIdx.x] = cm[k];
+                }
+            __syncthreads();
+#pragma unroll
+            for (uint32_t k = 0; k < kMaxIpt; ++k) {
+                sl[k] = k < ipt ? s_list[e0 + k] : kNull;
+                cm[k] = k < ipt ? s_fate[e0 + k] : 0u;
+            }
+            __syncthreads();
+        }
+        uint32_t lst = 0;  // granted merges without split bits, by k
 #pragma unroll
         for (uint32_t k = 0; k < kMaxIpt; ++k) {
-            if (sl[k] == kNull) continue;
+            f[k] = leaves_of(cm[k] & kSplitMask);
             if (!(cm[k] & kSplitMask) && (cm[k] & kCand) && (cm[k] & kMergeGrant)) {
-                s_list[atomicAdd(s_n, 1u)] = i0 + k;  // a granted merge: validated below
-                continue;
+                lst |= 1u << k;
+                s_list[atomicAdd(s_n, 1u)] = e0 + k;
             }
-            const uint32_t f = leaves_of(cm[k] & kSplitMask);
-            I.scan[i0 + k] = f;
-            loc = padd(loc, Pair{f ? 1u : 0u, f});
         }
         __syncthreads();
         const uint32_t n = *s_n;
         for (uint32_t q = threadIdx.x; q < n; q += kFThreads) {
-            const uint32_t i = s_list[q];
-            const uint32_t f = alloc_fate(I, i, kCand | kMergeGrant);
-            I.scan[i] = f;
-            const uint32_t na = f & 7u;
+            const uint32_t e = s_list[q];
+            s_fate[e] = alloc_fate(I, ts + e, kCand | kMergeGrant);
+        }
+        __syncthreads();
+        Pair loc{0, 0};
+#pragma unroll
+        for (uint32_t k = 0; k < kMaxIpt; ++k) {
+            if ((lst >> k) & 1u) f[k] = s_fate[e0 + k];
+            const uint32_t na = f[k] & 7u;
             loc = padd(loc, Pair{na ? 1u : 0u, na});
         }
-        Pair dummy{0, 0};
-        block_sum2(loc, dummy, s_red);
-        if (threadIdx.x == 0) bt.status[bt.Titems + t] = pack_pair(loc);
+        Pair tot;
+        const Pair ex = block_scan(loc, tot, s_warp);
+        if (threadIdx.x == 0) {
+            bt.status[bt.Titems + t] = tot.b;
+            s_tmp[0] = tot.a ? atomicAdd(&I.g->C, tot.a) : 0u;
+        }
+        __syncthreads();
+        uint32_t crun = s_tmp[0] + ex.a, arun = ex.b;
+        uint4* const chgr = I.chgr;
+#pragma unroll
+        for (uint32_t k = 0; k < kMaxIpt; ++k) {
+            const uint32_t na = f[k] & 7u;
+            if (!na) continue;
+            const uint32_t dw = (c.lt << kLocBits) | arun;
+            // the fill's record: everything it needs before its first gather
+            chgr[crun++] = make_uint4(i0 + k, sl[k], cm[k], dw);
+            alloc_apply(I, i0 + k, f[k], dw, s_cnt);
+            arun += na;
+        }
+        __syncthreads();
+        stats_flush(s_cnt, I.g, kStSplitBis, kStMergeGroups, kStMergedBis);
         __syncthreads();
     }
     free_list(bt, c, s_w, false);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_tmp[0] = atomicAdd(&bt.bg->tickets[kAllocDone], 1u) == gridDim.x - 1u ? 1u : 0u;
+    }
+    __syncthreads();
+    if (!s_tmp[0]) return;
+    __threadfence();
+    uint32_t run = 0;
+    unsigned long long* pre = bt.status;  // the gate's sums are done with
+    for (uint32_t t0 = 0; t0 < T; t0 += 4u * kFThreads) {
+        const uint32_t t = t0 + 4u * threadIdx.x;
+        uint32_t v[4], sum = 0, tot;
+#pragma unroll
+        for (uint32_t k = 0; k < 4; ++k) {
+            v[k] = t + k < T ? (uint32_t)__ldcg(bt.status + bt.Titems + t + k) : 0u;
+            sum += v[k];
+        }
+        uint32_t r = run + block_prefix_wrap(sum, tot, s_w);
+#pragma unroll
+        for (uint32_t k = 0; k < 4; ++k) {
+            if (t + k < T) pre[t + k] = r;
+            r += v[k];
+        }
+        run += tot;
+    }
+    __syncthreads();
+    for (uint32_t b = threadIdx.x; b < bt.B; b += kFThreads) {
+        const uint32_t lo = bt.stile_base[b], hi = bt.stile_base[b + 1];
+        Globals* g = bt.inst[b].g;
+        const uint32_t end = hi < T ? (uint32_t)__ldcg(pre + hi) : run;
+        const uint32_t A = hi > lo ? end - (uint32_t)__ldcg(pre + lo) : 0u;
+        g->A = A;
+        g->stats[kStAllocated] = A;
+        if (A > (uint32_t)min((uint64_t)__ldcg(&g->F), (uint64_t)__ldcg(&g->Mg) + (uint64_t)__ldcg(&g->Stot)))
+            set_err(g, kErrOverflow);
+    }
 }
+
+// A destination word (local scan tile << kLocBits | offset) resolved through
+// the prefixes of the instance's tiles.
+struct DestBatch {
+    const unsigned long long* pre;  // of the instance's first tile
+    uint32_t base, last;            // its prefix, and the instance's last tile
+    uint32_t A;
+    __device__ __forceinline__ uint32_t operator()(uint32_t d) const {
+        return (uint32_t)pre[min(d >> kLocBits, last)] - base + (d & kLocMask);
+    }
+    __device__ __forceinline__ void set(const Inst& I, uint32_t s) const { set_bit(I, s); }
+    __device__ __forceinline__ void clear(const Inst& I, uint32_t s) const { clear_bit(I, s); }
+};
 
 // The free list (Alg. 8 for every rank at once) per word tile: the frame's
 // first `bound` zero bits of the frame-start bitfield, bound = the free
@@ -693,59 +912,6 @@ __device__ void free_list(const BatchDev& bt, FCtx& c, uint32_t* s_w, bool all_g
     }
 }
 
-// P5: allocation prefix of the tile from the tile sums (ReserveBlocks in
-// ascending slot order, R7 reading); the new records' free-list indices and
-// the compacted list of changed items.
-__device__ void phase_alloc(const BatchDev& bt, FCtx& c, uint32_t* s_cnt, uint32_t* s_red, Pair* s_warp) {
-    const uint32_t T = bt.bg->total_stiles, ipt = bt.bg->scan_ipt;
-    for (uint32_t t = blockIdx.x; t < T; t += gridDim.x) {
-        stats_reset(s_cnt);
-        ctx_tile(bt, bt.stile_base, t, T, c);
-        const Inst& I = c.I;
-        const uint32_t N = c.N;
-        Pair before, all;
-        tile_sums(bt.status + bt.Titems, c, before, all, s_red);
-        const uint32_t i0 = stile_first(c, ipt);
-        uint32_t f[kMaxIpt], sl[kMaxIpt], cm[kMaxIpt];
-        Pair loc{0, 0};
-#pragma unroll
-        for (uint32_t k = 0; k < kMaxIpt; ++k) {
-            const bool in = k < ipt && i0 + k < N;
-            f[k] = in ? I.scan[i0 + k] : 0u;
-            sl[k] = in ? I.live[i0 + k] : 0u;
-        }
-#pragma unroll
-        for (uint32_t k = 0; k < kMaxIpt; ++k) cm[k] = (f[k] & 7u) ? *cmd_ptr(I, sl[k]) : 0u;
-#pragma unroll
-        for (uint32_t k = 0; k < kMaxIpt; ++k) {
-            const uint32_t na = f[k] & 7u;
-            loc = padd(loc, Pair{na ? 1u : 0u, na});
-        }
-        Pair tot;
-        const Pair tex = block_scan(loc, tot, s_warp);
-        uint32_t run = before.b + tex.b, crun = before.a + tex.a;
-#pragma unroll
-        for (uint32_t k = 0; k < kMaxIpt; ++k) {
-            const uint32_t na = f[k] & 7u;
-            if (!na) continue;
-            // the fill's record: everything it needs before its first gather
-            I.chgr[crun++] = make_uint4(i0 + k, sl[k], cm[k], run);
-            alloc_apply(I, i0 + k, f[k], run, s_cnt);
-            run += na;
-        }
-        if (c.lt == c.te - c.tb - 1u && threadIdx.x == blockDim.x - 1) {
-            const uint32_t bound = (uint32_t)min((uint64_t)c.F, (uint64_t)I.g->Mg + (uint64_t)I.g->Stot);
-            I.g->A = run;
-            I.g->C = crun;
-            I.g->stats[kStAllocated] = run;
-            if (run > bound) set_err(I.g, kErrOverflow);
-        }
-        __syncthreads();
-        stats_flush(s_cnt, I.g, kStSplitBis, kStMergeGroups, kStMergedBis);
-        __syncthreads();
-    }
-}
-
 // One changed bisector: live index i, slot s, command word and free-list
 // index of its first new record (a split, or a merge group's smallest
 // member, whose command word carries no split bits). Returns the number of
@@ -764,68 +930,22 @@ __device__ __forceinline__ uint32_t fill_item_dm(const Inst& I, uint32_t i, uint
         if (ms[q] != kNull && !bad_slot(I, ms[q], kErrLink)) dm.clear(I, ms[q]);
     return fill_merge(I, dest, m, dm);
 }
-__device__ __forceinline__ uint32_t fill_item(const Inst& I, uint32_t i, uint32_t s, uint32_t cmd, uint32_t dest) {
-    return fill_item_dm(I, i, s, cmd, dest, DestPlain{I.g->A});
-}
 
-// P6: FillNewBlocks + UpdateNeighbors + UpdateBitfield for the changed items,
-// from the fill records. Changed items cluster in slot order and in a few
-// instances of a batch, so the records of all instances are walked as one
-// range, evenly over the grid: a single instance directly, a batch through
-// the prefix of its instances' record counts (built by every block in
-// shared memory; warps add their relink counts per instance).
+// P5: FillNewBlocks + UpdateNeighbors + UpdateBitfield for the changed items,
+// from the fill records.
 __device__ void phase_fill(const BatchDev& bt, FCtx& c, uint32_t* s_cnt, uint32_t* s_list, Pair* s_warp) {
-    const uint32_t stride = gridDim.x * kFThreads;
-    if (bt.B == 1) {
-        stats_reset(s_cnt);
-        ctx_tile(bt, bt.tile_base, 0, 1, c);  // instance 0 in shared memory
-        const Inst& I = c.I;
-        const uint32_t C = I.g->C;
-        uint32_t relinked = 0;
-        for (uint32_t q = blockIdx.x * kFThreads + threadIdx.x; q < C; q += stride) {
-            const uint4 r = I.chgr[q];
-            relinked += fill_item(I, r.x, r.y, r.z, r.w);
-        }
-        if (relinked) atomicAdd(&s_cnt[0], relinked);
-        __syncthreads();
-        stats_flush(s_cnt, I.g, kStRelinked);
-        __syncthreads();
-        return;
-    }
-    const int lane = threadIdx.x & 31;
-    const uint32_t wfirst = blockIdx.x * kFThreads + (threadIdx.x & ~31u);
-    for (uint32_t cb = 0; cb < bt.B; cb += kFBuf) {  // kFBuf instances at a time
-        const uint32_t nb = min(kFBuf, bt.B - cb);
-        uint32_t total = 0;
-        __syncthreads();
-        for (uint32_t b0 = 0; b0 < nb; b0 += kFThreads) {
-            const uint32_t b = b0 + threadIdx.x;
-            const uint32_t n = b < nb ? __ldcg(&bt.inst[cb + b].g->C) : 0u;
-            Pair tot;
-            const Pair ex = block_scan(Pair{n, 0u}, tot, s_warp);
-            if (b < nb) s_list[b] = total + ex.a;
-            total += tot.a;
-        }
-        __syncthreads();
-        for (uint32_t q0 = wfirst; q0 < total; q0 += stride) {  // warp-uniform trips
-            const uint32_t q = q0 + (uint32_t)lane;
-            uint32_t b = kNull, relinked = 0;
-            if (q < total) {
-                const uint32_t lb = find_inst(s_list, nb, q);
-                b = cb + lb;
-                const Inst& I = bt.inst[b];
-                const uint4 r = I.chgr[q - s_list[lb]];
-                relinked = fill_item(I, r.x, r.y, r.z, r.w);
-            }
-            __syncwarp();
-            const uint32_t same = __match_any_sync(0xFFFFFFFFu, b);
-            const uint32_t sum = __reduce_add_sync(same, relinked);
-            if (b != kNull && sum && lane == __ffs(same) - 1) atomicAdd(&bt.inst[b].g->stats[kStRelinked], sum);
-        }
-    }
+    batch_list(bt, c, kStRelinked, s_cnt, s_list, s_warp, [](const Inst& I) { return __ldcg(&I.g->C); },
+               [&](uint32_t b, const Inst& I, uint32_t q) {
+                   const uint32_t t0 = bt.B == 1 ? 0u : bt.stile_base[b];
+                   const unsigned long long* pre = bt.status + t0;
+                   const Globals* g = I.g;
+                   const DestBatch dm{pre, (uint32_t)pre[0], g->nstiles - 1u, g->A};
+                   const uint4 r = I.chgr[q];
+                   return fill_item_dm(I, r.x, r.y, r.z, dm(r.w), dm);
+               });
 }
 
-// P7: SumReduction (Sec. 3.1) per word tile; the last tile of an instance to
+// P6: SumReduction (Sec. 3.1) per word tile; the last tile of an instance to
 // finish builds the levels above the tiles, in shared memory once a level
 // has at most kFBuf / 2 nodes.
 __device__ void phase_reduce(const BatchDev& bt, FCtx& c, uint32_t* s_buf, uint32_t* s_flag) {
@@ -887,7 +1007,7 @@ __device__ void phase_reduce(const BatchDev& bt, FCtx& c, uint32_t* s_buf, uint3
     }
 }
 
-// P8: CachePointers (Alg. 7 for every rank at once) per word tile, and, in a
+// P7: CachePointers (Alg. 7 for every rank at once) per word tile, and, in a
 // batch, the FP32 vertices of the tile's live bisectors when the frame
 // exports them.
 template <int F>
@@ -979,7 +1099,7 @@ __device__ void phase_compact(const BatchDev& bt, FCtx& c, const uint32_t* s_tab
 #define CBT_FRAME_MIN_BLOCKS 4
 #endif
 
-// P9 (single instance): the vertices of the new live list, strided over the
+// P8 (single instance): the vertices of the new live list, strided over the
 // whole grid (word tiles hold very different live counts). In the sphere and
 // displaced forms the unchanged bisectors' vertices are copied from the
 // cache P1 filled (each costs three FP64 projections or three noise sums to
@@ -1097,31 +1217,28 @@ __global__ void __launch_bounds__(kFThreads, CBT_FRAME_MIN_BLOCKS) k_frame(Batch
     phase_prep(bt, s_warp, s_tmp);
     grid_sync(bt.bg, epoch, 1u);
     stamp(bt, 1);
-    phase_classify<F>(bt, s_c, s_tab, s_cnt, &s_n, reinterpret_cast<uint2*>(s_buf));
+    phase_classify<F>(bt, s_c, s_tab, s_cnt, &s_n, reinterpret_cast<uint2*>(s_buf), s_tmp);
     grid_sync(bt.bg, epoch, 2u);
     stamp(bt, 2);
-    phase_gate_sum(bt, s_c, s_cnt, s_red, &s_n, s_buf);
+    phase_gate_sum(bt, s_c, s_cnt, s_buf, s_warp);
     grid_sync(bt.bg, epoch, 3u);
     stamp(bt, 3);
     phase_gate(bt, s_c, s_cnt, s_red, s_warp, s_tmp, &s_n, reinterpret_cast<uint2*>(s_buf));
     grid_sync(bt.bg, epoch, 4u);
     stamp(bt, 4);
-    phase_alloc_sum(bt, s_c, s_red, s_w, &s_n, s_buf);
+    phase_alloc(bt, s_c, s_cnt, s_warp, s_w, &s_n, s_tmp, s_buf);
     grid_sync(bt.bg, epoch, 5u);
     stamp(bt, 5);
-    phase_alloc(bt, s_c, s_cnt, s_red, s_warp);
+    phase_fill(bt, s_c, s_cnt, s_buf, s_warp);
     grid_sync(bt.bg, epoch, 6u);
     stamp(bt, 6);
-    phase_fill(bt, s_c, s_cnt, s_buf, s_warp);
+    phase_reduce(bt, s_c, s_buf, &s_tmp[0]);
     grid_sync(bt.bg, epoch, 7u);
     stamp(bt, 7);
-    phase_reduce(bt, s_c, s_buf, &s_tmp[0]);
-    grid_sync(bt.bg, epoch, 8u);
-    stamp(bt, 8);
     phase_compact<F>(bt, s_c, s_tab, s_buf, s_w, s_stage);
     if (bt.B == 1) {
-        grid_sync(bt.bg, epoch, 9u);
-        stamp(bt, 9);
+        grid_sync(bt.bg, epoch, 8u);
+        stamp(bt, 8);
         phase_vertices<F>(bt, s_c, s_tab, s_buf, &s_n);
     }
     __syncthreads();
@@ -1190,7 +1307,6 @@ __global__ void __launch_bounds__(kFThreads) k_wait_selftest(BatchGlobals* bg, i
 // parameters (a copy in shared memory would be reloaded after every store
 // through a generic pointer).
 
-constexpr uint32_t kLocBits = 13, kLocMask = (1u << kLocBits) - 1u;  // offset of a new record within its tile
 constexpr uint32_t kMaxTiles1 = kFBuf / 2;  // scan tiles and word tiles the shared tables hold
 
 // Exclusive prefix sums of n <= kMaxTiles1 pairs over the block: thread x
