@@ -413,9 +413,8 @@ class CBT:
         return slots[:n], heap[:n], links[:n]
 
     def vertices(self, origin, precision=0, fixed_shift=20, out=None, stream=None):
-        n = self.live_count(stream)
         if out is None:
-            out = torch.empty((max(n, 1), 3, 3), dtype=torch.float32, device=self.device)
+            out = torch.empty((max(self.live_count(stream), 1), 3, 3), dtype=torch.float32, device=self.device)
         o = (C.c_double * 3)(*[float(x) for x in origin])
         cnt = C.c_uint32()
         rc = _lib.cbt_vertices(self._h, _t_ptr(out), o, precision, fixed_shift, out.shape[0],

@@ -207,7 +207,7 @@ struct cbt_state {
     Inst inst;
     uint32_t* corner;  // [H][3] global points of the root corners: vert[h], vert[next h], V + face[h]
     uint32_t npts;     // global points: 1 + the largest in corner
-    uint32_t* h_ix = nullptr;  // pinned counts of the last cbt_index (made by its first call)
+    uint32_t* h_ix = nullptr;  // pinned counts: of the last cbt_index (words 0 to 2) and cbt_vertices (3)
     void* workspace;
     size_t bytes;
     int sms;
@@ -726,15 +726,27 @@ extern "C" int cbt_leaves(cbt_state* st, uint32_t* d_slots, uint64_t* d_heap, ui
     return cudaStreamSynchronize(s) == cudaSuccess ? CBT_OK : CBT_ECUDA;
 }
 
+namespace {
+// The state's page-locked counts (made by the first call that needs them) and
+// their address on the device.
+int pinned_counts(cbt_state* st, uint32_t** d) {
+    if (!st->h_ix && cudaMallocHost(reinterpret_cast<void**>(&st->h_ix), 16u) != cudaSuccess) {
+        st->h_ix = nullptr;
+        return CBT_ECUDA;
+    }
+    return cudaHostGetDevicePointer(reinterpret_cast<void**>(d), st->h_ix, 0) == cudaSuccess ? CBT_OK : CBT_ECUDA;
+}
+}  // namespace
+
 extern "C" int cbt_vertices(cbt_state* st, float* d_out, const double h_origin[3], uint32_t precision,
                             int32_t fixed_shift, uint32_t cap, uint32_t* h_count, cbt_stream_t stream) {
     if (!st || !d_out || !h_origin || precision > 2u || fixed_shift < 0 || fixed_shift > 62)
         return CBT_EINVAL;
-    uint32_t n = 0;
-    int rc = cbt_live_count(st, &n, stream);
+    // one synchronisation: the export checks the live count on the device
+    // (reading it back first, and waiting for that, took 8 us of 85 a call)
+    uint32_t* d_counts = nullptr;
+    int rc = pinned_counts(st, &d_counts);
     if (rc) return rc;
-    if (h_count) *h_count = n;
-    if (n > cap) return CBT_ENOMEM;
     cbt_batch* B = st->self;
     FrameP fp;
     std::memset(&fp, 0, sizeof(fp));
@@ -748,10 +760,14 @@ extern "C" int cbt_vertices(cbt_state* st, float* d_out, const double h_origin[3
     bt.fp0 = fp;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     launch_prep(bt, false, grid_prep(B), s);
+    bt.vcount = d_counts + 3;
     launch_vertices(bt, form_of(fp), std::max(1, static_cast<int>(std::min<uint32_t>(bt.Titems, static_cast<uint32_t>(st->sms) * 8u))), s);
     rc = check_launch();
     if (rc) return rc;
-    return cudaStreamSynchronize(s) == cudaSuccess ? CBT_OK : CBT_ECUDA;
+    if (cudaStreamSynchronize(s) != cudaSuccess) return CBT_ECUDA;
+    const uint32_t n = reinterpret_cast<volatile uint32_t*>(st->h_ix)[3];
+    if (h_count) *h_count = n;
+    return n > cap ? CBT_ENOMEM : CBT_OK;
 }
 
 extern "C" int cbt_host_device_pointer(void* h_ptr, void** d_ptr) {
@@ -804,10 +820,9 @@ extern "C" int cbt_index(cbt_state* st, const float* d_tri_vertices, void* d_wor
         (reinterpret_cast<uintptr_t>(d_heap) & 7u) || (reinterpret_cast<uintptr_t>(d_vertices) & 3u) ||
         (reinterpret_cast<uintptr_t>(d_tri_vertices) & 3u))
         return CBT_EINVAL;
-    if (!st->h_ix && cudaMallocHost(reinterpret_cast<void**>(&st->h_ix), 16u) != cudaSuccess) {
-        st->h_ix = nullptr;
-        return CBT_ECUDA;
-    }
+    uint32_t* d_counts = nullptr;
+    const int rc = pinned_counts(st, &d_counts);
+    if (rc) return rc;
     return launch_index(st->inst, st->corner, st->npts, triangles_cap, d_workspace, bytes, d_tri_vertices, d_vertices,
                         vertices_cap, d_indices, d_heap, st->sms, reinterpret_cast<cudaStream_t>(stream), st->h_ix,
                         h_nvertices, h_ntriangles);

@@ -211,6 +211,8 @@ struct BatchDev {
     unsigned long long* status;  // [2 * Titems + Twords] look-back descriptors
     uint32_t Titems, Twords, Trel;
     uint32_t* nout;              // optional [B]: live count at frame start per instance
+    uint32_t* vcount;            // the export on its own (B == 1): the live count goes here, in mapped
+                                 // host memory, and nothing else is written when it exceeds vcap
     uint32_t timing;             // one-launch frame: record phase boundaries
     uint32_t* tpre;              // single-instance frame: [2][Twords] ones before each word tile of
                                  // the next frame's starting bitfield, by frame parity

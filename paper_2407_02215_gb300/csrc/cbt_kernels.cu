@@ -659,7 +659,12 @@ __global__ void __launch_bounds__(kThreads, 3) k_vertices(BatchDev bt) {
         tile_begin(bt, bt.vtile_base, t, &s_b, &s_I, &s_fp, nullptr, b, lt);
         const Inst& I = s_I;
         const FrameP& fp = s_fp;
-        const uint32_t N = fp.vout ? min(I.sums[1], fp.vcap) : 0u;
+        uint32_t N = fp.vout ? min(I.sums[1], fp.vcap) : 0u;
+        if (bt.vcount) {
+            const uint32_t live = I.sums[1];
+            if (t == 0 && threadIdx.x == 0) *reinterpret_cast<volatile uint32_t*>(bt.vcount) = live;
+            if (live > fp.vcap) N = 0u;
+        }
         if (lt * kTileItems < N) {
             uint64_t hj[kItemsPerThread];
 #pragma unroll
