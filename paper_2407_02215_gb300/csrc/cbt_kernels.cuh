@@ -37,6 +37,7 @@ cudaError_t launch_frame(const BatchDev& bt, int form, int grid, cudaStream_t s)
 // It holds its scan-tile and word-tile tables in shared memory, so it takes
 // pools of at most kFrame1MaxCap slots with 64-word tiles.
 constexpr uint32_t kFrame1MaxCap = 1u << 22;
+constexpr uint32_t kFrame1SmallCap = 1u << 16;  // pools up to this run with two blocks per SM
 constexpr uint32_t kFrame1TileWords = 64;
 constexpr int kFrame1Phases = 8;
 int frame1_blocks_per_sm();
