@@ -97,7 +97,7 @@ struct Globals {
     // wish to merge) and requested split cost, summed by the walks; when their
     // sum fits the free slots every request is granted without the prefix gate
     unsigned long long rq_merge, rq_split;
-    uint32_t nwalk;  // single-instance frame: entries of the frame's walk list; batch frame: listed merge groups
+    uint32_t nwalk;  // single-instance frame: entries of the frame's walk list
     uint32_t marks_clean;  // 1 when the chain-mark words (chg) of the live slots are 0 (the
                            // single-instance frame leaves them so; the other frames clear this)
     uint32_t freel_full;   // 1 when freel lists every zero bit of the bitfield in slot order

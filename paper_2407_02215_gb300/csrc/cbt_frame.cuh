@@ -3,8 +3,8 @@
 // separated by grid-wide barriers instead of kernel boundaries.
 //
 //   P0 prep       frame counters, item-tile prefix, camera-relative roots
-//   P1 classify   LOD wishes, then the chain and group walks of the same tile
-//   P2 gate-sum   merge candidates among the listed groups, and their costs
+//   P1 classify   LOD wishes; what needs a walk listed, split costs bounded
+//   P2 gate-sum   chain and group walks of what the gate could grant; cost sums
 //   P3 gate       tile prefix from the tiles' cost sums, grants, chain marking
 //   P4 alloc      fates, tile-local allocation prefixes, fill records; free list
 //   P5 fill       new records, neighbour links, bitfield
@@ -198,7 +198,6 @@ __device__ void phase_prep(const BatchDev& bt, Pair* s_warp, uint32_t* s_tmp) {
                 g->Stot = 0;
                 g->C = 0;
                 g->done = 0;
-                g->nwalk = 0;
                 g->marks_clean = 0;
                 g->freel_full = 0;
                 tiles = (N + kTileItems - 1u) / kTileItems;
@@ -244,175 +243,251 @@ __device__ void phase_prep(const BatchDev& bt, Pair* s_warp, uint32_t* s_tmp) {
         const uint32_t nw = nb * (kFThreads / 32), wid = bb * (kFThreads / 32) + threadIdx.x / 32u;
         const uint32_t per = min(kRelRange, ((bt.Trel + nw - 1u) / nw + 31u) & ~31u);
         for (uint32_t e = wid * per; e < bt.Trel; e += nw * per) rel_range(bt, e, min(bt.Trel, e + per));
-        // the scan tiles' cost sums (at most one tile per kTileItems slots)
-        for (uint32_t t = bb * kFThreads + threadIdx.x; t < bt.Titems; t += nb * kFThreads) bt.status[t] = 0ull;
+        // the tiles' sums: costs per scan tile, lower bounds per item tile and
+        // per 32 item tiles
+        const uint32_t sums = 2u * bt.Titems + bt.Twords;
+        for (uint32_t t = bb * kFThreads + threadIdx.x; t < sums; t += nb * kFThreads) bt.status[t] = 0ull;
     }
 }
 
-constexpr uint32_t kWalkCap = kFBuf / 4;  // uint2 entries of the walk list (the groups found take the other half)
-static_assert(kWalkCap >= kTileItems, "a tile's walks fit");
-
-// Where the walks of an instance leave what the gate needs: the split costs
-// per scan tile (S items) and the list of its merge groups (the per-step
-// form's list of changed items), with its length in the counters.
-struct WalkOut {
-    unsigned long long* sums;
-    uint32_t S;
-    uint32_t* groups;
-    uint32_t* ngroups;
-};
-__device__ __forceinline__ WalkOut walk_out(const BatchDev& bt, const Inst& I, uint32_t b) {
-    return WalkOut{bt.status + (bt.B == 1 ? 0u : bt.stile_base[b]), kFThreads * bt.bg->scan_ipt, I.chg, &I.g->nwalk};
+// Lower-bound costs of the split wishes, per item tile of the batch and per 32
+// item tiles of instance b (after the scan tiles' sums; an instance has at
+// least as many word tiles as it has 32 item tiles).
+__device__ __forceinline__ unsigned long long* bound_sums(const BatchDev& bt) { return bt.status + bt.Titems; }
+__device__ __forceinline__ unsigned long long* bound_groups(const BatchDev& bt, uint32_t b) {
+    return bt.status + 2u * bt.Titems + (bt.B == 1 ? 0u : bt.wtile_base[b]);
 }
-
-// Walks of listed items on the frame-start state: the chain cost of a split
-// wish (command form of Alg. 3, its members recorded in its grp word for the
-// marking) and its share of the scan tile's sum; the Alg. 4 group of a merge
-// wish with an even heap ID (its smallest member records the members and is
-// listed).
-// Called by the whole block with at most kWalkCap entries, which the groups
-// found follow in shared memory until one atomic reserves their place; split
-// costs leave as one atomic per warp and scan tile. (An atomic per walk made
-// classify of a batch of 15M bisectors 900 us instead of 680.)
-__device__ __forceinline__ void walk_list(const Inst& I, const WalkOut& o, uint2* s_list, uint32_t n,
-                                          uint32_t* s_ng) {
-    const uint32_t lane = threadIdx.x & 31u;
-    uint32_t* s_groups = reinterpret_cast<uint32_t*>(s_list + kWalkCap);
-    if (threadIdx.x == 0) s_ng[0] = 0;
-    __syncthreads();
-    for (uint32_t q0 = threadIdx.x & ~31u; q0 < n; q0 += kFThreads) {  // warp-uniform
-        const uint32_t q = q0 + lane;
-        uint32_t cost = 0, t = kNull;
-        if (q < n) {
-            const uint2 e = s_list[q];
-            const uint32_t s = e.y, i = e.x & 0x7FFFFFFFu;
-            if (e.x & 0x80000000u) {
-                uint4 rec;
-                cost = chain_walk(I, s, depth_of(I.heap[s], I.ch), false, &rec);
-                I.scan[i] = cost;
-                I.grp[i] = rec;
-                t = i / o.S;
-            } else {
-                Group g;
-                if (find_group(I, s, g) && g.imin == 0) {
-                    I.grp[i] = make_uint4(g.m[0], g.m[1], g.m[2], g.m[3]);
-                    atomicOr(cmd_ptr(I, s), kGrpMin);
-                    s_groups[atomicAdd(s_ng, 1u)] = i;
-                }
-            }
-        }
-        __syncwarp();
-        if (__any_sync(0xFFFFFFFFu, cost != 0u)) {
-            const unsigned m = __match_any_sync(0xFFFFFFFFu, t);
-            const uint32_t sum = __reduce_add_sync(m, cost);
-            if (t != kNull && lane == (uint32_t)(__ffs(m) - 1)) atomicAdd(o.sums + t, (unsigned long long)sum);
-        }
-    }
-    __syncthreads();
-    const uint32_t ng = s_ng[0];
-    if (threadIdx.x == 0 && ng) s_ng[1] = atomicAdd(o.ngroups, ng);
-    __syncthreads();
-    for (uint32_t q = threadIdx.x; q < ng; q += kFThreads) o.groups[s_ng[1] + q] = s_groups[q];
+// A warp's 128 items of a tile: their walk entries (16 bits each: item, bit 7
+// for a split wish, bit 8 for one whose root halfedge has a Twin) from the
+// second word of the items' fill records (written only in P4), the number of
+// entries in the first.
+constexpr uint32_t kSubItems = kTileItems / (kFThreads / 32);
+static_assert(kSubItems == 128u, "7-bit items");
+__device__ __forceinline__ uint32_t* walk_region(const Inst& I, uint32_t i) {
+    return reinterpret_cast<uint32_t*>(I.chgr + i);
 }
-
-template <int F>
-__device__ __forceinline__ void classify_one(const Inst& I, const FrameP& fp, const WalkOut& o, uint64_t key,
-                                             uint32_t i, uint32_t s, uint64_t j, const uint32_t* s_tab,
-                                             uint32_t* s_cnt, bool chain, uint32_t* s_n, uint2* s_list) {
-    const uint32_t cmd = classify_item<F>(I, fp, key, i, s, j, s_tab, s_cnt, vc_form<F>(fp) && fp.vout);
-    const bool split = (cmd & kSplitWish) && chain;
-    const bool group = (cmd & kMergeWish) && !(cmd & kHeapOdd);
-    if (split || group) s_list[atomicAdd(s_n, 1u)] = make_uint2(i | (split ? 0x80000000u : 0u), s);
-    // the paper's gate: the cost classify_item has set, without a walk
-    if ((cmd & kSplitWish) && !chain) atomicAdd(o.sums + i / o.S, (unsigned long long)I.scan[i]);
+// Whether a split of bisector j has an allocation bound of 4, else 2: every
+// bisector under a root whose halfedge has a Twin has one (its refinement
+// edge is inside the root triangle, on an edge to the face's centroid, or on
+// that halfedge), and its chain then costs itself and the Twin's pair.
+__device__ __forceinline__ bool has_twin_bound(const Inst& I, uint64_t j) {
+    const int d = depth_of(j, I.ch);
+    const uint32_t h = d >= 0 ? (uint32_t)((j >> d) - (1ull << I.ch)) : kNull;
+    return h < I.H && !((__ldg(I.rbnd + (h >> 5)) >> (h & 31u)) & 1u);
 }
-
 
 // P1: wishes of every live bisector (Sec. 3.3 GenerateCommands with the R8
-// LOD reading), then the walks of the listed items. A single instance
-// strides its live list over the whole grid (balanced; the slot and heap ID
-// of the next rounds are loaded while the current item is classified); a
-// batch walks its item tiles.
+// LOD reading) over item tiles, each warp on its own 128 items of the tile;
+// the items that need a walk listed in place, and the split wishes' lower
+// bounds summed for the walks.
 template <int F>
-__device__ void phase_classify(const BatchDev& bt, FCtx& c, uint32_t* s_tab, uint32_t* s_cnt, uint32_t* s_n,
-                               uint2* s_list, uint32_t* s_ng) {
-    if (bt.B == 1) {
-        if (threadIdx.x == 0) *s_n = 0;
-        stats_reset(s_cnt);
-        ctx_tile(bt, bt.tile_base, 0, 1, c);
-        const Inst& I = c.I;
-        const FrameP& fp = c.fp;
-        const uint32_t N = c.N;
-        const bool chain = fp.gate != 1;
-        const WalkOut wo = walk_out(bt, I, c.b);
-        const uint64_t key = splitmix64(((uint64_t)fp.seed << 32) | (uint64_t)fp.frame);
-        const uint32_t stride = gridDim.x * kFThreads;
-        uint32_t i = blockIdx.x * kFThreads + threadIdx.x;
-        uint32_t sa = i < N ? I.live[i] : 0u;
-        uint64_t ja = i < N ? I.heap[sa] : 0ull;
-        uint32_t sb = i + stride < N ? I.live[i + stride] : 0u;
-        for (uint32_t base = blockIdx.x * kFThreads; base < N; base += stride, i += stride) {
-            const uint32_t sc = i + 2u * stride < N ? I.live[i + 2u * stride] : 0u;
-            const uint64_t jb = i + stride < N ? I.heap[sb] : 0ull;
-            if (i < N) classify_one<F>(I, fp, wo, key, i, sa, ja, s_tab, s_cnt, chain, s_n, s_list);
-            sa = sb;
-            ja = jb;
-            sb = sc;
-            __syncthreads();
-            const uint32_t n = *s_n;
-            __syncthreads();
-            if (n > kWalkCap - kFThreads) {  // block-uniform
-                walk_list(I, wo, s_list, n, s_ng);
-                __syncthreads();
-                if (threadIdx.x == 0) *s_n = 0;
-                __syncthreads();
-            }
-        }
-        __syncthreads();
-        walk_list(I, wo, s_list, *s_n, s_ng);
-        __syncthreads();
-        stats_flush(s_cnt, I.g, kStSplitWishes);
-        __syncthreads();
-        return;
-    }
-    const uint32_t T = bt.bg->total_tiles;
+__device__ void phase_classify(const BatchDev& bt, FCtx& c, uint32_t* s_tab, uint32_t* s_cnt) {
+    const uint32_t T = bt.bg->total_tiles, S = kFThreads * bt.bg->scan_ipt;
+    const uint32_t lane = threadIdx.x & 31u;
     for (uint32_t t = blockIdx.x; t < T; t += gridDim.x) {
-        if (threadIdx.x == 0) *s_n = 0;
         stats_reset(s_cnt);
         ctx_tile(bt, bt.tile_base, t, T, c);
         const Inst& I = c.I;
         const FrameP& fp = c.fp;
         const uint32_t N = c.N;
-        const uint32_t lt = c.lt;
         const bool chain = fp.gate != 1;
-        const WalkOut wo = walk_out(bt, I, c.b);
+        const bool cache = vc_form<F>(fp) && fp.vout;
         const uint64_t key = splitmix64(((uint64_t)fp.seed << 32) | (uint64_t)fp.frame);
+        const uint32_t w0 = c.lt * kTileItems + kSubItems * (threadIdx.x >> 5);
         uint32_t sl[kFPer];
         uint64_t hj[kFPer];
 #pragma unroll
         for (int k = 0; k < kFPer; ++k) {
-            const uint32_t i = lt * kTileItems + (uint32_t)k * kFThreads + threadIdx.x;
+            const uint32_t i = w0 + 32u * (uint32_t)k + lane;
             sl[k] = i < N ? I.live[i] : 0u;
         }
 #pragma unroll
-        for (int k = 0; k < kFPer; ++k) {
-            const uint32_t i = lt * kTileItems + (uint32_t)k * kFThreads + threadIdx.x;
-            hj[k] = i < N ? I.heap[sl[k]] : 0ull;
-        }
+        for (int k = 0; k < kFPer; ++k) hj[k] = w0 + 32u * (uint32_t)k + lane < N ? I.heap[sl[k]] : 0ull;
+        uint32_t n = 0, bound = 0, paper = 0;
+        if (w0 < N) {
+            uint32_t* const reg = walk_region(I, w0);
+            uint16_t* const list = reinterpret_cast<uint16_t*>(reg + 1);
 #pragma unroll 1
-        for (int k = 0; k < kFPer; ++k) {
-            const uint32_t i = lt * kTileItems + (uint32_t)k * kFThreads + threadIdx.x;
-            if (i < N) classify_one<F>(I, fp, wo, key, i, sl[0], hj[0], s_tab, s_cnt, chain, s_n, s_list);
+            for (uint32_t k = 0; k < (uint32_t)kFPer; ++k) {
+                const uint32_t x = 32u * k + lane, i = w0 + x;
+                bool split = false, walk = false, twin = false;
+                uint32_t cost = 0;
+                if (i < N) {
+                    const uint32_t cmd = classify_item<F>(I, fp, key, i, sl[0], hj[0], s_tab, s_cnt, cache);
+                    split = (cmd & kSplitWish) != 0u;
+                    twin = split && has_twin_bound(I, hj[0]);
+                    walk = (split && chain) || ((cmd & kMergeWish) && !(cmd & kHeapOdd));
+                    // the paper's gate: the cost classify_item has set, without a walk
+                    if (split && !chain) cost = 3u * (uint32_t)depth_of(hj[0], I.ch) + 4u;
+                }
+                const unsigned wm = __ballot_sync(0xFFFFFFFFu, walk);
+                if (walk)
+                    list[n + __popc(wm & ((1u << lane) - 1u))] =
+                        (uint16_t)(x | (split ? 128u : 0u) | (twin ? 256u : 0u));
+                n += __popc(wm);
+                if (chain)
+                    bound += 2u * (__popc(__ballot_sync(0xFFFFFFFFu, split)) + __popc(__ballot_sync(0xFFFFFFFFu, twin)));
+                else
+                    paper += __reduce_add_sync(0xFFFFFFFFu, cost);
 #pragma unroll
-            for (int q = 0; q + 1 < kFPer; ++q) {  // constant indices: registers, not local memory
-                sl[q] = sl[q + 1];
-                hj[q] = hj[q + 1];
+                for (int q = 0; q + 1 < kFPer; ++q) {  // constant indices: registers, not local memory
+                    sl[q] = sl[q + 1];
+                    hj[q] = hj[q + 1];
+                }
+            }
+            if (lane == 0) {
+                reg[0] = n;
+                if (bound) {
+                    atomicAdd(bound_sums(bt) + t, (unsigned long long)bound);
+                    atomicAdd(bound_groups(bt, c.b) + (c.lt >> 5), (unsigned long long)bound);
+                }
+                if (paper) atomicAdd(bt.status + (bt.B == 1 ? 0u : bt.stile_base[c.b]) + w0 / S, (unsigned long long)paper);
             }
         }
         __syncthreads();
-        walk_list(I, wo, s_list, *s_n, s_ng);
-        __syncthreads();
         stats_flush(s_cnt, I.g, kStSplitWishes);
+        __syncthreads();
+    }
+}
+
+// Alg. 4 group of s1 (heap ID j1, a merge wish) on the frame-start state,
+// walked only while s1 can be its smallest member and every member wishes
+// to merge: true when both hold, with the members (m[0] = s1, m[1] its
+// sibling, m[2] the bisector across the outer half of the refinement edge,
+// m[3] its sibling) and the parents' count.
+static __device__ bool group_if_mergeable(const Inst& I, uint32_t s1, uint64_t j1, Group& g) {
+    if (depth_of(j1, I.ch) < 1) return false;
+    const uint4 r1 = I.nb[s1];
+    const bool bit = j1 & 1ull;
+    const uint32_t s2 = bit ? r1.z : r1.y;
+    const uint32_t s3 = bit ? r1.y : r1.z;
+    if (s2 == kNull || bad_slot(I, s2, kErrLink)) return false;
+    if (s3 != kNull && bad_slot(I, s3, kErrLink)) return false;
+    const uint64_t j2 = I.heap[s2];
+    const uint32_t c2 = *cmd_ptr(I, s2);
+    uint64_t j3 = 0ull;
+    uint4 r3 = make_uint4(kNull, kNull, kNull, 0u);
+    uint32_t c3 = 0u;
+    if (s3 != kNull) {
+        j3 = I.heap[s3];
+        r3 = I.nb[s3];
+        c3 = *cmd_ptr(I, s3);
+    }
+    if ((j2 >> 1) != (j1 >> 1) || j2 < j1 || !(c2 & kMergeWish)) return false;
+    g.m[0] = s1;
+    g.m[1] = s2;
+    g.m[2] = g.m[3] = kNull;
+    g.n = 2;
+    g.np = 1;
+    g.imin = 0;
+    if (s3 != kNull) {
+        // the other pair's smaller member is its even one
+        if (bitlen64(j3) != bitlen64(j1) || (j3 >> 1) == (j1 >> 1) || (j3 & ~1ull) < j1 || !(c3 & kMergeWish))
+            return false;
+        const uint32_t s4 = bit ? r3.y : r3.z;
+        if (s4 == kNull || bad_slot(I, s4, kErrLink)) return false;
+        const uint64_t j4 = I.heap[s4];
+        const uint32_t c4 = *cmd_ptr(I, s4);
+        if ((j4 >> 1) != (j3 >> 1) || !(c4 & kMergeWish)) return false;
+        g.m[2] = s3;
+        g.m[3] = s4;
+        g.n = 4;
+        g.np = 2;
+    }
+    return true;
+}
+
+// P2: the walks, per item tile. A split wish is denied whatever its cost when
+// the lower bounds (2, or 4 with a Twin) of the instance's split wishes before
+// its tile plus its own exceed the free slots F: in a tile where the bounds
+// before it do so alone, no split here or later can be granted and their
+// costs are left out; else the bound stands in for such a wish's cost, so that
+// the splits after it are denied on these costs as on the true ones. The
+// other splits walk their chains (command form of Alg. 3: cost, members for
+// the marking). A merge wish with an even heap ID walks its Alg. 4 group
+// while it can be a candidate with this wish its smallest member, which then
+// records the members. Costs go to the scan tile's sums.
+// Without the bounds every wish of a full pool walked its chain only to be
+// denied: 6.6M wishes of a batch of 15M bisectors, 0.7M granted; its classify
+// with the walks took 680 us and the gate's sums 67, these two phases 427 and 343 (in a
+// nearly full 2^23-slot pool 290 and 10, now 165 and 110).
+__device__ void phase_walks(const BatchDev& bt, FCtx& c, uint32_t* s_cnt, unsigned long long* s_red, uint32_t* s_tmp,
+                            uint32_t* s_n) {
+    const uint32_t T = bt.bg->total_tiles, S = kFThreads * bt.bg->scan_ipt;
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    for (uint32_t t = blockIdx.x; t < T; t += gridDim.x) {
+        if (threadIdx.x < 3) s_tmp[threadIdx.x] = 0;
+        stats_reset(s_cnt);
+        ctx_tile(bt, bt.tile_base, t, T, c);
+        const Inst& I = c.I;
+        const uint32_t N = c.N, F = c.F, lt = c.lt, i0 = lt * kTileItems;
+        const uint32_t gate = c.fp.gate;
+        // the bounds before the tile: the earlier groups of 32 tiles, then the
+        // earlier tiles of its group
+        unsigned long long before = 0;
+        const unsigned long long* G = bound_groups(bt, c.b);
+        for (uint32_t g = threadIdx.x; g < (lt >> 5); g += kFThreads) before += __ldcg(G + g);
+        if (threadIdx.x < (lt & 31u)) before += __ldcg(bound_sums(bt) + t - 1u - threadIdx.x);
+        if (threadIdx.x >= kFThreads - kFThreads / 32) {  // entries of warp k's items
+            const uint32_t k = threadIdx.x - (kFThreads - kFThreads / 32);
+            s_n[k] = i0 + kSubItems * k < N ? *walk_region(I, i0 + kSubItems * k) : 0u;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xFFFFFFFFu, before, o);
+        if (lane == 0) s_red[warp] = before;
+        __syncthreads();
+        before = 0;
+        uint32_t n = 0;
+#pragma unroll
+        for (uint32_t w = 0; w < kFThreads / 32; ++w) {
+            before += s_red[w];
+            n += s_n[w];
+        }
+        const bool none = before > F;
+        uint32_t smc = 0, ssc = 0;
+        for (uint32_t q = threadIdx.x; q < n; q += kFThreads) {
+            uint32_t w = 0, x = q;
+#pragma unroll
+            for (uint32_t k = 0; k + 1u < kFThreads / 32; ++k) {  // the warp's items that hold entry q
+                const uint32_t m = s_n[k];
+                const bool past = w == k && x >= m;
+                x -= past ? m : 0u;
+                w += past ? 1u : 0u;
+            }
+            const uint32_t e = reinterpret_cast<const uint16_t*>(walk_region(I, i0 + kSubItems * w) + 1)[x];
+            const uint32_t i = i0 + kSubItems * w + (e & 127u);
+            if (e & 128u) {
+                if (none) continue;
+                const uint32_t own = (e & 256u) ? 4u : 2u;
+                uint32_t cost = own;
+                if (before + own <= F) {
+                    const uint32_t s = I.live[i];
+                    uint4 rec;
+                    cost = chain_walk(I, s, depth_of(I.heap[s], I.ch), false, &rec);
+                    I.grp[i] = rec;
+                }
+                I.scan[i] = cost;
+                ssc += cost;
+            } else {
+                const uint32_t s = I.live[i];
+                Group g;
+                if (group_if_mergeable(I, s, I.heap[s], g)) {
+                    const uint32_t mc = gate == 1 ? 2u : (uint32_t)g.np;
+                    I.grp[i] = make_uint4(g.m[0], g.m[1], g.m[2], g.m[3]);
+                    atomicOr(cmd_ptr(I, s), kGrpMin);
+                    I.scan[i] = mc << 24;
+                    smc += mc;
+                    atomicAdd(&s_cnt[0], 1u);
+                }
+            }
+        }
+        if (smc) atomicAdd(&s_tmp[0], smc);
+        if (ssc) atomicAdd(&s_tmp[1], ssc);
+        __syncthreads();
+        if (threadIdx.x == 0 && (s_tmp[0] | s_tmp[1]))
+            atomicAdd(bt.status + (bt.B == 1 ? 0u : bt.stile_base[c.b]) + i0 / S,
+                      ((unsigned long long)s_tmp[0] << 32) | s_tmp[1]);
+        stats_flush(s_cnt, I.g, kStMergeCand);
         __syncthreads();
     }
 }
@@ -475,25 +550,6 @@ __device__ __forceinline__ void batch_list(const BatchDev& bt, FCtx& c, int stat
             if (b != kNull && sum && lane == __ffs(same) - 1) atomicAdd(&bt.inst[b].g->stats[stat], sum);
         }
     }
-}
-
-// P2: the merge groups the walks listed: a group whose members all wish to
-// merge is a candidate; its cost goes to the top byte of its smallest
-// member's scan word and to its scan tile's sum (the walks added the split
-// costs). Reading only the listed items, not every live one's slot, scan and
-// command words, took this phase of a batch of 15M bisectors from 126 to
-// 67 us.
-__device__ void phase_gate_sum(const BatchDev& bt, FCtx& c, uint32_t* s_cnt, uint32_t* s_list, Pair* s_warp) {
-    const uint32_t S = kFThreads * bt.bg->scan_ipt;
-    batch_list(bt, c, kStMergeCand, s_cnt, s_list, s_warp, [](const Inst& I) { return __ldcg(&I.g->nwalk); },
-               [&](uint32_t b, const Inst& I, uint32_t q) {
-                   const uint32_t i = I.chg[q];
-                   const uint32_t mc = merge_cost(I, i, kGrpMin, frame_of(bt, b).gate);
-                   if (mc == 0u) return 0u;
-                   I.scan[i] = mc << 24;
-                   atomicAdd(bt.status + (bt.B == 1 ? 0u : bt.stile_base[b]) + i / S, (unsigned long long)mc << 32);
-                   return 1u;
-               });
 }
 
 // The ipt consecutive words from p + i0 (those at index >= n: `none`), as
@@ -580,6 +636,9 @@ __device__ void phase_gate(const BatchDev& bt, FCtx& c, uint32_t* s_cnt, uint32_
         ctx_tile(bt, bt.stile_base, t, T, c);
         const Inst& I = kOne ? bt.inst0 : c.I;
         const uint32_t N = c.N, F = c.F;
+        // a tile without requests has nothing to grant (its sums are 0; the
+        // instance's first tile also writes the totals)
+        if (c.lt != 0u && __ldcg(bt.status + t) == 0ull) continue;  // block-uniform
         const uint32_t i0 = stile_first(c, ipt);
         uint32_t sl[kMaxIpt], w[kMaxIpt];
         load_items(I.live, i0, ipt, N, kNull, sl);  // before the tile sums, which do not need them
@@ -1217,10 +1276,10 @@ __global__ void __launch_bounds__(kFThreads, CBT_FRAME_MIN_BLOCKS) k_frame(Batch
     phase_prep(bt, s_warp, s_tmp);
     grid_sync(bt.bg, epoch, 1u);
     stamp(bt, 1);
-    phase_classify<F>(bt, s_c, s_tab, s_cnt, &s_n, reinterpret_cast<uint2*>(s_buf), s_tmp);
+    phase_classify<F>(bt, s_c, s_tab, s_cnt);
     grid_sync(bt.bg, epoch, 2u);
     stamp(bt, 2);
-    phase_gate_sum(bt, s_c, s_cnt, s_buf, s_warp);
+    phase_walks(bt, s_c, s_cnt, reinterpret_cast<unsigned long long*>(s_buf), s_tmp, s_w);
     grid_sync(bt.bg, epoch, 3u);
     stamp(bt, 3);
     phase_gate(bt, s_c, s_cnt, s_red, s_warp, s_tmp, &s_n, reinterpret_cast<uint2*>(s_buf));
@@ -1371,53 +1430,6 @@ constexpr uint32_t kWalkCap1 = kFBuf / 4;  // uint4 entries of the block's list
 // one too (its chain then costs at least 4: itself and the Twin's pair,
 // Alg. 3); else the chain can cost 2.
 constexpr uint32_t kWalkSplit = 0x80000000u, kWalkInterior = 0x40000000u, kWalkIndex = 0x3FFFFFFFu;
-
-// Alg. 4 group of s1 (heap ID j1, a merge wish) on the frame-start state,
-// walked only while s1 can be its smallest member and every member wishes
-// to merge: true when both hold, with the members (m[0] = s1, m[1] its
-// sibling, m[2] the bisector across the outer half of the refinement edge,
-// m[3] its sibling) and the parents' count.
-static __device__ bool group_if_mergeable(const Inst& I, uint32_t s1, uint64_t j1, Group& g) {
-    if (depth_of(j1, I.ch) < 1) return false;
-    const uint4 r1 = I.nb[s1];
-    const bool bit = j1 & 1ull;
-    const uint32_t s2 = bit ? r1.z : r1.y;
-    const uint32_t s3 = bit ? r1.y : r1.z;
-    if (s2 == kNull || bad_slot(I, s2, kErrLink)) return false;
-    if (s3 != kNull && bad_slot(I, s3, kErrLink)) return false;
-    const uint64_t j2 = I.heap[s2];
-    const uint32_t c2 = *cmd_ptr(I, s2);
-    uint64_t j3 = 0ull;
-    uint4 r3 = make_uint4(kNull, kNull, kNull, 0u);
-    uint32_t c3 = 0u;
-    if (s3 != kNull) {
-        j3 = I.heap[s3];
-        r3 = I.nb[s3];
-        c3 = *cmd_ptr(I, s3);
-    }
-    if ((j2 >> 1) != (j1 >> 1) || j2 < j1 || !(c2 & kMergeWish)) return false;
-    g.m[0] = s1;
-    g.m[1] = s2;
-    g.m[2] = g.m[3] = kNull;
-    g.n = 2;
-    g.np = 1;
-    g.imin = 0;
-    if (s3 != kNull) {
-        // the other pair's smaller member is its even one
-        if (bitlen64(j3) != bitlen64(j1) || (j3 >> 1) == (j1 >> 1) || (j3 & ~1ull) < j1 || !(c3 & kMergeWish))
-            return false;
-        const uint32_t s4 = bit ? r3.y : r3.z;
-        if (s4 == kNull || bad_slot(I, s4, kErrLink)) return false;
-        const uint64_t j4 = I.heap[s4];
-        const uint32_t c4 = *cmd_ptr(I, s4);
-        if ((j4 >> 1) != (j3 >> 1) || !(c4 & kMergeWish)) return false;
-        g.m[2] = s3;
-        g.m[3] = s4;
-        g.n = 4;
-        g.np = 2;
-    }
-    return true;
-}
 
 __device__ __forceinline__ uint32_t scan_ipt1(uint32_t N) {
     const uint32_t per_round = gridDim.x * kFThreads;
@@ -1734,12 +1746,7 @@ __device__ void phase_classify1(const BatchDev& bt, FCtx& c, uint32_t* s_tab, ui
         if (i < N) {
             split = (cmd & kSplitWish) != 0u;
             walk = split || ((cmd & kMergeWish) && !(cmd & kHeapOdd));
-            // every bisector under a root whose halfedge has a Twin has one
-            // (its refinement edge is inside the root triangle, on an edge
-            // to the face's centroid, or on that halfedge)
-            const int d = depth_of(ja, I.ch);
-            const uint32_t h = d >= 0 ? (uint32_t)((ja >> d) - (1ull << I.ch)) : kNull;
-            interior = split && h < I.H && !((__ldg(I.rbnd + (h >> 5)) >> (h & 31u)) & 1u);
+            interior = split && has_twin_bound(I, ja);
         }
         const unsigned wm = __ballot_sync(0xFFFFFFFFu, walk), sm = __ballot_sync(0xFFFFFFFFu, split);
         if (walk)
