@@ -82,6 +82,41 @@ __global__ void __launch_bounds__(kThreads) k_prep(BatchDev bt, int frame_start)
     for (uint32_t e = tid; e < bt.Trel; e += nth) rel_entry(bt, e);
 }
 
+// The slots and command words of a thread's items of an item tile (0 past the
+// live count), all loads out before the first is used: interleaved with the
+// lists' shared-memory atomics they went out one dependent pair at a time.
+__device__ __forceinline__ void load_tile_commands(const Inst& I, uint32_t lt, uint32_t N,
+                                                   uint32_t (&sl)[kItemsPerThread], uint32_t (&cm)[kItemsPerThread]) {
+    const uint32_t* const live = I.live;
+    const uint2* const cd = I.cd;
+#pragma unroll
+    for (int k = 0; k < kItemsPerThread; ++k) {
+        const uint32_t i = lt * kTileItems + (uint32_t)k * kThreads + threadIdx.x;
+        sl[k] = i < N ? live[i] : kNull;
+    }
+#pragma unroll
+    for (int k = 0; k < kItemsPerThread; ++k) cm[k] = sl[k] != kNull ? cd[sl[k]].x : 0u;
+}
+
+// The same for the consecutive items a thread holds of a scan tile, with their
+// slots in two 16-byte loads (base is a multiple of kScanPerThread).
+__device__ __forceinline__ void load_scan_commands(const Inst& I, uint32_t base, uint32_t N,
+                                                   uint32_t (&sl)[kScanPerThread], uint32_t (&cm)[kScanPerThread]) {
+    static_assert(kScanPerThread % 4 == 0, "16-byte loads");
+    const uint2* const cd = I.cd;
+#pragma unroll
+    for (int k = 0; k < kScanPerThread; k += 4) {
+        uint4 v = make_uint4(kNull, kNull, kNull, kNull);
+        if (base + k < N) v = *reinterpret_cast<const uint4*>(I.live + base + k);
+        sl[k] = v.x;
+        sl[k + 1] = base + k + 1 < N ? v.y : kNull;
+        sl[k + 2] = base + k + 2 < N ? v.z : kNull;
+        sl[k + 3] = base + k + 3 < N ? v.w : kNull;
+    }
+#pragma unroll
+    for (int k = 0; k < kScanPerThread; ++k) cm[k] = sl[k] != kNull ? cd[sl[k]].x : 0u;
+}
+
 __global__ void __launch_bounds__(kThreads) k_walk(BatchDev bt) {
     __shared__ uint32_t s_b, s_n;
     __shared__ Inst s_I;
@@ -95,15 +130,14 @@ __global__ void __launch_bounds__(kThreads) k_walk(BatchDev bt) {
         const FrameP& fp = frame_of(bt, b);
         const bool chain = fp.gate != 1;
         const uint32_t N = I.g->N;
+        uint32_t sl[kItemsPerThread], cm[kItemsPerThread];
+        load_tile_commands(I, lt, N, sl, cm);
 #pragma unroll
         for (int k = 0; k < kItemsPerThread; ++k) {
             const uint32_t i = lt * kTileItems + (uint32_t)k * kThreads + threadIdx.x;
-            if (i >= N) continue;
-            const uint32_t s = I.live[i];
-            const uint32_t cmd = *cmd_ptr(I, s);
-            const bool split = (cmd & kSplitWish) != 0u;
-            const bool need = (split && chain) || ((cmd & kMergeWish) && !(cmd & kHeapOdd));
-            if (need) s_list[atomicAdd(&s_n, 1u)] = make_uint2(i | (split ? 0x80000000u : 0u), s);
+            const bool split = (cm[k] & kSplitWish) != 0u;
+            const bool need = (split && chain) || ((cm[k] & kMergeWish) && !(cm[k] & kHeapOdd));
+            if (need) s_list[atomicAdd(&s_n, 1u)] = make_uint2(i | (split ? 0x80000000u : 0u), sl[k]);
         }
         __syncthreads();
         const uint32_t n = s_n;
@@ -184,30 +218,49 @@ __global__ void __launch_bounds__(kScanThreads) k_gate(BatchDev bt) {
     __shared__ Pair s_excl;
     __shared__ Inst s_I;
     __shared__ uint32_t s_cnt[kBlockStats];
+    __shared__ uint32_t s_n;
+    __shared__ uint16_t s_list[kScanItems];
+    __shared__ uint8_t s_val[kScanItems];
     const uint32_t T = ld_volatile(&bt.bg->total_stiles);
     unsigned long long* status = bt.status;
     for (;;) {
         const uint32_t t = next_ticket(bt.bg, 0, &s_tile);
         if (t >= T) break;
         uint32_t b, lt;
-        if (threadIdx.x == 0) s_mg = 0;
+        if (threadIdx.x == 0) s_mg = s_n = 0;
         tile_begin(bt, bt.stile_base, t, &s_b, &s_I, nullptr, s_cnt, b, lt);
         const Inst& I = s_I;
         const uint32_t gate = frame_of(bt, b).gate;
         const uint32_t N = I.g->N, F = I.g->F;
         const uint32_t base = lt * kScanItems + threadIdx.x * kScanPerThread;
+        uint32_t sl[kScanPerThread], cm[kScanPerThread];
+        load_scan_commands(I, base, N, sl, cm);
+        uint32_t sc[kScanPerThread];
+#pragma unroll
+        for (int k = 0; k < kScanPerThread; k += 4) {
+            uint4 x = make_uint4(0u, 0u, 0u, 0u);
+            if (base + k < N) x = *reinterpret_cast<const uint4*>(I.scan + base + k);
+            sc[k] = x.x, sc[k + 1] = x.y, sc[k + 2] = x.z, sc[k + 3] = x.w;
+        }
+        // the groups' checks (group record, then the members' command words)
+        // from a list, spread over the block
+        const uint32_t e0 = threadIdx.x * kScanPerThread;
+#pragma unroll
+        for (int k = 0; k < kScanPerThread; ++k)
+            if (cm[k] & kGrpMin) s_list[atomicAdd(&s_n, 1u)] = (uint16_t)(e0 + k);
+        __syncthreads();
+        const uint32_t ng = s_n;
+        for (uint32_t q = threadIdx.x; q < ng; q += kScanThreads) {
+            const uint32_t e = s_list[q];
+            s_val[e] = (uint8_t)merge_cost(I, lt * kScanItems + e, kGrpMin, gate);
+        }
+        __syncthreads();
         Pair v[kScanPerThread];
         Pair loc{0, 0};
 #pragma unroll
         for (int k = 0; k < kScanPerThread; ++k) {
-            const uint32_t i = base + k;
-            v[k] = Pair{0, 0};
-            if (i < N) {
-                const uint32_t s = I.live[i];
-                const uint32_t cmd = *cmd_ptr(I, s);
-                v[k] = Pair{merge_cost(I, i, cmd, gate), I.scan[i]};
-                loc = padd(loc, v[k]);
-            }
+            v[k] = Pair{(cm[k] & kGrpMin) ? s_val[e0 + k] : 0u, sl[k] != kNull ? sc[k] : 0u};
+            loc = padd(loc, v[k]);
         }
         Pair tot;
         const Pair tex = block_scan(loc, tot, s_warp);
@@ -220,7 +273,7 @@ __global__ void __launch_bounds__(kScanThreads) k_gate(BatchDev bt) {
             if (i >= N) continue;
             const bool cand = v[k].a > 0;
             const bool granted = cand && run.a <= F;
-            if (cand) atomicOr(cmd_ptr(I, I.live[i]), granted ? (kCand | kMergeGrant) : kCand);
+            if (cand) atomicOr(cmd_ptr(I, sl[k]), granted ? (kCand | kMergeGrant) : kCand);
             if (granted) atomicMax(&s_mg, run.a);
             I.scan[i] = run.b;
             count_stat(s_cnt, 0, cand);
@@ -250,17 +303,15 @@ __global__ void __launch_bounds__(kThreads) k_scatter(BatchDev bt) {
         const Inst& I = s_I;
         const uint32_t N = I.g->N;
         const uint64_t F = I.g->F, Mg = ld_volatile(&I.g->Mg);
+        uint32_t sl[kItemsPerThread], cm[kItemsPerThread], run[kItemsPerThread];
+        load_tile_commands(I, lt, N, sl, cm);
+#pragma unroll
+        for (int k = 0; k < kItemsPerThread; ++k)
+            run[k] = (cm[k] & kSplitWish) ? I.scan[lt * kTileItems + (uint32_t)k * kThreads + threadIdx.x] : 0u;
 #pragma unroll
         for (int k = 0; k < kItemsPerThread; ++k) {
-            const uint32_t i = lt * kTileItems + (uint32_t)k * kThreads + threadIdx.x;
-            bool granted = false;
-            if (i < N) {
-                const uint32_t s = I.live[i];
-                if (*cmd_ptr(I, s) & kSplitWish) {
-                    granted = Mg + (uint64_t)I.scan[i] <= F;
-                    if (granted) s_list[atomicAdd(&s_n, 1u)] = s;
-                }
-            }
+            const bool granted = (cm[k] & kSplitWish) && Mg + (uint64_t)run[k] <= F;
+            if (granted) s_list[atomicAdd(&s_n, 1u)] = sl[k];
             count_stat(s_cnt, 0, granted);
         }
         __syncthreads();
@@ -283,25 +334,45 @@ __global__ void __launch_bounds__(kScanThreads) k_alloc(BatchDev bt) {
     __shared__ Pair s_excl;
     __shared__ Inst s_I;
     __shared__ uint32_t s_cnt[kBlockStats];
+    __shared__ uint32_t s_n;
+    __shared__ uint16_t s_list[kScanItems];
+    __shared__ uint8_t s_val[kScanItems];
     const uint32_t T = ld_volatile(&bt.bg->total_stiles);
     unsigned long long* status = bt.status + bt.Titems;
     for (;;) {
         const uint32_t t = next_ticket(bt.bg, 1, &s_tile);
         if (t >= T) break;
         uint32_t b, lt;
+        if (threadIdx.x == 0) s_n = 0;
         tile_begin(bt, bt.stile_base, t, &s_b, &s_I, nullptr, s_cnt, b, lt);
         const Inst& I = s_I;
         const uint32_t N = I.g->N;
         const uint32_t base = lt * kScanItems + threadIdx.x * kScanPerThread;
         // fate per item, 4 bits each: allocation count (0-4) and whether the
         // item is a merge at its smallest member
+        uint32_t sl[kScanPerThread], cm[kScanPerThread];
+        load_scan_commands(I, base, N, sl, cm);
+        // granted merges are validated from a list, spread over the block
+        const uint32_t e0 = threadIdx.x * kScanPerThread;
+        uint32_t lst = 0;
+#pragma unroll
+        for (int k = 0; k < kScanPerThread; ++k)
+            if (!(cm[k] & kSplitMask) && (cm[k] & kCand) && (cm[k] & kMergeGrant)) {
+                lst |= 1u << k;
+                s_list[atomicAdd(&s_n, 1u)] = (uint16_t)(e0 + k);
+            }
+        __syncthreads();
+        const uint32_t nm = s_n;
+        for (uint32_t q = threadIdx.x; q < nm; q += kScanThreads) {
+            const uint32_t e = s_list[q];
+            s_val[e] = (uint8_t)alloc_fate(I, lt * kScanItems + e, kCand | kMergeGrant);
+        }
+        __syncthreads();
         uint32_t packed = 0;
         Pair loc{0, 0};
 #pragma unroll
         for (int k = 0; k < kScanPerThread; ++k) {
-            const uint32_t i = base + k;
-            if (i >= N) continue;
-            const uint32_t f = alloc_fate(I, i, *cmd_ptr(I, I.live[i]));
+            const uint32_t f = ((lst >> k) & 1u) ? s_val[e0 + k] : leaves_of(cm[k] & kSplitMask);
             const uint32_t na = f & 7u;
             packed |= f << (4 * k);
             loc = padd(loc, Pair{na ? 1u : 0u, na});
