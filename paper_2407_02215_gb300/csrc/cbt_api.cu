@@ -31,8 +31,8 @@ constexpr uint32_t kLaunchesPerStep[kNumKernels] = {1, 1, 1, 1, 1, 1, 1, 1, 2, 1
 const char* const kPhaseNames[kFramePhases] = {"prep", "classify", "gate_sum", "gate",    "alloc",
                                                "fill", "reduce",   "compact", "vertices"};
 // phases of the single-instance frame (k_frame1)
-const char* const kPhaseNames1[kFrame1Phases] = {"prep",  "classify", "walks", "gate",
-                                                 "alloc", "fill",     "final", "vertices"};
+const char* const kPhaseNames1[kFrame1Phases] = {"prep",  "classify", "walks",   "gate",
+                                                 "alloc", "fill",     "vertices"};
 constexpr uint32_t kFusedTileWords = 64;
 constexpr uint32_t kFusedMaxTileWords = 128;
 
@@ -49,8 +49,8 @@ uint32_t item_tiles(uint32_t cap) { return (cap + kTileItems - 1u) / kTileItems;
 
 // Per-instance arrays.
 struct Layout {
-    size_t globals, heap, nb, cd, bits, sums, live, freel, scan, grp, chg, chgr, vc, root64, rel, corner, rbnd, batch,
-        total;
+    size_t globals, heap, nb, cd, bits, sums, live, freel, scan, grp, chg, chgr, vc, root64, rel, corner, rbnd, freel2,
+        clr, batch, total;
     uint32_t cap, W, ch;
 };
 
@@ -118,6 +118,8 @@ bool make_layout(int32_t H, int32_t D, Layout& L) {
     L.rel = take(72u * h);
     L.corner = take(12u * h);
     L.rbnd = take(4u * ((h + 31u) / 32u));
+    L.freel2 = take(4u * cap);
+    L.clr = take(4u * L.W);
     const uint32_t Hh = static_cast<uint32_t>(H);
     const BatchLayout B = batch_layout(1, &L.cap, &L.W, &Hh);
     L.batch = take(B.total);
@@ -612,6 +614,8 @@ extern "C" int cbt_create(int32_t H, const int32_t* twin, const int32_t* next, c
     I.sums = reinterpret_cast<uint32_t*>(b + L.sums);
     I.live = reinterpret_cast<uint32_t*>(b + L.live);
     I.freel = reinterpret_cast<uint32_t*>(b + L.freel);
+    I.freel2 = reinterpret_cast<uint32_t*>(b + L.freel2);
+    I.clr = reinterpret_cast<uint32_t*>(b + L.clr);
     I.scan = reinterpret_cast<uint32_t*>(b + L.scan);
     I.grp = reinterpret_cast<uint4*>(b + L.grp);
     I.chg = reinterpret_cast<uint32_t*>(b + L.chg);
@@ -652,6 +656,7 @@ extern "C" int cbt_create(int32_t H, const int32_t* twin, const int32_t* next, c
     double* d_hpos = reinterpret_cast<double*>(b + L.rel + align256(12u * h));
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     cudaMemsetAsync(I.g, 0, sizeof(Globals), s);
+    cudaMemsetAsync(I.clr, 0, 4u * L.W, s);
     cudaMemcpyAsync(d_ints, ints.data(), 12u * h, cudaMemcpyHostToDevice, s);
     cudaMemcpyAsync(d_hpos, hpos.data(), 24u * h, cudaMemcpyHostToDevice, s);
     cudaMemcpyAsync(st->corner, corner.data(), 12u * h, cudaMemcpyHostToDevice, s);

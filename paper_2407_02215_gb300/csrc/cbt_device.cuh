@@ -12,6 +12,9 @@
 //                    root, sums[W + w] = popc(bits[w]) (Sec. 3.1)
 //   live[cap]  u32   slots of the live bisectors, ascending (Alg. 7 for all i)
 //   freel[cap] u32   the first A zero bits of the frame-start bitfield (Alg. 8)
+//   freel2[cap] u32  single-instance frame: the other free list (this frame's and
+//                    the next one's change places every frame)
+//   clr[W]     u32   single-instance frame: bits cleared this frame; 0 between frames
 //   scan[cap]  u32   per live index: split cost, then its running total
 //   grp[cap]   uint4 per live index: the members of the merge group whose
 //                    smallest member it is, or of a split wish's chain
@@ -100,8 +103,9 @@ struct Globals {
     uint32_t nwalk;  // single-instance frame: entries of the frame's walk list
     uint32_t marks_clean;  // 1 when the chain-mark words (chg) of the live slots are 0 (the
                            // single-instance frame leaves them so; the other frames clear this)
-    uint32_t freel_full;   // 1 when freel lists every zero bit of the bitfield in slot order
-                           // (the single-instance frame leaves it so; the other frames clear this)
+    uint32_t freel_full;   // bit 0: a free list of every zero bit of the bitfield in slot order is kept, in
+                           // freel or (bit 1) freel2, and the word tiles' prefix in the same one of its two
+                           // buffers (the single-instance frame leaves it so; the other frames clear this)
     uint32_t pad[64 - 39];
 };
 static_assert(sizeof(Globals) == 256, "Globals must be 256 bytes");
@@ -129,6 +133,8 @@ struct Inst {
     uint32_t cap, W, D, H, ch, max_depth;
     uint32_t ntiles_items;  // ceil(cap / kTileItems)
     uint32_t pad_;
+    uint32_t* freel2;       // single-instance frame: the other free list
+    uint32_t* clr;          // single-instance frame: the frame's cleared bits, 0 between frames
     const uint32_t* rbnd;   // bit h: halfedge h has no Twin (mesh boundary), [ceil(H / 32)]
 };
 
@@ -215,7 +221,7 @@ struct BatchDev {
                                  // host memory, and nothing else is written when it exceeds vcap
     uint32_t timing;             // one-launch frame: record phase boundaries
     uint32_t* tpre;              // single-instance frame: [2][Twords] ones before each word tile of
-                                 // the next frame's starting bitfield, by frame parity
+                                 // the next frame's starting bitfield (which: the instance's freel_full)
 };
 
 constexpr int kThreads = 256;

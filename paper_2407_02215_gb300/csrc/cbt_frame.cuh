@@ -720,7 +720,7 @@ __device__ void phase_gate(const BatchDev& bt, FCtx& c, uint32_t* s_cnt, uint32_
 }
 
 __device__ void free_list(const BatchDev& bt, FCtx& c, uint32_t* s_w, bool all_granted,
-                          const unsigned long long* tcounts = nullptr);
+                          const unsigned long long* tcounts = nullptr, uint32_t* list = nullptr);
 
 // Exclusive prefix of one word per thread over the block, without saturation
 // (sums over a whole batch may wrap; differences of prefixes are taken).
@@ -892,6 +892,7 @@ struct DestBatch {
     __device__ __forceinline__ uint32_t operator()(uint32_t d) const {
         return (uint32_t)pre[min(d >> kLocBits, last)] - base + (d & kLocMask);
     }
+    __device__ __forceinline__ const uint32_t* freel(const Inst& I) const { return I.freel; }
     __device__ __forceinline__ void set(const Inst& I, uint32_t s) const { set_bit(I, s); }
     __device__ __forceinline__ void clear(const Inst& I, uint32_t s) const { clear_bit(I, s); }
 };
@@ -904,8 +905,9 @@ struct DestBatch {
 // With `tcounts` (single instance, word tiles of the frame's tile counts)
 // the ones before a word tile are summed over the block from those counts
 // instead of read down the sum tree one level at a time.
+// `list`: where it goes (the instance's first free list by default).
 __device__ void free_list(const BatchDev& bt, FCtx& c, uint32_t* s_w, bool all_granted,
-                          const unsigned long long* tcounts) {
+                          const unsigned long long* tcounts, uint32_t* list) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     for (uint32_t wt = blockIdx.x; wt < bt.Twords; wt += gridDim.x) {
         ctx_tile(bt, bt.wtile_base, wt, bt.Twords, c);
@@ -960,7 +962,7 @@ __device__ void free_list(const BatchDev& bt, FCtx& c, uint32_t* s_w, bool all_g
             }
             __syncthreads();
             uint64_t r = zeros_before + s_w[warp] + (inc - mine);
-            uint32_t* const freel = I.freel;  // in a register across the stores
+            uint32_t* const freel = list ? list : I.freel;  // in a register across the stores
             while (z && r < bound) {
                 freel[r] = w * 32u + (uint32_t)(__ffs(z) - 1);
                 ++r;
@@ -1324,7 +1326,7 @@ __global__ void __launch_bounds__(kFThreads) k_wait_selftest(BatchGlobals* bg, i
 // ===================================================== one instance, fewer phases
 //
 // k_frame1: the frame of a single instance (a batch of one), with the same
-// results as k_frame in seven phases, or six when the frame's requests all
+// results as k_frame in six phases, or five when the frame's requests all
 // fit the free slots or nothing is exported:
 //   P0 prep      frame counters; the camera-relative roots; the word-tile
 //                counts copied; the chain-mark words of the live slots and
@@ -1352,14 +1354,14 @@ __global__ void __launch_bounds__(kFThreads) k_wait_selftest(BatchGlobals* bg, i
 //                word holds the tile and the offset within it), the fill
 //                records per tile, the bits cleared per word tile; the free
 //                list only when the last frame was not this kernel
-//   P5 fill      the tiles' record and allocation offsets in shared memory;
-//                new records, links and bits
-//   P6 final     every word tile's new count (frame-start count, clears, and
-//                its share of the first A zero bits), hence the sum tree;
-//                per 16-word part of a word tile (one warp), its rows of the
-//                new live list and, from its zero bits, of the next frame's
-//                free list (every zero bit in slot order)
-//   P7 vertices  the export of the new list (FP32, fixed point, FP64
+//   P5 fill      on half of the blocks the tiles' record and allocation
+//                offsets in shared memory, new records and links; on the
+//                others every word tile's new count (frame-start count,
+//                clears, and its share of the first A zero bits), hence the
+//                sum tree, and per word tile (one warp) its new words, its
+//                rows of the new live list and, from its zero bits, of the
+//                next frame's free list (every zero bit in slot order)
+//   P6 vertices  the export of the new list (FP32, fixed point, FP64
 //                evaluated; sphere and displaced forms copied from the cache
 //                of P1), 32 rows per warp, warp-major
 // The instance descriptor and the frame parameters are read from the launch
@@ -1399,13 +1401,30 @@ __device__ __forceinline__ Pair block_table(uint32_t n, Load load, Store store, 
 // tiles' allocation offsets in shared memory.
 struct DestTiles {
     const uint32_t* apre;
+    const uint32_t* list;  // the frame's free list
     uint32_t A;
     __device__ __forceinline__ uint32_t operator()(uint32_t d) const {
         return apre[min(d >> kLocBits, kMaxTiles1 - 1u)] + (d & kLocMask);
     }
-    __device__ __forceinline__ void set(const Inst& I, uint32_t s) const { set_bit(I, s); }
-    __device__ __forceinline__ void clear(const Inst& I, uint32_t s) const { clear_bit(I, s); }
+    __device__ __forceinline__ const uint32_t* freel(const Inst&) const { return list; }
+    // the bitfield is rewritten from its frame-start words and the clear masks
+    __device__ __forceinline__ void set(const Inst&, uint32_t) const {}
+    __device__ __forceinline__ void clear(const Inst&, uint32_t) const {}
 };
+
+// What the last frame left, read from its flag word (freel_full) at the start:
+// bit 0 that it was this kernel, bit 1 in which of their two buffers the free
+// list and the ones before each word tile then are (0 without bit 0). The fill
+// reads the one buffer while the next frame's is written beside it.
+struct Carry {
+    uint32_t w;
+    __device__ __forceinline__ bool ok() const { return (w & 1u) != 0u; }
+    __device__ __forceinline__ uint32_t buffer() const { return (w & 1u) ? (w >> 1) & 1u : 0u; }
+};
+// The free list of the current frame (ahead = 0) or the next one (ahead = 1).
+__device__ __forceinline__ uint32_t* free_list1(const BatchDev& bt, Carry carry, uint32_t ahead) {
+    return (carry.buffer() ^ ahead) ? bt.inst0.freel2 : bt.inst0.freel;
+}
 
 // Word-tile counts of the single-instance frame, one 64-bit word per word
 // tile (2^tbits slots, its sum-tree node at nt + t): the node's frame-start
@@ -1941,6 +1960,14 @@ __device__ __forceinline__ uint32_t fate_group_granted(const Inst& I, uint32_t i
     return ok ? ((m.z == kNull ? 1u : 2u) | 8u) : 0u;
 }
 
+// The most this frame can allocate: the free slots, or the requests granted.
+__device__ __forceinline__ uint32_t alloc_bound1(const BatchDev& bt, const FCtx& c, bool all_granted) {
+    const Globals* g = bt.inst0.g;
+    const uint64_t req = all_granted ? __ldcg(&g->rq_merge) + __ldcg(&g->rq_split)
+                                     : (uint64_t)__ldcg(&g->Mg) + (uint64_t)__ldcg(&g->Stot);
+    return (uint32_t)min((uint64_t)c.F, req);
+}
+
 // P4 (single instance): per scan tile the fate of every item (allocation
 // count, bit 3 for a merging group), the tile-local exclusive prefix of
 // (changed, allocations), the fill records in the tile's region of chgr
@@ -1949,7 +1976,7 @@ __device__ __forceinline__ uint32_t fate_group_granted(const Inst& I, uint32_t i
 // request was granted, the chain marks are ORed into the command words (the
 // fill reads them there). Then the free list. Group validations run from a
 // list (dependent loads), their fates returned through shared memory.
-__device__ void phase_alloc1(const BatchDev& bt, FCtx& c, bool all_granted, bool carried, uint32_t tbits,
+__device__ void phase_alloc1(const BatchDev& bt, FCtx& c, bool all_granted, Carry carry, uint32_t tbits,
                              uint32_t* s_cnt, Pair* s_warp, uint32_t* s_w, uint32_t* s_n, uint32_t* s_buf) {
     const uint32_t T = bt.bg->total_stiles, ipt = bt.bg->scan_ipt;
     const uint32_t S = kFThreads * ipt;
@@ -2049,7 +2076,10 @@ __device__ void phase_alloc1(const BatchDev& bt, FCtx& c, bool all_granted, bool
         s_hist[threadIdx.x] = 0u;
         if (threadIdx.x == 0) *s_n = 0;
         __syncthreads();
+        uint32_t* const clr = I.clr;
         auto cleared = [&](uint32_t slot) {
+            if (slot >= I.cap) return;  // never: the callers have checked it
+            atomicOr(clr + (slot >> 5), 1u << (slot & 31u));
             const uint32_t node = (I.cap + slot) >> tbits;
             if (node - hbase < (uint32_t)kFThreads)
                 atomicAdd(&s_hist[node - hbase], 1u);
@@ -2099,17 +2129,21 @@ __device__ void phase_alloc1(const BatchDev& bt, FCtx& c, bool all_granted, bool
     }
     // the last frame's final phase listed every zero bit of this frame's
     // starting bitfield, unless another form of the frame ran since
-    if (!carried) free_list(bt, c, s_w, all_granted, tile_counts(bt));
+    if (!carry.ok()) free_list(bt, c, s_w, all_granted, tile_counts(bt), free_list1(bt, carry, 0u));
 }
 
-// P5 (single instance): every block scans the tiles' (changed, allocation)
-// totals into shared memory; the changed records of the frame, one range
-// strided evenly over the grid, are then filled with their destinations
-// resolved through the allocation offsets. The records are FillNewBlocks +
-// UpdateNeighbors + UpdateBitfield, the bit changes also moving the word
-// tiles' sum-tree nodes.
-__device__ void phase_fill1(const BatchDev& bt, FCtx& c, bool all_granted, uint32_t* s_cnt, uint32_t* s_buf,
-                            Pair* s_warp) {
+// P5 (single instance) has two parts that share nothing they write, each on
+// half of the blocks, so that the one's dependent loads overlap the other's
+// (one after the other, with a barrier between, they took 15.4 and 9.9 us of
+// the 124 us grid frame; together 18.8 us).
+//
+// The fill: every block scans the tiles' (changed, allocation) totals into
+// shared memory; the changed records of the frame, one range strided evenly
+// over the part's blocks, are then filled with their destinations resolved
+// through the allocation offsets: FillNewBlocks + UpdateNeighbors. (`fb` of
+// `nfb`: the block's place in the part.)
+__device__ void phase_fill1(const BatchDev& bt, FCtx& c, bool all_granted, Carry carry, uint32_t fb, uint32_t nfb, uint32_t* s_cnt,
+                            uint32_t* s_buf, Pair* s_warp) {
     stats_reset(s_cnt);
     ctx_tile(bt, bt.tile_base, 0, 1, c);
     const Inst& I = bt.inst0;
@@ -2120,29 +2154,26 @@ __device__ void phase_fill1(const BatchDev& bt, FCtx& c, bool all_granted, uint3
         __syncthreads();
         return;
     }
-    const Pair carry = block_table(
+    const Pair all = block_table(
         T, [&](uint32_t t) { return unpack_pair(__ldcg(bt.status + bt.Titems + t)); },
         [&](uint32_t t, Pair ex) {
             s_cpre[t] = ex.a;
             s_apre[t] = ex.b;
         },
         s_warp);
-    const uint32_t C = carry.a;
-    const uint64_t req = all_granted ? __ldcg(&I.g->rq_merge) + __ldcg(&I.g->rq_split)
-                                     : (uint64_t)I.g->Mg + (uint64_t)I.g->Stot;
-    const uint32_t bound = (uint32_t)min((uint64_t)c.F, req);
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        I.g->A = carry.b;
+    const uint32_t C = all.a;
+    const uint32_t bound = alloc_bound1(bt, c, all_granted);
+    if (fb == 0 && threadIdx.x == 0) {
+        I.g->A = all.b;
         I.g->C = C;
-        I.g->stats[kStAllocated] = carry.b;
-        if (carry.b > bound) set_err(I.g, kErrOverflow);
+        I.g->stats[kStAllocated] = all.b;
+        if (all.b > bound) set_err(I.g, kErrOverflow);
     }
-    const DestTiles dm{s_apre, min(carry.b, bound)};
+    const DestTiles dm{s_apre, free_list1(bt, carry, 0u), min(all.b, bound)};
     uint32_t relinked = 0;
-    // 32 records per warp, warp-major over the grid: with fewer records than
+    // 32 records per warp, warp-major over the blocks: with fewer records than
     // threads, every SM still gets its share
-    for (uint32_t q = ((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32u + (threadIdx.x & 31u); q < C;
-         q += gridDim.x * kFThreads) {
+    for (uint32_t q = ((threadIdx.x >> 5) * nfb + fb) * 32u + (threadIdx.x & 31u); q < C; q += nfb * kFThreads) {
         uint32_t lo = 0, hi = T;  // the last tile whose first record is at or before q
         while (lo < hi) {
             const uint32_t mid = (lo + hi) >> 1;
@@ -2161,55 +2192,70 @@ __device__ void phase_fill1(const BatchDev& bt, FCtx& c, bool all_granted, uint3
     __syncthreads();
 }
 
-// P6 (single instance). Every block computes each word tile's new count
-// from the tile counts of the frame (no bitfield read) and scans them into
-// shared memory: the new live count and each tile's first row. Block 0
-// writes the nodes above the tiles as differences of that scan; a warp per
-// word tile rebuilds the tile's node and the nodes below it from its words
-// (the count checked against the scan) and writes the tile's rows of the new
-// live list. The vertices follow in their own phase, over the whole list.
-__device__ void phase_final1(const BatchDev& bt, FCtx& c, uint32_t* s_buf, Pair* s_warp, uint32_t* s_tmp,
-                             uint32_t tbits, bool carried) {
+// The lowest k of the set bits of z.
+__device__ __forceinline__ uint32_t lowest_set(uint32_t z, int k) {
+    if (k <= 0) return 0u;
+    if (k >= __popc(z)) return z;
+    uint32_t t = z;
+    for (; k > 0; --k) t &= t - 1u;
+    return z ^ t;
+}
+
+// The final part: UpdateBitfield, SumReduction and CachePointers, from what
+// the allocation left: the frame-start bitfield, the bits cleared (clr) and
+// the count A of new records, which take the first A zero bits (Alg. 8).
+// Every block of it computes each word tile's new count and scans them into
+// shared memory: the new live count and each tile's first row. The first
+// block writes the sum tree's nodes above the tiles as differences of that
+// scan; a warp per word tile rewrites the tile's words, the nodes from the
+// tile down (the count checked against the scan), and the tile's rows of the
+// new live list and, from the zero bits, of the next frame's free list.
+__device__ void phase_final1(const BatchDev& bt, FCtx& c, bool all_granted, uint32_t rb, uint32_t nrb, uint32_t* s_buf,
+                             Pair* s_warp, uint32_t* s_red, uint32_t tbits, Carry carry) {
     ctx_tile(bt, bt.tile_base, 0, 1, c);
     const Inst& I = bt.inst0;
     const uint32_t W = I.W, TW = min(W, bt.tw), nt = I.cap >> tbits;
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    uint32_t* s_tpre = s_buf;
+    uint32_t* s_tpre = s_buf;               // ones before each tile in the new bitfield
+    uint32_t* s_old = s_buf + kMaxTiles1;   // and in the frame-start one
     if (nt > kMaxTiles1 || TW > 64u) {  // the host keeps pools within the tables
-        if (blockIdx.x == 0 && threadIdx.x == 0) set_err(I.g, kErrOverflow);
+        if (rb == 0 && threadIdx.x == 0) set_err(I.g, kErrOverflow);
         return;
     }
-    // each word tile's new count: frame-start count - cleared + set, the set
-    // ones being the tile's share of the first A zero bits
-    const unsigned long long* tc = tile_counts(bt);
-    const uint32_t A = __ldcg(&I.g->A), TS = 1u << tbits;
+    const uint32_t T = min(bt.bg->total_stiles, kMaxTiles1);
+    Pair sum{0, 0}, none{0, 0};
+    for (uint32_t t = threadIdx.x; t < T; t += kFThreads)
+        sum.b += unpack_pair(__ldcg(bt.status + bt.Titems + t)).b;
+    block_sum2(sum, none, s_red);
+    const uint32_t A = min(sum.b, alloc_bound1(bt, c, all_granted)), TS = 1u << tbits;
     // the ones before each tile at frame start: kept by the last frame's
-    // final phase (`carried`: the last frame was this kernel) in the buffer of
-    // this frame's parity, else scanned here from the tile counts (into
-    // s_tpre); then the new counts from them, scanned in place, and kept for
-    // the next frame in the other buffer
-    const uint32_t par = bt.fp0.frame & 1u;
-    const uint32_t* tpre_in = bt.tpre + par * bt.Twords;
-    uint32_t* tpre_out = bt.tpre + (par ^ 1u) * bt.Twords;
-    if (!carried)
+    // final part when that was this kernel, else scanned here from the tile
+    // counts; then the new counts from them, scanned, and kept for the next
+    // frame in the other buffer
+    const unsigned long long* tc = tile_counts(bt);
+    const uint32_t cur = carry.buffer();
+    const uint32_t* tpre_in = bt.tpre + cur * bt.Twords;
+    uint32_t* tpre_out = bt.tpre + (cur ^ 1u) * bt.Twords;
+    if (carry.ok()) {
+        for (uint32_t t = threadIdx.x; t < nt; t += kFThreads) s_old[t] = __ldcg(tpre_in + t);
+        __syncthreads();
+    } else {
         block_table(nt, [&](uint32_t t) { return Pair{(uint32_t)(__ldcg(tc + t) >> 32), 0u}; },
-                    [&](uint32_t t, Pair ex) { s_tpre[t] = ex.a; }, s_warp);
+                    [&](uint32_t t, Pair ex) { s_old[t] = ex.a; }, s_warp);
+    }
     const Pair tot = block_table(
         nt,
         [&](uint32_t t) {
             const unsigned long long w = __ldcg(tc + t);
             const uint32_t old = (uint32_t)(w >> 32), clr = (uint32_t)w;
-            const uint32_t before = carried ? __ldcg(tpre_in + t) : s_tpre[t];
-            const long long zb = (long long)t * TS - before;  // zero bits before the tile at frame start
+            const long long zb = (long long)t * TS - s_old[t];  // zero bits before the tile at frame start
             const long long set = min(max((long long)A - zb, 0ll), (long long)(TS - old));
             return Pair{old - clr + (uint32_t)set, 0u};
         },
         [&](uint32_t t, Pair ex) { s_tpre[t] = ex.a; }, s_warp);
-    for (uint32_t t = blockIdx.x + threadIdx.x * gridDim.x; t < nt; t += kFThreads * gridDim.x) tpre_out[t] = s_tpre[t];
-    if (threadIdx.x == 0) s_tmp[0] = 0;
-    __syncthreads();
+    for (uint32_t t = rb + threadIdx.x * nrb; t < nt; t += kFThreads * nrb) tpre_out[t] = s_tpre[t];
     const uint32_t Nn = tot.a;
-    if (blockIdx.x == 0) {
+    if (rb == 0) {
         // node m (1 <= m < nt) covers tile nodes [m 2^k, (m + 1) 2^k) at 2^k
         // tiles per node of its level
         const int lnt = 31 - __clz((int)nt);
@@ -2221,69 +2267,76 @@ __device__ void phase_final1(const BatchDev& bt, FCtx& c, uint32_t* s_buf, Pair*
         if (threadIdx.x == 0) {
             I.g->stats[kStLiveAfter] = Nn;
             if (nt == 1u) I.sums[1] = Nn;
+            I.g->marks_clean = 1u;  // read by the next frame
+            I.g->freel_full = 1u | ((cur ^ 1u) << 1);
         }
     }
-    // word tiles (TW <= 64 words: lane holds words lane and 32 + lane): the
-    // levels below the tile node (whose value, from the scan, is checked
-    // against the words' popcounts), then the tile's slice of the new live
-    // list (Alg. 7 for every index, in slot order): word by word, lane b
-    // tests bit b and the set ones take consecutive rows, so every store of
-    // the list is one contiguous run
-    // the instance's fields in registers (a store through a generic pointer
-    // would otherwise make the compiler reload them from shared memory)
+    // the instance's fields in registers
     uint32_t* const marks = chain_marks(I);
     uint32_t* const live = I.live;
-    uint32_t* const freel = I.freel;
+    uint32_t* const freel = free_list1(bt, carry, 1u);
     uint32_t* const sums = I.sums;
-    const uint32_t* const bits = I.bits;
+    uint32_t* const bits = I.bits;
+    uint32_t* const clr = I.clr;
     const uint32_t cap = I.cap;
     const uint32_t vmask = cap < 32u ? (1u << cap) - 1u : 0xFFFFFFFFu;  // the slots of a word
-    if (blockIdx.x == 0 && threadIdx.x == 0) {  // read by the next frame
-        I.g->marks_clean = 1u;
-        I.g->freel_full = 1u;
-    }
-    const uint32_t nwarps = gridDim.x * (kFThreads / 32u);
+    const uint32_t nwarps = nrb * (kFThreads / 32u);
     const uint32_t lt_mask = (1u << lane) - 1u;
-    // a word tile in Q parts of UW words, one warp each (warp-major over the
-    // grid); every part reads the tile's words for its prefix, the first
-    // also rebuilds the tile's levels of the sum tree
-    const uint32_t Q = TW >= 64u ? 4u : TW >= 32u ? 2u : 1u, UW = TW / Q;
-    for (uint32_t u = warp * gridDim.x + blockIdx.x; u < nt * Q; u += nwarps) {
-        const uint32_t wt = u / Q, q = u % Q;
+    // a word tile (TW <= 64 words) per warp: lane holds words lane and 32 + lane
+    for (uint32_t wt = warp * nrb + rb; wt < nt; wt += nwarps) {
         const uint32_t w0 = wt * TW + lane, w1 = w0 + 32u;
-        const uint32_t x0 = lane < TW ? __ldcg(bits + w0) : 0u;
-        const uint32_t x1 = 32u + lane < TW ? __ldcg(bits + w1) : 0u;
+        const bool h0 = lane < TW, h1 = 32u + lane < TW;
+        uint32_t x0 = h0 ? __ldcg(bits + w0) : 0u, x1 = h1 ? __ldcg(bits + w1) : 0u;
+        const uint32_t c0 = h0 ? __ldcg(clr + w0) : 0u, c1 = h1 ? __ldcg(clr + w1) : 0u;
         const uint32_t r0 = s_tpre[wt];
-        uint32_t v0 = __popc(x0), v1 = __popc(x1);
-        // ones in the tile before the part's first word q UW
-        const uint32_t pre = __reduce_add_sync(0xFFFFFFFFu, (lane < q * UW ? v0 : 0u) + (32u + lane < q * UW ? v1 : 0u));
-        if (q == 0u) {
-            if (TW > 1u) {
-                if (lane < TW) sums[W + w0] = v0;
-                if (32u + lane < TW) sums[W + w1] = v1;
-            }
+        {  // the tile's share of the first A zero bits, by the zeros before each word
+            const uint32_t z0 = h0 ? ~x0 & vmask : 0u, z1 = h1 ? ~x1 & vmask : 0u;
+            uint32_t e0 = __popc(z0), e1 = __popc(z1);
 #pragma unroll
-            for (uint32_t L = 1; L <= 5; ++L) {
-                v0 += __shfl_down_sync(0xFFFFFFFFu, v0, 1u << (L - 1u));
-                v1 += __shfl_down_sync(0xFFFFFFFFu, v1, 1u << (L - 1u));
-                if ((1u << L) < TW && (lane & ((1u << L) - 1u)) == 0u) {
-                    if (lane < TW) sums[(W + w0) >> L] = v0;
-                    if (32u + lane < TW) sums[(W + w1) >> L] = v1;
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y0 = __shfl_up_sync(0xFFFFFFFFu, e0, o), y1 = __shfl_up_sync(0xFFFFFFFFu, e1, o);
+                if ((int)lane >= o) {
+                    e0 += y0;
+                    e1 += y1;
                 }
             }
-            const uint32_t half0 = __shfl_sync(0xFFFFFFFFu, v0, 0), half1 = __shfl_sync(0xFFFFFFFFu, v1, 0);
-            const uint32_t node = (wt + 1u < nt ? s_tpre[wt + 1u] : Nn) - r0;
-            if (lane == 0) {
-                if (half0 + half1 != node) set_err(I.g, kErrLink);
-                if (nt > 1u) sums[nt + wt] = node;  // (a single tile's node is the root, written above)
+            e1 += __shfl_sync(0xFFFFFFFFu, e0, 31);
+            const int left = (int)min((long long)A - ((long long)wt * TS - s_old[wt]), 4096ll);  // A less the zeros before the tile
+            x0 = (x0 & ~c0) | lowest_set(z0, left - (int)(e0 - __popc(z0)));
+            x1 = (x1 & ~c1) | lowest_set(z1, left - (int)(e1 - __popc(z1)));
+        }
+        if (h0) bits[w0] = x0;
+        if (h1) bits[w1] = x1;
+        if (c0) clr[w0] = 0u;
+        if (c1) clr[w1] = 0u;
+        uint32_t v0 = __popc(x0), v1 = __popc(x1);
+        if (TW > 1u) {
+            if (h0) sums[W + w0] = v0;
+            if (h1) sums[W + w1] = v1;
+        }
+#pragma unroll
+        for (uint32_t L = 1; L <= 5; ++L) {
+            v0 += __shfl_down_sync(0xFFFFFFFFu, v0, 1u << (L - 1u));
+            v1 += __shfl_down_sync(0xFFFFFFFFu, v1, 1u << (L - 1u));
+            if ((1u << L) < TW && (lane & ((1u << L) - 1u)) == 0u) {
+                if (h0) sums[(W + w0) >> L] = v0;
+                if (h1) sums[(W + w1) >> L] = v1;
             }
         }
-        // the part's rows of the live list and, from its zero bits, of the
-        // next frame's free list (Alg. 8 for every rank; every earlier tile
-        // holds 2^tbits slots)
-        uint32_t row = r0 + pre, zrow = wt * TS - r0 + (q * UW * 32u - pre);
+        const uint32_t half0 = __shfl_sync(0xFFFFFFFFu, v0, 0), half1 = __shfl_sync(0xFFFFFFFFu, v1, 0);
+        const uint32_t node = (wt + 1u < nt ? s_tpre[wt + 1u] : Nn) - r0;
+        if (lane == 0) {
+            if (half0 + half1 != node) set_err(I.g, kErrLink);
+            if (nt > 1u) sums[nt + wt] = node;  // (a single tile's node is the root, written above)
+        }
+        // the tile's rows of the live list (Alg. 7 for every index) and, from
+        // its zero bits, of the next frame's free list (Alg. 8 for every rank;
+        // every earlier tile holds 2^tbits slots): word by word, lane b tests
+        // bit b and the set ones take consecutive rows, so every store is one
+        // contiguous run
+        uint32_t row = r0, zrow = wt * TS - r0;
 #pragma unroll 4
-        for (uint32_t i = q * UW; i < (q + 1u) * UW; ++i) {
+        for (uint32_t i = 0; i < TW; ++i) {
             const uint32_t x = __shfl_sync(0xFFFFFFFFu, i < 32u ? x0 : x1, i & 31u);
             const uint32_t z = ~x & vmask;
             const uint32_t sl = (wt * TW + i) * 32u + lane;
@@ -2320,7 +2373,7 @@ __global__ void __launch_bounds__(kFThreads, CBT_FRAME_MIN_BLOCKS) k_frame1(Batc
     };
     stamp(bt, 0);
     // read before any block can reach the final phase, which sets it
-    const bool carried = __ldcg(&bt.inst0.g->freel_full) != 0u;
+    const Carry carry{__ldcg(&bt.inst0.g->freel_full)};
     // the decode tables are fetched now and stored after prep's own loads
     // have gone out
     static_assert(kFThreads == 256, "dec_fetch splits the table over 256 threads");
@@ -2344,19 +2397,20 @@ __global__ void __launch_bounds__(kFThreads, CBT_FRAME_MIN_BLOCKS) k_frame1(Batc
         sync();
     }
     stamp(bt, 4);
-    phase_alloc1(bt, s_c, all_granted, carried, tbits, s_cnt, s_warp, s_w, &s_n, s_buf);
+    phase_alloc1(bt, s_c, all_granted, carry, tbits, s_cnt, s_warp, s_w, &s_n, s_buf);
     sync();
     stamp(bt, 5);
-    phase_fill1(bt, s_c, all_granted, s_cnt, s_buf, s_warp);
-    sync();
-    stamp(bt, 6);
-    phase_final1(bt, s_c, s_buf, s_warp, s_tmp, tbits, carried);
+    const uint32_t half = gridDim.x / 2u, nfb = gridDim.x - half;  // half of the blocks for the final part
+    if (blockIdx.x < nfb) phase_fill1(bt, s_c, all_granted, carry, blockIdx.x, nfb, s_cnt, s_buf, s_warp);
+    if (half == 0u || blockIdx.x >= nfb)
+        phase_final1(bt, s_c, all_granted, half ? blockIdx.x - nfb : 0u, half ? half : 1u, s_buf, s_warp, s_red, tbits,
+                     carry);
     if (bt.fp0.vout) {
         sync();
-        stamp(bt, 7);
+        stamp(bt, 6);
         vertices_of<F>(bt.inst0, bt.fp0, s_tab, s_buf, &s_n);
     } else {
-        stamp(bt, 7);
+        stamp(bt, 6);
     }
     __syncthreads();
     if (threadIdx.x == 0) {

@@ -39,7 +39,7 @@ cudaError_t launch_frame(const BatchDev& bt, int form, int grid, cudaStream_t s)
 constexpr uint32_t kFrame1MaxCap = 1u << 22;
 constexpr uint32_t kFrame1SmallCap = 1u << 16;  // pools up to this run with two blocks per SM
 constexpr uint32_t kFrame1TileWords = 64;
-constexpr int kFrame1Phases = 8;
+constexpr int kFrame1Phases = 7;
 int frame1_blocks_per_sm();
 cudaError_t launch_frame1(const BatchDev& bt, int form, int grid, uint32_t tbits, cudaStream_t s);
 // The same per vertex form (cbt_frame.cuh, one source file per form so that

@@ -948,12 +948,13 @@ __device__ __forceinline__ void clear_bit(const Inst& I, uint32_t s) {
     atomicAnd(I.bits + (s >> 5), ~(1u << (s & 31u)));
 }
 
-// How the fill reads a destination word and updates the bitfield: here the
+// How the fill reads a destination word and the free list and updates the bitfield: here the
 // word is the free-list index itself and A the frame's allocation count
 // (the single-instance frame has a form that resolves tile-local words).
 struct DestPlain {
     uint32_t A;
     __device__ __forceinline__ uint32_t operator()(uint32_t d) const { return d; }
+    __device__ __forceinline__ const uint32_t* freel(const Inst& I) const { return I.freel; }
     __device__ __forceinline__ void set(const Inst& I, uint32_t s) const { set_bit(I, s); }
     __device__ __forceinline__ void clear(const Inst& I, uint32_t s) const { clear_bit(I, s); }
 };
@@ -988,7 +989,7 @@ static __device__ void across_resolve(const Inst& I, Across& a, int E, bool hv, 
                 set_err(I.g, kErrLink);
                 continue;
             }
-            a.slot[E][h] = I.freel[yd + leaf];
+            a.slot[E][h] = dm.freel(I)[yd + leaf];
             a.rev[E][h] = edge;
         }
     } else if (yc.x & kMerged) {
@@ -997,7 +998,7 @@ static __device__ void across_resolve(const Inst& I, Across& a, int E, bool hv, 
             set_err(I.g, kErrLink);
             return;
         }
-        a.slot[E][0] = I.freel[yd];
+        a.slot[E][0] = dm.freel(I)[yd];
         a.rev[E][0] = (yc.x & kHeapOdd) ? (uint32_t)kNe : (uint32_t)kPe;
     } else {
         if (hv) {
@@ -1047,7 +1048,7 @@ static __device__ uint32_t fill_split(const Inst& I, uint32_t s, uint32_t cmd, u
     const uint4 rx = I.nb[s];
     uint32_t slots[4];
 #pragma unroll
-    for (int l = 0; l < 4; ++l) slots[l] = (uint32_t)l < n ? I.freel[dest + (uint32_t)l] : 0u;
+    for (int l = 0; l < 4; ++l) slots[l] = (uint32_t)l < n ? dm.freel(I)[dest + (uint32_t)l] : 0u;
     Across a;
     across_load(I, rx, a);
     const bool xodd = (cmd & kDepthOdd) != 0u;
@@ -1126,7 +1127,7 @@ __device__ __forceinline__ void edge_resolve(const Inst& I, Edge1& a, const DM& 
             set_err(I.g, kErrLink);
             return;
         }
-        a.slot = I.freel[yd + leaf];
+        a.slot = dm.freel(I)[yd + leaf];
         a.rev = edge;
     } else if (a.yc.x & kMerged) {
         const uint32_t yd = dm(a.yc.y);
@@ -1134,7 +1135,7 @@ __device__ __forceinline__ void edge_resolve(const Inst& I, Edge1& a, const DM& 
             set_err(I.g, kErrLink);
             return;
         }
-        a.slot = I.freel[yd];
+        a.slot = dm.freel(I)[yd];
         a.rev = (a.yc.x & kHeapOdd) ? (uint32_t)kNe : (uint32_t)kPe;
     } else {
         a.slot = a.y;
@@ -1172,7 +1173,7 @@ static __device__ uint32_t fill_merge(const Inst& I, uint32_t dest, const uint4 
 #pragma unroll
     for (int k = 0; k < 2; ++k) {  // unrolled loops keep everything in registers
         if (k == np) break;
-        ps[k] = I.freel[dest + (uint32_t)k];
+        ps[k] = dm.freel(I)[dest + (uint32_t)k];
         const uint32_t u = ms[2 * k], v = ms[2 * k + 1];
         if (bad_slot(I, u, kErrLink) || bad_slot(I, v, kErrLink)) return 0u;
         ju[k] = I.heap[u];
