@@ -234,6 +234,35 @@ constexpr uint32_t kScanItems = kScanThreads * kScanPerThread;  // 4096 live ind
 constexpr uint32_t kMaxTileWords = 256;                       // up to 8192 bits per tile
 constexpr uint32_t kMinTileWords = 64;
 
+// -------------------------------------------------------- dependent launches
+
+// The kernels of the indexed export, and prep and the vertices on their own,
+// are launched with programmatic stream serialisation: the next kernel's
+// blocks are brought in while the last ones of this kernel run, and wait here
+// for this kernel's end and its writes, so that the launch and the ramp
+// between two kernels overlap (the export of 0.9M triangles after a frame:
+// 276 -> 267 us; the vertices of 0.9M bisectors: 54 -> 51; the reduction with
+// its compaction, and a whole per-step frame, gained nothing). Called first in
+// every such kernel; what an earlier kernel of the sequence writes is not read
+// through the read-only path (__ldg or const __restrict__).
+__device__ __forceinline__ void sequence_begin() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <typename... P, typename... A>
+cudaError_t launch_sequence(void (*kernel)(P...), unsigned grid, unsigned block, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // ------------------------------------------------------------------ bits
 
 __device__ __forceinline__ int bitlen64(uint64_t x) { return 64 - __clzll((long long)x); }

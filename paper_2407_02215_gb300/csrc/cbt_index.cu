@@ -69,13 +69,14 @@ __device__ __forceinline__ int root_corner(uint64_t j, int d, int v) {
 // The live count N is read on the device (the CBT root); a count above the
 // capacity the workspace was carved for is reported and nothing is done.
 __device__ __forceinline__ uint32_t live_n(const Inst& I, uint32_t cap) {
-    const uint32_t n = __ldg(I.sums + 1);
+    const uint32_t n = __ldcg(I.sums + 1);
     return n <= cap ? n : 0u;
 }
 
 // Counts and tile counts cleared, every root point's smallest occurrence
 // set to none.
 __global__ void __launch_bounds__(kIThreads) k_index_init(IndexWs ws, uint32_t words) {
+    sequence_begin();
     for (uint32_t k = blockIdx.x * kIThreads + threadIdx.x; k < words || k < ws.npts; k += gridDim.x * kIThreads) {
         if (k < words) ws.cnt[k] = 0u;
         if (k < ws.npts) ws.rootrep[k] = kNull;
@@ -84,9 +85,10 @@ __global__ void __launch_bounds__(kIThreads) k_index_init(IndexWs ws, uint32_t w
 
 __global__ void __launch_bounds__(kIThreads) k_index_roots(Inst I, const uint32_t* corner, IndexWs ws,
                                                            uint32_t cap) {
+    sequence_begin();
     const uint32_t N = live_n(I, cap);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-        ws.cnt[2] = __ldg(I.sums + 1);
+        ws.cnt[2] = __ldcg(I.sums + 1);
         if (ws.cnt[2] > cap) atomicOr(ws.cnt, kIxCap);
     }
     for (uint32_t i = blockIdx.x * kIThreads + threadIdx.x; i < N; i += gridDim.x * kIThreads) {
@@ -177,6 +179,7 @@ __device__ uint32_t fan_min(const Inst& I, uint32_t* err, uint32_t s0, uint32_t 
 // occurrence, or the fan's first); representatives flagged and counted per
 // tile.
 __global__ void __launch_bounds__(kIThreads) k_index_fans(Inst I, IndexWs ws, uint32_t cap) {
+    sequence_begin();
     const uint32_t N = live_n(I, cap), n3 = 3u * N;
     const uint32_t lane = threadIdx.x & 31u;
     for (uint32_t base = blockIdx.x * kIThreads; base < n3; base += gridDim.x * kIThreads) {
@@ -236,6 +239,7 @@ __global__ void __launch_bounds__(kIThreads) k_index_fans(Inst I, IndexWs ws, ui
 }
 
 __global__ void __launch_bounds__(kIThreads) k_index_ids(Inst I, IndexWs ws, uint32_t cap) {
+    sequence_begin();
     __shared__ Pair s_warp[kIThreads / 32 + 1];
     const uint32_t n3 = 3u * live_n(I, cap);
     constexpr uint32_t kPer = kITile / kIThreads;
@@ -261,6 +265,7 @@ __global__ void __launch_bounds__(kIThreads) k_index_ids(Inst I, IndexWs ws, uin
 __global__ void __launch_bounds__(kIThreads) k_index_write(Inst I, IndexWs ws, uint32_t cap, const float* tri,
                                                            float* verts, uint32_t vcap, uint32_t* idx,
                                                            uint64_t* ids, uint32_t* h_cnt) {
+    sequence_begin();
     const uint32_t N = live_n(I, cap), n3 = 3u * N;
     // the earlier launches have set every count
     if (blockIdx.x == 0 && threadIdx.x < 3u)
@@ -346,11 +351,11 @@ int launch_index(const Inst& I, const uint32_t* corner, uint32_t npts, uint32_t 
     const uint32_t most = static_cast<uint32_t>(sms) * 8u;
     auto grid = [&](uint32_t work) { return work == 0 ? 1u : (work < most ? work : most); };
     // sized for the capacity; every kernel reads the live count on the device
-    k_index_init<<<grid(((words > npts ? words : npts) + kIThreads - 1u) / kIThreads), kIThreads, 0, s>>>(ws, words);
-    k_index_roots<<<grid((cap + kIThreads - 1u) / kIThreads), kIThreads, 0, s>>>(I, corner, ws, cap);
-    k_index_fans<<<grid((n3 + kIThreads - 1u) / kIThreads), kIThreads, 0, s>>>(I, ws, cap);
-    k_index_ids<<<grid(ntiles), kIThreads, 0, s>>>(I, ws, cap);
-    k_index_write<<<grid((n3 + kIThreads - 1u) / kIThreads), kIThreads, 0, s>>>(I, ws, cap, tri, verts, vcap,
+    launch_sequence(k_index_init, grid(((words > npts ? words : npts) + kIThreads - 1u) / kIThreads), kIThreads, s, ws, words);
+    launch_sequence(k_index_roots, grid((cap + kIThreads - 1u) / kIThreads), kIThreads, s, I, corner, ws, cap);
+    launch_sequence(k_index_fans, grid((n3 + kIThreads - 1u) / kIThreads), kIThreads, s, I, ws, cap);
+    launch_sequence(k_index_ids, grid(ntiles), kIThreads, s, I, ws, cap);
+    launch_sequence(k_index_write, grid((n3 + kIThreads - 1u) / kIThreads), kIThreads, s, I, ws, cap, tri, verts, vcap,
                                                                                 idx, ids, d_cnt);
     if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) return CBT_ECUDA;
     uint32_t cnt[3];

@@ -20,6 +20,7 @@ namespace cbtgpu {
 // (block 0), the look-back descriptors zeroed, and the camera-relative root
 // tables. FP64 is used here only to subtract the eye from the root vertices.
 __global__ void __launch_bounds__(kThreads) k_prep(BatchDev bt, int frame_start) {
+    sequence_begin();
     __shared__ uint32_t s_carry, s_scarry, s_live;
     __shared__ Pair s_warp[kThreads / 32 + 1];
     const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x;
@@ -718,6 +719,7 @@ __global__ void __launch_bounds__(kThreads) k_leaves(Inst I, uint32_t* slots, ui
 // over static tiles of its pool capacity (tiles past the live count exit).
 template <int F>
 __global__ void __launch_bounds__(kThreads, 3) k_vertices(BatchDev bt) {
+    sequence_begin();
     __shared__ uint32_t s_b;
     __shared__ Inst s_I;
     __shared__ FrameP s_fp;
@@ -769,7 +771,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_vertices(BatchDev bt) {
 // ---------------------------------------------------------------- launch
 
 void launch_prep(const BatchDev& bt, bool frame_start, int grid, cudaStream_t s) {
-    k_prep<<<grid, kThreads, 0, s>>>(bt, frame_start ? 1 : 0);
+    launch_sequence(k_prep, grid, kThreads, s, bt, frame_start ? 1 : 0);
 }
 void launch_classify(const BatchDev& bt, int form, int grid, cudaStream_t s) {
     switch (form) {
@@ -790,9 +792,9 @@ void launch_cbt(const BatchDev& bt, int grid, cudaStream_t s) {
 }
 void launch_vertices(const BatchDev& bt, int form, int grid, cudaStream_t s) {
     switch (form) {
-        case kFormF32: k_vertices<kFormF32><<<grid, kThreads, 0, s>>>(bt); break;
-        case kFormFixed: k_vertices<kFormFixed><<<grid, kThreads, 0, s>>>(bt); break;
-        default: k_vertices<kFormAny><<<grid, kThreads, 0, s>>>(bt); break;
+        case kFormF32: launch_sequence(k_vertices<kFormF32>, grid, kThreads, s, bt); break;
+        case kFormFixed: launch_sequence(k_vertices<kFormFixed>, grid, kThreads, s, bt); break;
+        default: launch_sequence(k_vertices<kFormAny>, grid, kThreads, s, bt); break;
     }
 }
 void launch_init(const Inst& I, const int32_t* twin, const int32_t* next, const int32_t* prev,

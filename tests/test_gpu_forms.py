@@ -114,3 +114,29 @@ def test_batch_of_all_forms(fused):
                 want = o.vertices(fp.eye, fp.precision, fp.fixed_shift, fp.sphere_radius, frame=fp)
                 got = rows[b, :o.live_count].cpu().numpy()
                 assert np.array_equal(got.view(np.uint32), want.view(np.uint32)), f"frame {k} instance {b}"
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("sphere", [False, True], ids=["flat", "sphere"])
+def test_form_changing_every_frame(sphere):
+    """One instance of a small mesh whose frames change form, and now and then
+    execution form: its root table is rewritten in another layout each time."""
+    import torch
+
+    import paper_2407_02215_gb300 as P
+    P.build_library()
+    names = [n for n in FORMS if n.startswith("sphere") == sphere]
+    scenes = {n: _scene(n) for n in names}
+    mesh, max_depth, _ = scenes[names[0]]
+    g, o = P.CBT(mesh, D, max_depth, point_cache=sphere), Oracle(mesh, D, max_depth)
+    rows = torch.zeros((1 << D, 3, 3), dtype=torch.float32, device="cuda")
+    for k in range(40):
+        fp = scenes[names[k % len(names)]][2][k // 2]
+        g.set_fused(k % 11 != 7)
+        g.update(fp, vertices_out=rows)
+        o.update(fp)
+        assert g.stats()["error"] == 0
+        assert_same_state(g, o, f"frame {k}")
+        want = o.vertices(fp.eye, fp.precision, fp.fixed_shift, fp.sphere_radius, frame=fp)
+        got = rows[:o.live_count].cpu().numpy()
+        assert np.array_equal(got.view(np.uint32), want.view(np.uint32)), f"frame {k}: vertices"
