@@ -56,7 +56,7 @@ struct Layout {
 
 // A batch region for instances with the given pool sizes and halfedge counts.
 struct BatchLayout {
-    size_t inst, fps, bg, tile_base, ctile_base, stile_base, wtile_base, vtile_base, rel_base, status, tpre, total;
+    size_t inst, fps, bg, tile_base, ctile_base, stile_base, wtile_base, vtile_base, rel_base, status, tpre, wish, total;
     uint32_t Titems, TwordsMax, Trel;
 };
 
@@ -84,6 +84,7 @@ BatchLayout batch_layout(uint32_t n, const uint32_t* cap, const uint32_t* W, con
     L.rel_base = take(4u * (n + 1u));
     L.status = take(8u * (2u * static_cast<size_t>(L.Titems) + L.TwordsMax));
     L.tpre = take(4u * 2u * static_cast<size_t>(L.TwordsMax));
+    L.wish = take(8u * static_cast<size_t>(L.Titems));
     L.total = off;
     return L;
 }
@@ -280,6 +281,7 @@ int batch_build(cbt_state* const* states, uint32_t n, char* region, cudaStream_t
     d.bg = reinterpret_cast<BatchGlobals*>(region + B->L.bg);
     d.status = reinterpret_cast<unsigned long long*>(region + B->L.status);
     d.tpre = reinterpret_cast<uint32_t*>(region + B->L.tpre);
+    d.wish = reinterpret_cast<unsigned long long*>(region + B->L.wish);
     std::vector<Inst> insts(n);
     for (uint32_t b = 0; b < n; ++b) insts[b] = states[b]->inst;
     std::memset(&d.inst0, 0, sizeof(Inst));

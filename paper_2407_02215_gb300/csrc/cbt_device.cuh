@@ -100,7 +100,7 @@ struct Globals {
     // wish to merge) and requested split cost, summed by the walks; when their
     // sum fits the free slots every request is granted without the prefix gate
     unsigned long long rq_merge, rq_split;
-    uint32_t nwalk;  // single-instance frame: entries of the frame's walk list
+    uint32_t nwalk;  // single-instance frame: entries of the frame's walk list (0 between its frames)
     uint32_t marks_clean;  // 1 when the chain-mark words (chg) of the live slots are 0 (the
                            // single-instance frame leaves them so; the other frames clear this)
     uint32_t freel_full;   // bit 0: a free list of every zero bit of the bitfield in slot order is kept, in
@@ -220,6 +220,8 @@ struct BatchDev {
     uint32_t* vcount;            // the export on its own (B == 1): the live count goes here, in mapped
                                  // host memory, and nothing else is written when it exceeds vcap
     uint32_t timing;             // one-launch frame: record phase boundaries
+    unsigned long long* wish;    // single-instance frame: [Titems] the split wishes' lower-bound costs per scan
+                                 // tile, 0 between frames of that kernel
     uint32_t* tpre;              // single-instance frame: [2][Twords] ones before each word tile of
                                  // the next frame's starting bitfield (which: the instance's freel_full)
 };

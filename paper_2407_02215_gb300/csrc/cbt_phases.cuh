@@ -205,9 +205,14 @@ __device__ __forceinline__ void tile_begin(const BatchDev& bt, const uint32_t* b
 // Entry le of an instance's camera-relative root table: the frame's eye
 // subtracted in FP64, then rounded to the frame's precision (FP32, fixed
 // point at 2^shift, or FP64; the sphere form keeps the absolute roots).
-__device__ __forceinline__ void rel_store(const double* root64, void* rel, Globals* g, const double* eye,
-                                          uint32_t precision, int32_t shift, uint32_t le) {
-    const double diff = __dsub_rn(root64[le], eye[le % 3u]);
+// (v: the root vertex's coordinate root64[le].)
+__device__ __forceinline__ void rel_put(double v, void* rel, Globals* g, const double* eye, uint32_t precision,
+                                        int32_t shift, uint32_t le) {
+    if (precision == 3) {
+        static_cast<double*>(rel)[le] = v;  // absolute: the projection needs it
+        return;
+    }
+    const double diff = __dsub_rn(v, eye[le % 3u]);
     if (precision == 1) {
         const double sc = __dmul_rn(diff, pow2d(shift));
         long long x = 0;
@@ -218,11 +223,13 @@ __device__ __forceinline__ void rel_store(const double* root64, void* rel, Globa
         static_cast<long long*>(rel)[le] = x;
     } else if (precision == 2) {
         static_cast<double*>(rel)[le] = diff;
-    } else if (precision == 3) {
-        static_cast<double*>(rel)[le] = root64[le];  // absolute: the projection needs it
     } else {
         static_cast<float*>(rel)[le] = __double2float_rn(diff);
     }
+}
+__device__ __forceinline__ void rel_store(const double* root64, void* rel, Globals* g, const double* eye,
+                                          uint32_t precision, int32_t shift, uint32_t le) {
+    rel_put(root64[le], rel, g, eye, precision, shift, le);
 }
 
 // Entry e of the batch's root tables (instances laid out by rel_base).
@@ -542,10 +549,11 @@ __device__ __forceinline__ void sphere_points(const Inst& I, const FrameP& fp, u
     }
 }
 
+// gen: the frame's cache generation (0: read from the instance's counters).
 __device__ __forceinline__ void sphere_wishes(const Inst& I, const FrameP& fp, uint32_t s, uint64_t j, int d,
                                               uint32_t h, const uint32_t* tab, bool& split, bool& merge,
-                                              float* keep) {
-    const unsigned long long gen = I.g->pc_gen;
+                                              float* keep, unsigned long long gen) {
+    if (gen == 0ull) gen = I.g->pc_gen;
     const ulonglong2 tag = I.pct[s];
     if (tag.x != j || tag.y != gen) {
         if (float_weights(d))
@@ -575,21 +583,27 @@ __device__ __forceinline__ void sphere_wishes(const Inst& I, const FrameP& fp, u
 
 // A new generation of the sphere-point cache when a LOD frame of the sphere
 // form has a shape (radius, displacement) other than the one the current
-// generation was made with. Called for each instance by one thread, at the
-// frame's start, before any classify.
-__device__ __forceinline__ void pc_generation(Globals* g, const FrameP& fp) {
-    if (fp.precision != 3u || fp.mode != 0u) return;
+// generation was made with: the frame's generation, from the counters the
+// last frame left (pc_generation_of), and its storing (pc_generation), by one
+// thread per instance, with no thread of the other kind running.
+__device__ __forceinline__ bool pc_changed(const Globals* g, const FrameP& fp) {
+    if (fp.precision != 3u || fp.mode != 0u) return false;
     const unsigned long long rb = (unsigned long long)__double_as_longlong(fp.radius);
     const uint32_t a = __float_as_uint(fp.damp), f = __float_as_uint(fp.dfreq);
-    if (g->pc_gen == 0ull || g->pc_radius != rb || g->pc_damp != a || g->pc_dfreq != f || g->pc_doct != fp.doct ||
-        g->pc_dseed != fp.dseed) {
-        g->pc_gen += 1ull;
-        g->pc_radius = rb;
-        g->pc_damp = a;
-        g->pc_dfreq = f;
-        g->pc_doct = fp.doct;
-        g->pc_dseed = fp.dseed;
-    }
+    return g->pc_gen == 0ull || g->pc_radius != rb || g->pc_damp != a || g->pc_dfreq != f || g->pc_doct != fp.doct ||
+           g->pc_dseed != fp.dseed;
+}
+__device__ __forceinline__ unsigned long long pc_generation_of(const Globals* g, const FrameP& fp) {
+    return g->pc_gen + (pc_changed(g, fp) ? 1ull : 0ull);
+}
+__device__ __forceinline__ void pc_generation(Globals* g, const FrameP& fp) {
+    if (!pc_changed(g, fp)) return;
+    g->pc_gen += 1ull;
+    g->pc_radius = (unsigned long long)__double_as_longlong(fp.radius);
+    g->pc_damp = __float_as_uint(fp.damp);
+    g->pc_dfreq = __float_as_uint(fp.dfreq);
+    g->pc_doct = fp.doct;
+    g->pc_dseed = fp.dseed;
 }
 
 // Compatibility chain of bisector b on the frame-start state (command form
@@ -675,7 +689,7 @@ static __device__ uint32_t chain_walk(const Inst& I, uint32_t b, int d, bool sca
 template <int F>
 __device__ __forceinline__ bool item_wishes(const Inst& I, const FrameP& fp, uint64_t key, uint32_t s, uint64_t j,
                                             const uint32_t* tab, bool& split, bool& merge, float* keep = nullptr,
-                                            bool* kept = nullptr) {
+                                            bool* kept = nullptr, unsigned long long gen = 0) {
     const int d = depth_of(j, I.ch);
     const uint32_t h = (uint32_t)((j >> d) - (1ull << I.ch));
     split = merge = false;
@@ -684,7 +698,7 @@ __device__ __forceinline__ bool item_wishes(const Inst& I, const FrameP& fp, uin
     switch (fp.mode) {
         case 0:
             if (precision_in<F>(fp) == 3u && I.pc)
-                sphere_wishes(I, fp, s, j, d, h, tab, split, merge, keep);
+                sphere_wishes(I, fp, s, j, d, h, tab, split, merge, keep, gen);
             else
                 lod_wishes<F>(I, fp, j, d, h, tab, split, merge, keep);
             if (kept) *kept = keep != nullptr;
@@ -733,9 +747,9 @@ __device__ __forceinline__ uint32_t store_command(const Inst& I, const FrameP& f
 template <int F>
 __device__ __forceinline__ uint32_t classify_item(const Inst& I, const FrameP& fp, uint64_t key, uint32_t i,
                                                   uint32_t s, uint64_t j, const uint32_t* tab, uint32_t* s_cnt,
-                                                  bool cache = false, bool merge_in = false) {
+                                                  bool cache = false, bool merge_in = false, unsigned long long gen = 0) {
     bool split, merge, kept;
-    if (!item_wishes<F>(I, fp, key, s, j, tab, split, merge, cache ? I.vc + 9ull * s : nullptr, &kept)) {
+    if (!item_wishes<F>(I, fp, key, s, j, tab, split, merge, cache ? I.vc + 9ull * s : nullptr, &kept, gen)) {
         set_err(I.g, kErrLink);
         if (!merge_in) *cmd_ptr(I, s) = 0u;
         I.scan[i] = 0u;
