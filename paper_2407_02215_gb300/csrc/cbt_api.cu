@@ -35,6 +35,7 @@ const char* const kPhaseNames1[kFrame1Phases] = {"prep",  "classify", "walks",  
                                                  "alloc", "fill",     "vertices"};
 constexpr uint32_t kFusedTileWords = 64;
 constexpr uint32_t kFusedMaxTileWords = 128;
+constexpr size_t kPinnedCounts = 16;  // after a batch's pinned frame parameters: a state's counts
 
 size_t align256(size_t x) { return (x + 255u) & ~static_cast<size_t>(255u); }
 
@@ -210,7 +211,8 @@ struct cbt_state {
     Inst inst;
     uint32_t* corner;  // [H][3] global points of the root corners: vert[h], vert[next h], V + face[h]
     uint32_t npts;     // global points: 1 + the largest in corner
-    uint32_t* h_ix = nullptr;  // pinned counts: of the last cbt_index (words 0 to 2) and cbt_vertices (3)
+    uint32_t* h_ix;  // pinned counts, after self's frame parameters: of the last cbt_index (words 0 to 2) and
+                     // cbt_vertices (3)
     void* workspace;
     size_t bytes;
     int sms;
@@ -289,7 +291,7 @@ int batch_build(cbt_state* const* states, uint32_t n, char* region, cudaStream_t
     int rc = CBT_OK;
     if (cudaMemcpyAsync(region + B->L.inst, insts.data(), sizeof(Inst) * n, cudaMemcpyHostToDevice, s) ||
         cudaMemsetAsync(d.bg, 0, sizeof(BatchGlobals), s) ||
-        cudaMallocHost(reinterpret_cast<void**>(&B->h_fps), sizeof(FrameP) * n) ||
+        cudaMallocHost(reinterpret_cast<void**>(&B->h_fps), sizeof(FrameP) * n + kPinnedCounts) ||
         cudaEventCreateWithFlags(&B->staged, cudaEventDisableTiming))
         rc = CBT_ECUDA;
     B->tw = fused_tile_words(B);  // the one-launch frame is the default form
@@ -689,6 +691,7 @@ extern "C" int cbt_create(int32_t H, const int32_t* twin, const int32_t* next, c
         delete st;
         return rc;
     }
+    st->h_ix = reinterpret_cast<uint32_t*>(st->self->h_fps + 1);
     *out = st;
     return CBT_OK;
 }
@@ -737,13 +740,8 @@ extern "C" int cbt_leaves(cbt_state* st, uint32_t* d_slots, uint64_t* d_heap, ui
 }
 
 namespace {
-// The state's page-locked counts (made by the first call that needs them) and
-// their address on the device.
+// The address on the device of the state's page-locked counts.
 int pinned_counts(cbt_state* st, uint32_t** d) {
-    if (!st->h_ix && cudaMallocHost(reinterpret_cast<void**>(&st->h_ix), 16u) != cudaSuccess) {
-        st->h_ix = nullptr;
-        return CBT_ECUDA;
-    }
     return cudaHostGetDevicePointer(reinterpret_cast<void**>(d), st->h_ix, 0) == cudaSuccess ? CBT_OK : CBT_ECUDA;
 }
 }  // namespace
@@ -876,7 +874,6 @@ extern "C" int cbt_stats(cbt_state* st, cbt_frame_stats* out, cbt_stream_t strea
 
 extern "C" void cbt_destroy(cbt_state* st) {
     if (!st) return;
-    if (st->h_ix) cudaFreeHost(st->h_ix);
     batch_free(st->self);
     delete st;
 }
