@@ -126,6 +126,38 @@ __device__ __forceinline__ void ctx_tile(const BatchDev& bt, const uint32_t* bas
     __syncthreads();
 }
 
+// The tiles of a phase handed out as blocks finish: tile blockIdx.x first, then
+// by a counter, taken while the current tile is worked on. What a tile costs
+// differs and clusters (grants and chains at an instance's start, culled
+// regions): with tiles dealt round robin the batch frame waited for its
+// slowest blocks, and with four consecutive tiles at a time it was slower
+// still (batch of 15M bisectors: 1744 and 1953 us; handed out 1684).
+struct TileFeed {
+    uint32_t* ticket;
+    uint32_t* s;  // [2] in shared memory
+    uint32_t p = 0, ahead = 0;
+    __device__ __forceinline__ TileFeed(uint32_t* t, uint32_t* shared) : ticket(t), s(shared) {}
+    __device__ __forceinline__ void take() {
+        if (threadIdx.x == 0) ahead = gridDim.x + atomicAdd(ticket, 1u);
+    }
+    __device__ __forceinline__ uint32_t first() {
+        take();
+        return blockIdx.x;
+    }
+    // With the whole block, at the end of a tile.
+    __device__ __forceinline__ uint32_t next() {
+        if (threadIdx.x == 0) s[p] = ahead;
+        __syncthreads();
+        const uint32_t t = s[p];
+        p ^= 1u;
+        take();
+        return t;
+    }
+};
+// Counters of the phases (tickets of the batch; kAllocDone is the last).
+enum : int { kFeedClassify = 0, kFeedWalks, kFeedGate, kFeedAlloc, kFeedCompact, kFeeds };
+static_assert(kFeeds <= kAllocDone, "counters of their own");
+
 __device__ __forceinline__ unsigned long long pack_pair(Pair p) {
     return ((unsigned long long)p.a << 32) | (unsigned long long)p.b;
 }
@@ -232,7 +264,7 @@ __device__ void phase_prep(const BatchDev& bt, Pair* s_warp, uint32_t* s_tmp) {
             bt.bg->scan_ipt = ipt;
             bt.bg->live_total = s_tmp[2];
             bt.bg->t[kFramePhases] = 0;
-            bt.bg->tickets[kAllocDone] = 0;
+            for (int k = 0; k < 8; ++k) bt.bg->tickets[k] = 0;
         }
     }
     // block 0 sets up the instances; the others share the root tables in
@@ -284,7 +316,9 @@ template <int F>
 __device__ void phase_classify(const BatchDev& bt, FCtx& c, uint32_t* s_tab, uint32_t* s_cnt) {
     const uint32_t T = bt.bg->total_tiles, S = kFThreads * bt.bg->scan_ipt;
     const uint32_t lane = threadIdx.x & 31u;
-    for (uint32_t t = blockIdx.x; t < T; t += gridDim.x) {
+    __shared__ uint32_t s_feed[2];
+    TileFeed feed(&bt.bg->tickets[kFeedClassify], s_feed);
+    for (uint32_t t = feed.first(); t < T; t = feed.next()) {
         stats_reset(s_cnt);
         ctx_tile(bt, bt.tile_base, t, T, c);
         const Inst& I = c.I;
@@ -415,7 +449,9 @@ __device__ void phase_walks(const BatchDev& bt, FCtx& c, uint32_t* s_cnt, unsign
                             uint32_t* s_n) {
     const uint32_t T = bt.bg->total_tiles, S = kFThreads * bt.bg->scan_ipt;
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    for (uint32_t t = blockIdx.x; t < T; t += gridDim.x) {
+    __shared__ uint32_t s_feed[2];
+    TileFeed feed(&bt.bg->tickets[kFeedWalks], s_feed);
+    for (uint32_t t = feed.first(); t < T; t = feed.next()) {
         if (threadIdx.x < 3) s_tmp[threadIdx.x] = 0;
         stats_reset(s_cnt);
         ctx_tile(bt, bt.tile_base, t, T, c);
@@ -630,7 +666,9 @@ template <bool kOne = false>
 __device__ void phase_gate(const BatchDev& bt, FCtx& c, uint32_t* s_cnt, uint32_t* s_red, Pair* s_warp,
                            uint32_t* s_tmp, uint32_t* s_n, uint2* s_list, bool always_recorded = false) {
     const uint32_t T = bt.bg->total_stiles, ipt = bt.bg->scan_ipt;
-    for (uint32_t t = blockIdx.x; t < T; t += gridDim.x) {
+    __shared__ uint32_t s_feed[2];
+    TileFeed feed(&bt.bg->tickets[kFeedGate], s_feed);
+    for (uint32_t t = kOne ? blockIdx.x : feed.first(); t < T; t = kOne ? t + gridDim.x : feed.next()) {
         if (threadIdx.x == 0) *s_n = 0;
         stats_reset(s_cnt);
         ctx_tile(bt, bt.stile_base, t, T, c);
@@ -764,7 +802,9 @@ __device__ void phase_alloc(const BatchDev& bt, FCtx& c, uint32_t* s_cnt, Pair* 
     const uint32_t T = bt.bg->total_stiles, ipt = bt.bg->scan_ipt, S = kFThreads * ipt;
     uint32_t* s_list = s_buf;              // local item indices to validate
     uint32_t* s_fate = s_buf + kFBuf / 2;  // their fates, by local item index
-    for (uint32_t t = blockIdx.x; t < T; t += gridDim.x) {
+    __shared__ uint32_t s_feed[2];
+    TileFeed feed(&bt.bg->tickets[kFeedAlloc], s_feed);
+    for (uint32_t t = feed.first(); t < T; t = feed.next()) {
         if (threadIdx.x == 0) *s_n = 0;
         stats_reset(s_cnt);
         ctx_tile(bt, bt.stile_base, t, T, c);
@@ -1075,7 +1115,9 @@ template <int F>
 __device__ void phase_compact(const BatchDev& bt, FCtx& c, const uint32_t* s_tab, uint32_t* s_buf,
                               uint32_t* s_w, float* s_stage) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (uint32_t wt = blockIdx.x; wt < bt.Twords; wt += gridDim.x) {
+    __shared__ uint32_t s_feed[2];
+    TileFeed feed(&bt.bg->tickets[kFeedCompact], s_feed);
+    for (uint32_t wt = feed.first(); wt < bt.Twords; wt = feed.next()) {
         ctx_tile(bt, bt.wtile_base, wt, bt.Twords, c);
         const Inst& I = c.I;
         const FrameP& fp = c.fp;
