@@ -90,6 +90,11 @@ BatchLayout batch_layout(uint32_t n, const uint32_t* cap, const uint32_t* W, con
     return L;
 }
 
+// What cbt_create stages in the relative vertices' region: the halfedge
+// operators and, 256-byte aligned after them, the positions. Larger than the
+// region's 72 bytes per halfedge for a single triangle.
+size_t rel_stage(size_t h) { return align256(12u * h) + 24u * h; }
+
 bool make_layout(int32_t H, int32_t D, Layout& L) {
     if (H < 3 || D < 1 || D > 30) return false;
     L.ch = ceil_log2(static_cast<uint32_t>(H));
@@ -117,7 +122,7 @@ bool make_layout(int32_t H, int32_t D, Layout& L) {
     L.chgr = take(16u * cap);
     L.vc = take(36u * cap);
     L.root64 = take(72u * h);
-    L.rel = take(72u * h);
+    L.rel = take(std::max(72u * h, rel_stage(h)));
     L.corner = take(12u * h);
     L.rbnd = take(4u * ((h + 31u) / 32u));
     L.freel2 = take(4u * cap);
@@ -657,7 +662,7 @@ extern "C" int cbt_create(int32_t H, const int32_t* twin, const int32_t* next, c
     st->corner = reinterpret_cast<uint32_t*>(b + L.corner);
     st->npts = h ? 1u + *std::max_element(corner.begin(), corner.end()) : 0u;
     int32_t* d_ints = reinterpret_cast<int32_t*>(b + L.rel);
-    double* d_hpos = reinterpret_cast<double*>(b + L.rel + align256(12u * h));
+    double* d_hpos = reinterpret_cast<double*>(b + L.rel + rel_stage(h) - 24u * h);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     cudaMemsetAsync(I.g, 0, sizeof(Globals), s);
     cudaMemsetAsync(I.clr, 0, 4u * L.W, s);

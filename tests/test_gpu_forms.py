@@ -140,3 +140,31 @@ def test_form_changing_every_frame(sphere):
         want = o.vertices(fp.eye, fp.precision, fp.fixed_shift, fp.sphere_radius, frame=fp)
         got = rows[:o.live_count].cpu().numpy()
         assert np.array_equal(got.view(np.uint32), want.view(np.uint32)), f"frame {k}: vertices"
+
+
+@pytest.mark.gpu
+def test_separate_triangles_displaced():
+    """t triangles that share no point: a warp's 32 bisectors have from a few
+    up to more than 64 distinct points, so its displaced points are evaluated
+    in a part of a pass, one pass and two. Exact, as above."""
+    import torch
+
+    import paper_2407_02215_gb300 as P
+    P.build_library()
+    rng = np.random.default_rng(11)
+    for t in (1, 2, 4, 5, 6, 8, 9, 10, 11, 12, 21, 22, 33):
+        pos = rng.uniform(-1.0, 1.0, (t, 1, 3)) * [4.0, 4.0, 0.0] + rng.uniform(0.2, 1.0, (t, 3, 3)) * [[1, 0, 0], [0, 1, 0], [-1, -1, 0]]
+        mesh = W.meshes._mesh("separate", np.arange(3 * t).reshape(t, 3).tolist(), pos)
+        eye = np.array([0.1, 0.2, 3.0])
+        fp = W.cameras.frame_params(W.cameras.Camera(eye=eye, target=eye - [0.0, 0.0, 1.0], up=[0.0, 1.0, 0.0]), 180.0,
+                                    precision=PREC_FP32, disp_amplitude=0.05, disp_frequency=3.0, disp_octaves=6, disp_seed=5)
+        g, o = P.CBT(mesh, 10, 12), Oracle(mesh, 10, 12)
+        rows = torch.zeros((1 << 10, 3, 3), dtype=torch.float32, device="cuda")
+        for k in range(4):
+            g.update(fp, vertices_out=rows)
+            o.update(fp)
+            assert g.stats()["error"] == 0
+            assert_same_state(g, o, f"{t} triangles frame {k}")
+            want = o.vertices(fp.eye, fp.precision, fp.fixed_shift, fp.sphere_radius, frame=fp)
+            got = rows[:o.live_count].cpu().numpy()
+            assert np.array_equal(got.view(np.uint32), want.view(np.uint32)), f"{t} triangles frame {k}: vertices"
