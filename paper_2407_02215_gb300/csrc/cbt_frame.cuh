@@ -1573,8 +1573,9 @@ __device__ void phase_prep1(const BatchDev& bt, uint32_t tbits, uint32_t N) {
 // ones with a hash table in shared memory and evaluates those alone, spread
 // over its lanes. The results are those of evaluating each point, because a
 // point is only shared when the inputs of its evaluation are equal bit for bit.
-// The terrain's classify phase (877k leaves, six octaves) went from 126 to 106 us, the wave
-// planet's (117k) from 43 to 41, its frame from 109 to 102.
+// The terrain's classify phase (877k leaves, six octaves) went from 126 to 106 us (98
+// with two points per lane at a time, fbm2_pair), the wave planet's (117k) from
+// 43 to 41, its frame from 109 to 102.
 template <int F>
 constexpr bool kSharedPoints = F == kFormF32Disp || F == kFormSphere;
 constexpr uint32_t kPtSlots = 1024;  // hash slots (bytes) per warp, eight times its points
@@ -1647,12 +1648,24 @@ __device__ __forceinline__ void lod_wishes_shared(const Inst& I, const FrameP& f
             return *reinterpret_cast<volatile u64*>(key + id) == mine[k];
         });
 #pragma unroll 1
-        for (uint32_t q = lane; q < n; q += 32u) {
-            const uint32_t id = list[q];
-            const u64 v = key[id];
-            const float f = fbm2(__uint_as_float((uint32_t)v), __uint_as_float((uint32_t)(v >> 32)), fp.dfreq, fp.doct,
-                                 fp.dseed);
-            pts[2u * id] = __float_as_uint(f);  // only this lane reads the key of a listed point from here on
+        for (uint32_t base = 0; base < n; base += 64u) {
+            const uint32_t q = base + lane;
+            if (base + 32u < n) {  // two points per lane; the second may repeat the first
+                const bool two = q + 32u < n;
+                const uint32_t id = list[q], id2 = two ? list[q + 32u] : id;
+                const u64 v = key[id], v2 = key[id2];
+                const float2 f = fbm2_pair(make_float2(__uint_as_float((uint32_t)v), __uint_as_float((uint32_t)(v >> 32))),
+                                           make_float2(__uint_as_float((uint32_t)v2), __uint_as_float((uint32_t)(v2 >> 32))),
+                                           fp.dfreq, fp.doct, fp.dseed);
+                // only this lane reads the keys of its listed points from here on
+                pts[2u * id] = __float_as_uint(f.x);
+                if (two) pts[2u * id2] = __float_as_uint(f.y);
+            } else if (q < n) {
+                const uint32_t id = list[q];
+                const u64 v = key[id];
+                pts[2u * id] = __float_as_uint(fbm2(__uint_as_float((uint32_t)v), __uint_as_float((uint32_t)(v >> 32)),
+                                                    fp.dfreq, fp.doct, fp.dseed));
+            }
         }
         __syncwarp();
 #pragma unroll
