@@ -578,7 +578,10 @@ __device__ __forceinline__ void batch_list(const BatchDev& bt, FCtx& c, int stat
             if (q < total) {
                 const uint32_t lb = find_inst(s_list, nb, q);
                 b = cb + lb;
-                r = body(b, bt.inst[b], q - s_list[lb]);
+                // A copy: its fields stay in registers across the body's stores, after which
+                // they would be loaded again (64 instances, 1.1M changed bisectors: 227 us, 262).
+                const Inst I = bt.inst[b];
+                r = body(b, I, q - s_list[lb]);
             }
             __syncwarp();
             const uint32_t same = __match_any_sync(0xFFFFFFFFu, b);
