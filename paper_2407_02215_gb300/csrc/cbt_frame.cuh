@@ -455,7 +455,10 @@ __device__ void phase_walks(const BatchDev& bt, FCtx& c, uint32_t* s_cnt, unsign
         if (threadIdx.x < 3) s_tmp[threadIdx.x] = 0;
         stats_reset(s_cnt);
         ctx_tile(bt, bt.tile_base, t, T, c);
-        const Inst& I = c.I;
+        // a copy: read again from shared memory after every store otherwise
+        // (batch of 64: 307 us, 329; the same in the other phases gained nothing
+        // or, in classify, cost registers: 407 us, 538)
+        const Inst I = c.I;
         const uint32_t N = c.N, F = c.F, lt = c.lt, i0 = lt * kTileItems;
         const uint32_t gate = c.fp.gate;
         // the bounds before the tile: the earlier groups of 32 tiles, then the
