@@ -51,13 +51,13 @@ uint32_t item_tiles(uint32_t cap) { return (cap + kTileItems - 1u) / kTileItems;
 // Per-instance arrays.
 struct Layout {
     size_t globals, heap, nb, cd, bits, sums, live, freel, scan, grp, chg, chgr, vc, root64, rel, corner, rbnd, freel2,
-        clr, batch, total;
+        clr, tpre, wish, batch, total;
     uint32_t cap, W, ch;
 };
 
 // A batch region for instances with the given pool sizes and halfedge counts.
 struct BatchLayout {
-    size_t inst, fps, bg, tile_base, ctile_base, stile_base, wtile_base, vtile_base, rel_base, status, tpre, wish, total;
+    size_t inst, fps, bg, tile_base, ctile_base, stile_base, wtile_base, vtile_base, rel_base, status, total;
     uint32_t Titems, TwordsMax, Trel;
 };
 
@@ -84,8 +84,6 @@ BatchLayout batch_layout(uint32_t n, const uint32_t* cap, const uint32_t* W, con
     L.vtile_base = take(4u * (n + 1u));
     L.rel_base = take(4u * (n + 1u));
     L.status = take(8u * (2u * static_cast<size_t>(L.Titems) + L.TwordsMax));
-    L.tpre = take(4u * 2u * static_cast<size_t>(L.TwordsMax));
-    L.wish = take(8u * static_cast<size_t>(L.Titems));
     L.total = off;
     return L;
 }
@@ -127,6 +125,8 @@ bool make_layout(int32_t H, int32_t D, Layout& L) {
     L.rbnd = take(4u * ((h + 31u) / 32u));
     L.freel2 = take(4u * cap);
     L.clr = take(4u * L.W);
+    L.tpre = take(4u * 2u * static_cast<size_t>(word_tiles(L.W, kFrame1TileWords)));
+    L.wish = take(8u * static_cast<size_t>(item_tiles(L.cap)));
     const uint32_t Hh = static_cast<uint32_t>(H);
     const BatchLayout B = batch_layout(1, &L.cap, &L.W, &Hh);
     L.batch = take(B.total);
@@ -287,8 +287,6 @@ int batch_build(cbt_state* const* states, uint32_t n, char* region, cudaStream_t
     d.rel_base = reinterpret_cast<const uint32_t*>(region + B->L.rel_base);
     d.bg = reinterpret_cast<BatchGlobals*>(region + B->L.bg);
     d.status = reinterpret_cast<unsigned long long*>(region + B->L.status);
-    d.tpre = reinterpret_cast<uint32_t*>(region + B->L.tpre);
-    d.wish = reinterpret_cast<unsigned long long*>(region + B->L.wish);
     std::vector<Inst> insts(n);
     for (uint32_t b = 0; b < n; ++b) insts[b] = states[b]->inst;
     std::memset(&d.inst0, 0, sizeof(Inst));
@@ -625,6 +623,8 @@ extern "C" int cbt_create(int32_t H, const int32_t* twin, const int32_t* next, c
     I.freel = reinterpret_cast<uint32_t*>(b + L.freel);
     I.freel2 = reinterpret_cast<uint32_t*>(b + L.freel2);
     I.clr = reinterpret_cast<uint32_t*>(b + L.clr);
+    I.tpre = reinterpret_cast<uint32_t*>(b + L.tpre);
+    I.wish = reinterpret_cast<unsigned long long*>(b + L.wish);
     I.scan = reinterpret_cast<uint32_t*>(b + L.scan);
     I.grp = reinterpret_cast<uint4*>(b + L.grp);
     I.chg = reinterpret_cast<uint32_t*>(b + L.chg);

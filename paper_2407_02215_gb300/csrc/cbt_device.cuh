@@ -15,6 +15,10 @@
 //   freel2[cap] u32  single-instance frame: the other free list (this frame's and
 //                    the next one's change places every frame)
 //   clr[W]     u32   single-instance frame: bits cleared this frame; 0 between frames
+//   tpre[2 W/64] u32 single-instance frame: ones before each word tile, this
+//                    frame's and the next one's
+//   wish[cap/1024] u64 single-instance frame: lower-bound split costs per scan
+//                    tile; 0 between frames
 //   scan[cap]  u32   per live index: split cost, then its running total
 //   grp[cap]   uint4 per live index: the members of the merge group whose
 //                    smallest member it is, or of a split wish's chain
@@ -135,6 +139,12 @@ struct Inst {
     uint32_t pad_;
     uint32_t* freel2;       // single-instance frame: the other free list
     uint32_t* clr;          // single-instance frame: the frame's cleared bits, 0 between frames
+    // What freel_full vouches for lies with the instance, not with the batch that launches the frame:
+    // cbt_update and a batch of one may take turns on it.
+    uint32_t* tpre;            // single-instance frame: [2][word tiles] ones before each word tile of the next
+                               // frame's starting bitfield (which: freel_full)
+    unsigned long long* wish;  // single-instance frame: [item tiles] the split wishes' lower-bound costs per scan
+                               // tile, 0 between frames of that kernel
     const uint32_t* rbnd;   // bit h: halfedge h has no Twin (mesh boundary), [ceil(H / 32)]
 };
 
@@ -220,10 +230,6 @@ struct BatchDev {
     uint32_t* vcount;            // the export on its own (B == 1): the live count goes here, in mapped
                                  // host memory, and nothing else is written when it exceeds vcap
     uint32_t timing;             // one-launch frame: record phase boundaries
-    unsigned long long* wish;    // single-instance frame: [Titems] the split wishes' lower-bound costs per scan
-                                 // tile, 0 between frames of that kernel
-    uint32_t* tpre;              // single-instance frame: [2][Twords] ones before each word tile of
-                                 // the next frame's starting bitfield (which: the instance's freel_full)
 };
 
 constexpr int kThreads = 256;
