@@ -1235,6 +1235,9 @@ __device__ void vertices_of(const Inst& I, const FrameP& fp, const uint32_t* s_t
         // s_list, the staging its back) with one coalesced store per word
         const uint32_t lane = threadIdx.x & 31u;
         float* stage = reinterpret_cast<float*>(s_list) + (kFBuf - 288u * (kFThreads / 32)) + 288u * (threadIdx.x >> 5);
+        // the list's length as every thread of the block counts it: *s_n itself
+        // may already hold the next round's rows when a slow warp looks
+        uint32_t cnt = 0;
         for (uint32_t base = blockIdx.x * kFThreads; base < n; base += stride) {
             const uint32_t i = base + threadIdx.x;
             bool cached = false;
@@ -1256,16 +1259,16 @@ __device__ void vertices_of(const Inst& I, const FrameP& fp, const uint32_t* s_t
             for (uint32_t w = lane; w < 288u; w += 32u)
                 if ((m >> (w / 9u)) & 1u) dst[w] = stage[w];
             __syncwarp();
-            __syncthreads();
-            const uint32_t cnt = *s_n;
+            cnt += (uint32_t)__syncthreads_count(i < n && !cached);
             if (cnt > kFBuf - 288u * (kFThreads / 32) - kFThreads) {  // block-uniform: keep clear of the staging
                 evaluate(cnt);
                 __syncthreads();
+                cnt = 0;
                 if (threadIdx.x == 0) *s_n = 0;
                 __syncthreads();
             }
         }
-        evaluate(*s_n);
+        evaluate(cnt);
         return;
     }
     // warp-uniform rounds of 32 consecutive rows (warp-major over the grid,
