@@ -3,6 +3,8 @@
 
 namespace cbtgpu {
 
+template cudaError_t launch_frame_form<kFormF32Disp>(const BatchDev&, int, cudaStream_t);
+template int frame_blocks_form<kFormF32Disp>();
 template cudaError_t launch_frame1_form<kFormF32Disp>(const BatchDev&, int, uint32_t, cudaStream_t);
 template int frame1_blocks_form<kFormF32Disp>();
 
