@@ -131,14 +131,16 @@ __device__ __forceinline__ void ctx_tile(const BatchDev& bt, const uint32_t* bas
 // differs and clusters (grants and chains at an instance's start, culled
 // regions): with tiles dealt round robin the batch frame waited for its
 // slowest blocks, and with four consecutive tiles at a time it was slower
-// still (batch of 15M bisectors: 1744 and 1953 us; handed out 1684).
+// still (batch of 15M bisectors: 1744 and 1953 us; handed out 1684). With at
+// most one of the T tiles per block there is nothing to hand out (the gate of
+// 65k bisectors in a pool of 2^23 slots: 9.3 us with tickets, 8.1 without).
 struct TileFeed {
     uint32_t* ticket;
     uint32_t* s;  // [2] in shared memory
-    uint32_t p = 0, ahead = 0;
-    __device__ __forceinline__ TileFeed(uint32_t* t, uint32_t* shared) : ticket(t), s(shared) {}
+    uint32_t T, p = 0, ahead = kNull;
+    __device__ __forceinline__ TileFeed(uint32_t* t, uint32_t* shared, uint32_t tiles) : ticket(t), s(shared), T(tiles) {}
     __device__ __forceinline__ void take() {
-        if (threadIdx.x == 0) ahead = gridDim.x + atomicAdd(ticket, 1u);
+        if (threadIdx.x == 0 && T > gridDim.x) ahead = gridDim.x + atomicAdd(ticket, 1u);
     }
     __device__ __forceinline__ uint32_t first() {
         take();
@@ -146,6 +148,7 @@ struct TileFeed {
     }
     // With the whole block, at the end of a tile.
     __device__ __forceinline__ uint32_t next() {
+        if (T <= gridDim.x) return kNull;
         if (threadIdx.x == 0) s[p] = ahead;
         __syncthreads();
         const uint32_t t = s[p];
@@ -308,17 +311,38 @@ __device__ __forceinline__ bool has_twin_bound(const Inst& I, uint64_t j) {
     return h < I.H && !((__ldg(I.rbnd + (h >> 5)) >> (h & 31u)) & 1u);
 }
 
+// Whether classify takes a single instance's T item tiles in four parts of 256
+// items, a warp one round of 32, or whole, a warp four rounds: whole tiles of
+// a pool that holds few bisectors leave blocks idle beside others that run
+// four rounds in a row. The parts' shared lists cost FP32 more than they give
+// once half of the blocks have a tile, the forms with longer evaluations once
+// every block has two (2^23-slot pools, 608 blocks; whole and in parts, us: FP32,
+// 65k live 18.0 and 7.4, 239k 17.6 and 14.4, 562k 26.6 and 27.5; fixed point,
+// 366k 47 and 36, 1.0M 100 and 90; projected, 107k 140 and 39, 814k 294 and 199,
+// 2.3M 541 and 535; displaced, 567k 143 and 118, 1.4M 290 and 291).
+template <int F>
+__device__ __forceinline__ bool classify_in_parts(uint32_t T) {
+    return F == kFormF32 ? 2u * T <= gridDim.x : T < 2u * gridDim.x;
+}
+// The same for the walks, each of whose parts adds up the bounds before its
+// tile: while every part has a block of its own (65k live, 64 tiles: 11.6 and
+// 8.2 us; 239k 12.9 and 17.2).
+__device__ __forceinline__ bool walks_in_parts(uint32_t T) { return T * (uint32_t)kFPer <= gridDim.x; }
+
 // P1: wishes of every live bisector (Sec. 3.3 GenerateCommands with the R8
 // LOD reading) over item tiles, each warp on its own 128 items of the tile;
 // the items that need a walk listed in place, and the split wishes' lower
 // bounds summed for the walks.
-template <int F>
+template <int F, bool kParts>
 __device__ void phase_classify(const BatchDev& bt, FCtx& c, uint32_t* s_tab, uint32_t* s_cnt) {
     const uint32_t T = bt.bg->total_tiles, S = kFThreads * bt.bg->scan_ipt;
-    const uint32_t lane = threadIdx.x & 31u;
-    __shared__ uint32_t s_feed[2];
-    TileFeed feed(&bt.bg->tickets[kFeedClassify], s_feed);
-    for (uint32_t t = feed.first(); t < T; t = feed.next()) {
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    const uint32_t rounds = kParts ? 1u : (uint32_t)kFPer, units = kParts ? T * kFPer : T;
+    __shared__ uint32_t s_feed[2], s_part[2];
+    TileFeed feed(&bt.bg->tickets[kFeedClassify], s_feed, units);
+    for (uint32_t u = feed.first(); u < units; u = feed.next()) {
+        const uint32_t t = kParts ? u / kFPer : u, q = kParts ? u % kFPer : 0u;
+        if (threadIdx.x < 2) s_part[threadIdx.x] = 0;
         stats_reset(s_cnt);
         ctx_tile(bt, bt.tile_base, t, T, c);
         const Inst& I = c.I;
@@ -327,22 +351,24 @@ __device__ void phase_classify(const BatchDev& bt, FCtx& c, uint32_t* s_tab, uin
         const bool chain = fp.gate != 1;
         const bool cache = vc_form<F>(fp) && fp.vout;
         const uint64_t key = splitmix64(((uint64_t)fp.seed << 32) | (uint64_t)fp.frame);
-        const uint32_t w0 = c.lt * kTileItems + kSubItems * (threadIdx.x >> 5);
+        // the warp's 128 items and its first round of 32 in them
+        const uint32_t w0 = c.lt * kTileItems + kSubItems * (kParts ? 2u * q + (warp >> 2) : warp);
+        const uint32_t k0 = kParts ? warp & 3u : 0u;
         uint32_t sl[kFPer];
         uint64_t hj[kFPer];
 #pragma unroll
         for (int k = 0; k < kFPer; ++k) {
-            const uint32_t i = w0 + 32u * (uint32_t)k + lane;
-            sl[k] = i < N ? I.live[i] : 0u;
+            const uint32_t i = w0 + 32u * (k0 + (uint32_t)k) + lane;
+            sl[k] = (uint32_t)k < rounds && i < N ? I.live[i] : kNull;
         }
 #pragma unroll
-        for (int k = 0; k < kFPer; ++k) hj[k] = w0 + 32u * (uint32_t)k + lane < N ? I.heap[sl[k]] : 0ull;
+        for (int k = 0; k < kFPer; ++k) hj[k] = sl[k] != kNull ? I.heap[sl[k]] : 0ull;
         uint32_t n = 0, bound = 0, paper = 0;
         if (w0 < N) {
             uint32_t* const reg = walk_region(I, w0);
             uint16_t* const list = reinterpret_cast<uint16_t*>(reg + 1);
 #pragma unroll 1
-            for (uint32_t k = 0; k < (uint32_t)kFPer; ++k) {
+            for (uint32_t k = k0; k < k0 + rounds; ++k) {
                 const uint32_t x = 32u * k + lane, i = w0 + x;
                 bool split = false, walk = false, twin = false;
                 uint32_t cost = 0;
@@ -355,6 +381,10 @@ __device__ void phase_classify(const BatchDev& bt, FCtx& c, uint32_t* s_tab, uin
                     if (split && !chain) cost = 3u * (uint32_t)depth_of(hj[0], I.ch) + 4u;
                 }
                 const unsigned wm = __ballot_sync(0xFFFFFFFFu, walk);
+                if (kParts) {  // the four warps of the 128 items append to one list
+                    if (lane == 0) n = atomicAdd(&s_part[warp >> 2], (uint32_t)__popc(wm));
+                    n = __shfl_sync(0xFFFFFFFFu, n, 0);
+                }
                 if (walk)
                     list[n + __popc(wm & ((1u << lane) - 1u))] =
                         (uint16_t)(x | (split ? 128u : 0u) | (twin ? 256u : 0u));
@@ -370,7 +400,7 @@ __device__ void phase_classify(const BatchDev& bt, FCtx& c, uint32_t* s_tab, uin
                 }
             }
             if (lane == 0) {
-                reg[0] = n;
+                if (!kParts) reg[0] = n;
                 if (bound) {
                     atomicAdd(bound_sums(bt) + t, (unsigned long long)bound);
                     atomicAdd(bound_groups(bt, c.b) + (c.lt >> 5), (unsigned long long)bound);
@@ -379,6 +409,7 @@ __device__ void phase_classify(const BatchDev& bt, FCtx& c, uint32_t* s_tab, uin
             }
         }
         __syncthreads();
+        if (kParts && lane == 0 && k0 == 0u && w0 < N) *walk_region(I, w0) = s_part[warp >> 2];
         stats_flush(s_cnt, I.g, kStSplitWishes);
         __syncthreads();
     }
@@ -445,13 +476,16 @@ static __device__ bool group_if_mergeable(const Inst& I, uint32_t s1, uint64_t j
 // denied: 6.6M wishes of a batch of 15M bisectors, 0.7M granted; its classify
 // with the walks took 680 us and the gate's sums 67, these two phases 427 and 343 (in a
 // nearly full 2^23-slot pool 290 and 10, now 165 and 110).
+template <bool kParts>
 __device__ void phase_walks(const BatchDev& bt, FCtx& c, uint32_t* s_cnt, unsigned long long* s_red, uint32_t* s_tmp,
                             uint32_t* s_n) {
     const uint32_t T = bt.bg->total_tiles, S = kFThreads * bt.bg->scan_ipt;
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    const uint32_t regions = kParts ? 2u : kFThreads / 32, units = kParts ? T * kFPer : T;
     __shared__ uint32_t s_feed[2];
-    TileFeed feed(&bt.bg->tickets[kFeedWalks], s_feed);
-    for (uint32_t t = feed.first(); t < T; t = feed.next()) {
+    TileFeed feed(&bt.bg->tickets[kFeedWalks], s_feed, units);
+    for (uint32_t u = feed.first(); u < units; u = feed.next()) {
+        const uint32_t t = kParts ? u / kFPer : u;
         if (threadIdx.x < 3) s_tmp[threadIdx.x] = 0;
         stats_reset(s_cnt);
         ctx_tile(bt, bt.tile_base, t, T, c);
@@ -459,7 +493,8 @@ __device__ void phase_walks(const BatchDev& bt, FCtx& c, uint32_t* s_cnt, unsign
         // (batch of 64: 307 us, 329; the same in the other phases gained nothing
         // or, in classify, cost registers: 407 us, 538)
         const Inst I = c.I;
-        const uint32_t N = c.N, F = c.F, lt = c.lt, i0 = lt * kTileItems;
+        const uint32_t N = c.N, F = c.F, lt = c.lt;
+        const uint32_t i0 = lt * kTileItems + (kParts ? 2u * kSubItems * (u % kFPer) : 0u);  // the unit's first item
         const uint32_t gate = c.fp.gate;
         // the bounds before the tile: the earlier groups of 32 tiles, then the
         // earlier tiles of its group
@@ -469,7 +504,7 @@ __device__ void phase_walks(const BatchDev& bt, FCtx& c, uint32_t* s_cnt, unsign
         if (threadIdx.x < (lt & 31u)) before += __ldcg(bound_sums(bt) + t - 1u - threadIdx.x);
         if (threadIdx.x >= kFThreads - kFThreads / 32) {  // entries of warp k's items
             const uint32_t k = threadIdx.x - (kFThreads - kFThreads / 32);
-            s_n[k] = i0 + kSubItems * k < N ? *walk_region(I, i0 + kSubItems * k) : 0u;
+            s_n[k] = k < regions && i0 + kSubItems * k < N ? *walk_region(I, i0 + kSubItems * k) : 0u;
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xFFFFFFFFu, before, o);
@@ -673,7 +708,7 @@ __device__ void phase_gate(const BatchDev& bt, FCtx& c, uint32_t* s_cnt, uint32_
                            uint32_t* s_tmp, uint32_t* s_n, uint2* s_list, bool always_recorded = false) {
     const uint32_t T = bt.bg->total_stiles, ipt = bt.bg->scan_ipt;
     __shared__ uint32_t s_feed[2];
-    TileFeed feed(&bt.bg->tickets[kFeedGate], s_feed);
+    TileFeed feed(&bt.bg->tickets[kFeedGate], s_feed, T);
     for (uint32_t t = kOne ? blockIdx.x : feed.first(); t < T; t = kOne ? t + gridDim.x : feed.next()) {
         if (threadIdx.x == 0) *s_n = 0;
         stats_reset(s_cnt);
@@ -809,7 +844,7 @@ __device__ void phase_alloc(const BatchDev& bt, FCtx& c, uint32_t* s_cnt, Pair* 
     uint32_t* s_list = s_buf;              // local item indices to validate
     uint32_t* s_fate = s_buf + kFBuf / 2;  // their fates, by local item index
     __shared__ uint32_t s_feed[2];
-    TileFeed feed(&bt.bg->tickets[kFeedAlloc], s_feed);
+    TileFeed feed(&bt.bg->tickets[kFeedAlloc], s_feed, T);
     for (uint32_t t = feed.first(); t < T; t = feed.next()) {
         if (threadIdx.x == 0) *s_n = 0;
         stats_reset(s_cnt);
@@ -1122,7 +1157,7 @@ __device__ void phase_compact(const BatchDev& bt, FCtx& c, const uint32_t* s_tab
                               uint32_t* s_w, float* s_stage) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     __shared__ uint32_t s_feed[2];
-    TileFeed feed(&bt.bg->tickets[kFeedCompact], s_feed);
+    TileFeed feed(&bt.bg->tickets[kFeedCompact], s_feed, bt.Twords);
     for (uint32_t wt = feed.first(); wt < bt.Twords; wt = feed.next()) {
         ctx_tile(bt, bt.wtile_base, wt, bt.Twords, c);
         const Inst& I = c.I;
@@ -1308,7 +1343,7 @@ __device__ void phase_vertices(const BatchDev& bt, FCtx& c, const uint32_t* s_ta
     vertices_of<F>(c.I, c.fp, s_tab, s_list, s_n);
 }
 
-template <int F>
+template <int F, bool kOne>
 __global__ void __launch_bounds__(kFThreads, CBT_FRAME_MIN_BLOCKS) k_frame(BatchDev bt) {
     __shared__ FCtx s_c;
     __shared__ __align__(16) uint32_t s_tab[kDecTabWords];
@@ -1329,10 +1364,16 @@ __global__ void __launch_bounds__(kFThreads, CBT_FRAME_MIN_BLOCKS) k_frame(Batch
     phase_prep(bt, s_warp, s_tmp);
     grid_sync(bt.bg, epoch, 1u);
     stamp(bt, 1);
-    phase_classify<F>(bt, s_c, s_tab, s_cnt);
+    if (kOne && classify_in_parts<F>(bt.bg->total_tiles))
+        phase_classify<F, true>(bt, s_c, s_tab, s_cnt);
+    else
+        phase_classify<F, false>(bt, s_c, s_tab, s_cnt);
     grid_sync(bt.bg, epoch, 2u);
     stamp(bt, 2);
-    phase_walks(bt, s_c, s_cnt, reinterpret_cast<unsigned long long*>(s_buf), s_tmp, s_w);
+    if (kOne && walks_in_parts(bt.bg->total_tiles))
+        phase_walks<true>(bt, s_c, s_cnt, reinterpret_cast<unsigned long long*>(s_buf), s_tmp, s_w);
+    else
+        phase_walks<false>(bt, s_c, s_cnt, reinterpret_cast<unsigned long long*>(s_buf), s_tmp, s_w);
     grid_sync(bt.bg, epoch, 3u);
     stamp(bt, 3);
     phase_gate(bt, s_c, s_cnt, s_red, s_warp, s_tmp, &s_n, reinterpret_cast<uint2*>(s_buf));
@@ -1348,7 +1389,7 @@ __global__ void __launch_bounds__(kFThreads, CBT_FRAME_MIN_BLOCKS) k_frame(Batch
     grid_sync(bt.bg, epoch, 7u);
     stamp(bt, 7);
     phase_compact<F>(bt, s_c, s_tab, s_buf, s_w, s_stage);
-    if (bt.B == 1) {
+    if (kOne) {
         grid_sync(bt.bg, epoch, 8u);
         stamp(bt, 8);
         phase_vertices<F>(bt, s_c, s_tab, s_buf, &s_n);
@@ -1357,7 +1398,7 @@ __global__ void __launch_bounds__(kFThreads, CBT_FRAME_MIN_BLOCKS) k_frame(Batch
     if (threadIdx.x == 0) {
         if (bt.timing) atomicMax(&bt.bg->t[kFramePhases], global_ns());
         if (blockIdx.x == 0) {
-            bt.bg->bar_epoch = epoch + (bt.B == 1 ? kBarriers + 1u : kBarriers) * gridDim.x;
+            bt.bg->bar_epoch = epoch + (kOne ? kBarriers + 1u : kBarriers) * gridDim.x;
             if (ld_volatile(&bt.bg->abort))
                 for (uint32_t b = 0; b < bt.B; ++b) set_err(bt.inst[b].g, kErrTimeout);
         }
@@ -2548,7 +2589,9 @@ cudaError_t launch_coop(void (*kernel)(A...), int grid, cudaStream_t s, A... arg
 
 template <int F>
 cudaError_t launch_frame_form(const BatchDev& bt, int grid, cudaStream_t s) {
-    return launch_coop<BatchDev>(k_frame<F>, grid, s, bt);
+    if constexpr (F != kFormAny)
+        if (bt.B == 1) return launch_coop<BatchDev>(k_frame<F, true>, grid, s, bt);
+    return launch_coop<BatchDev>(k_frame<F, false>, grid, s, bt);
 }
 template <int F>
 cudaError_t launch_frame1_form(const BatchDev& bt, int grid, uint32_t tbits, cudaStream_t s) {
@@ -2556,8 +2599,13 @@ cudaError_t launch_frame1_form(const BatchDev& bt, int grid, uint32_t tbits, cud
 }
 template <int F>
 int frame_blocks_form() {
-    int n = 0;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_frame<F>, kFThreads, 0) == cudaSuccess ? n : 0;
+    int n = 0, m = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_frame<F, false>, kFThreads, 0) != cudaSuccess) return 0;
+    if constexpr (F != kFormAny) {
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&m, k_frame<F, true>, kFThreads, 0) != cudaSuccess) return 0;
+        return n < m ? n : m;
+    }
+    return n;
 }
 template <int F>
 int frame1_blocks_form() {

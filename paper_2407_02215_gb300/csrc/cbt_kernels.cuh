@@ -44,7 +44,8 @@ int frame1_blocks_per_sm();
 cudaError_t launch_frame1(const BatchDev& bt, int form, int grid, uint32_t tbits, cudaStream_t s);
 // The same per vertex form (cbt_frame.cuh, one source file per form so that
 // they compile in parallel). Both frames exist for every form, the batch frame
-// also for kFormAny (frames that differ).
+// also for kFormAny (frames that differ) and, but for that, once more for a
+// single instance.
 template <int F>
 cudaError_t launch_frame_form(const BatchDev& bt, int grid, cudaStream_t s);
 template <int F>
