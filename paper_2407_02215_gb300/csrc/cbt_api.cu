@@ -196,10 +196,13 @@ struct cbt_batch {
     int fused_grid1 = 0; // the same for the single-instance frame (0: not available)
     bool last_frame1 = false;  // the last fused frame ran the single-instance kernel
     bool use_graph = false;
-    cudaGraphExec_t exec = nullptr;
-    uint32_t exec_tw = 0, exec_mult = 0;
-    bool exec_vertices = false, exec_fused = false;
-    int exec_form = kFormAny;
+    // the frame as a graph, one per form of its kernels: frames that change
+    // their form now and then replay what was captured for it before
+    struct Graph {
+        cudaGraphExec_t exec = nullptr;
+        uint32_t tw = 0, mult = 0, launches = 0;
+        bool vertices = false, fused = false;
+    } graph[kForms];
     bool timing = false;
     cudaEvent_t ev[kNumKernels + 1] = {};
     uint32_t timed = 0, launches = 0;
@@ -324,7 +327,8 @@ int batch_build(cbt_state* const* states, uint32_t n, char* region, cudaStream_t
 
 void batch_free(cbt_batch* B) {
     if (!B) return;
-    if (B->exec) cudaGraphExecDestroy(B->exec);
+    for (auto& g : B->graph)
+        if (g.exec) cudaGraphExecDestroy(g.exec);
     if (B->timing)
         for (auto& e : B->ev) cudaEventDestroy(e);
     for (auto& e : B->tune_ev)
@@ -504,11 +508,11 @@ int batch_update(cbt_batch* B, const cbt_frame* frames, cudaStream_t s) {
         // the graph copies the frame parameters from pinned staging
         if (B->staged_pending) cudaEventSynchronize(B->staged);
         std::memcpy(B->h_fps, fps.data(), sizeof(FrameP) * n);
-        if (!B->exec || B->exec_tw != B->tw || B->exec_mult != B->grid_mult || B->exec_vertices != vertices ||
-            B->exec_fused != B->fused || B->exec_form != form) {
-            if (B->exec) {
-                cudaGraphExecDestroy(B->exec);
-                B->exec = nullptr;
+        cbt_batch::Graph& G = B->graph[B->fused ? form : step_form(form)];
+        if (!G.exec || G.tw != B->tw || G.mult != B->grid_mult || G.vertices != vertices || G.fused != B->fused) {
+            if (G.exec) {
+                cudaGraphExecDestroy(G.exec);
+                G.exec = nullptr;
             }
             cudaStream_t cs;
             if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking)) return CBT_ECUDA;
@@ -520,16 +524,17 @@ int batch_update(cbt_batch* B, const cbt_frame* frames, cudaStream_t s) {
             const cudaError_t e1 = cudaStreamEndCapture(cs, &g);
             cudaStreamDestroy(cs);
             if (e1 != cudaSuccess || !g) return CBT_ECUDA;
-            const cudaError_t e2 = cudaGraphInstantiate(&B->exec, g, 0);
+            const cudaError_t e2 = cudaGraphInstantiate(&G.exec, g, 0);
             cudaGraphDestroy(g);
             if (e2 != cudaSuccess) return CBT_ECUDA;
-            B->exec_tw = B->tw;
-            B->exec_mult = B->grid_mult;
-            B->exec_vertices = vertices;
-            B->exec_fused = B->fused;
-            B->exec_form = form;
+            G.tw = B->tw;
+            G.mult = B->grid_mult;
+            G.vertices = vertices;
+            G.fused = B->fused;
+            G.launches = B->launches;
         }
-        if (cudaGraphLaunch(B->exec, s) != cudaSuccess) return CBT_ECUDA;
+        B->launches = G.launches;
+        if (cudaGraphLaunch(G.exec, s) != cudaSuccess) return CBT_ECUDA;
         cudaEventRecord(B->staged, s);
         B->staged_pending = true;
         B->timed = 0;

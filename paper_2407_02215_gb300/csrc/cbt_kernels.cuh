@@ -9,7 +9,9 @@
 namespace cbtgpu {
 
 // Launch entry points (defined in cbt_kernels.cu). form: the batch's vertex
-// form, or kFormAny when its frames differ.
+// form, or kFormAny when its frames differ; step_form(form): the one that the
+// per-step kernels are compiled for and run it as.
+inline int step_form(int form) { return form == kFormF32 || form == kFormFixed ? form : kFormAny; }
 void launch_prep(const BatchDev& bt, bool frame_start, int grid, cudaStream_t s);
 void launch_classify(const BatchDev& bt, int form, int grid, cudaStream_t s);
 void launch_walk(const BatchDev& bt, int grid, cudaStream_t s);
