@@ -777,8 +777,8 @@ extern "C" int cbt_vertices(cbt_state* st, float* d_out, const double h_origin[3
     bt.fps = nullptr;
     bt.fp0 = fp;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    launch_prep(bt, false, grid_prep(B), s);
     bt.vcount = d_counts + 3;
+    launch_prep(bt, false, grid_prep(B), s);
     launch_vertices(bt, form_of(fp), std::max(1, static_cast<int>(std::min<uint32_t>(bt.Titems, static_cast<uint32_t>(st->sms) * 8u))), s);
     rc = check_launch();
     if (rc) return rc;

@@ -80,6 +80,8 @@ __global__ void __launch_bounds__(kThreads) k_prep(BatchDev bt, int frame_start)
         const uint32_t nstat = 2u * bt.Titems + bt.Twords;
         for (uint32_t k = tid; k < nstat; k += nth) bt.status[k] = 0ull;
     }
+    // an export on its own that k_vertices will refuse leaves the state as it is
+    if (bt.vcount && bt.inst[0].sums[1] > bt.fp0.vcap) return;
     for (uint32_t e = tid; e < bt.Trel; e += nth) rel_entry(bt, e);
 }
 
