@@ -1871,7 +1871,7 @@ __device__ void phase_classify1(const BatchDev& bt, FCtx& c, uint32_t* s_tab, ui
         if (kSharedPoints<F> && shared)
             cmd = classify_shared<F>(I, fp, i < N, i, sa, ja, s_tab, s_cnt, slots, pts, cache);
         else if (i < N)
-            cmd = classify_item<F>(I, fp, key, i, sa, ja, s_tab, s_cnt, cache, false, gen);
+            cmd = classify_item<F>(I, fp, key, i, sa, ja, s_tab, s_cnt, cache, gen);
         if (i < N) {
             split = (cmd & kSplitWish) != 0u;
             walk = split || ((cmd & kMergeWish) && !(cmd & kHeapOdd));

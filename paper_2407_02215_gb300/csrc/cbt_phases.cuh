@@ -723,15 +723,11 @@ __device__ __forceinline__ bool item_wishes(const Inst& I, const FrameP& fp, uin
 
 // The command word of slot s (live index i, heap ID j) and its scan word.
 __device__ __forceinline__ uint32_t store_command(const Inst& I, const FrameP& fp, uint32_t i, uint32_t s, uint64_t j,
-                                                  bool split, bool merge, bool kept, uint32_t* s_cnt,
-                                                  bool merge_in = false) {
+                                                  bool split, bool merge, bool kept, uint32_t* s_cnt) {
     const int d = depth_of(j, I.ch);
     const uint32_t cmd = (split ? kSplitWish : 0u) | (merge ? kMergeWish : 0u) |
                          ((d & 1) ? kDepthOdd : 0u) | ((j & 1ull) ? kHeapOdd : 0u) | (kept ? kVcValid : 0u);
-    if (merge_in)
-        atomicOr(cmd_ptr(I, s), cmd);
-    else
-        *cmd_ptr(I, s) = cmd;
+    *cmd_ptr(I, s) = cmd;
     // the paper's gate charges 3d + 4 without walking the chain (k_walk
     // computes the exact chain cost otherwise)
     I.scan[i] = (split && fp.gate == 1) ? 3u * (uint32_t)d + 4u : 0u;
@@ -742,20 +738,18 @@ __device__ __forceinline__ uint32_t store_command(const Inst& I, const FrameP& f
 // With `cache` (the one-launch frame exporting sphere-form or displaced
 // vertices) the LOD test's vertices go to vc[s] and the command word says so
 // (kVcValid): the export then copies them instead of evaluating them again.
-// With `merge_in` the word is ORed in: it was cleared before the phase and
-// other bisectors' chain walks may mark it while this one classifies.
 template <int F>
 __device__ __forceinline__ uint32_t classify_item(const Inst& I, const FrameP& fp, uint64_t key, uint32_t i,
                                                   uint32_t s, uint64_t j, const uint32_t* tab, uint32_t* s_cnt,
-                                                  bool cache = false, bool merge_in = false, unsigned long long gen = 0) {
+                                                  bool cache = false, unsigned long long gen = 0) {
     bool split, merge, kept;
     if (!item_wishes<F>(I, fp, key, s, j, tab, split, merge, cache ? I.vc + 9ull * s : nullptr, &kept, gen)) {
         set_err(I.g, kErrLink);
-        if (!merge_in) *cmd_ptr(I, s) = 0u;
+        *cmd_ptr(I, s) = 0u;
         I.scan[i] = 0u;
         return 0u;
     }
-    return store_command(I, fp, i, s, j, split, merge, kept, s_cnt, merge_in);
+    return store_command(I, fp, i, s, j, split, merge, kept, s_cnt);
 }
 
 // Pointer chases of the frame, after classify: the compatibility-chain cost
