@@ -123,10 +123,12 @@ bool make_layout(int32_t H, int32_t D, Layout& L) {
     L.rel = take(std::max(72u * h, rel_stage(h)));
     L.corner = take(12u * h);
     L.rbnd = take(4u * ((h + 31u) / 32u));
-    L.freel2 = take(4u * cap);
-    L.clr = take(4u * L.W);
-    L.tpre = take(4u * 2u * static_cast<size_t>(word_tiles(L.W, kFrame1TileWords)));
-    L.wish = take(8u * static_cast<size_t>(item_tiles(L.cap)));
+    // the single-instance frame's own arrays: pools above its tables do without
+    const size_t one = L.cap <= kFrame1MaxCap ? 1u : 0u;
+    L.freel2 = take(one * 4u * cap);
+    L.clr = take(one * 4u * L.W);
+    L.tpre = take(one * 4u * 2u * word_tiles(L.W, kFrame1TileWords));
+    L.wish = take(one * 8u * item_tiles(L.cap));
     const uint32_t Hh = static_cast<uint32_t>(H);
     const BatchLayout B = batch_layout(1, &L.cap, &L.W, &Hh);
     L.batch = take(B.total);
@@ -626,10 +628,12 @@ extern "C" int cbt_create(int32_t H, const int32_t* twin, const int32_t* next, c
     I.sums = reinterpret_cast<uint32_t*>(b + L.sums);
     I.live = reinterpret_cast<uint32_t*>(b + L.live);
     I.freel = reinterpret_cast<uint32_t*>(b + L.freel);
-    I.freel2 = reinterpret_cast<uint32_t*>(b + L.freel2);
-    I.clr = reinterpret_cast<uint32_t*>(b + L.clr);
-    I.tpre = reinterpret_cast<uint32_t*>(b + L.tpre);
-    I.wish = reinterpret_cast<unsigned long long*>(b + L.wish);
+    if (L.cap <= kFrame1MaxCap) {
+        I.freel2 = reinterpret_cast<uint32_t*>(b + L.freel2);
+        I.clr = reinterpret_cast<uint32_t*>(b + L.clr);
+        I.tpre = reinterpret_cast<uint32_t*>(b + L.tpre);
+        I.wish = reinterpret_cast<unsigned long long*>(b + L.wish);
+    }
     I.scan = reinterpret_cast<uint32_t*>(b + L.scan);
     I.grp = reinterpret_cast<uint4*>(b + L.grp);
     I.chg = reinterpret_cast<uint32_t*>(b + L.chg);
@@ -670,7 +674,7 @@ extern "C" int cbt_create(int32_t H, const int32_t* twin, const int32_t* next, c
     double* d_hpos = reinterpret_cast<double*>(b + L.rel + rel_stage(h) - 24u * h);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     cudaMemsetAsync(I.g, 0, sizeof(Globals), s);
-    cudaMemsetAsync(I.clr, 0, 4u * L.W, s);
+    if (I.clr) cudaMemsetAsync(I.clr, 0, 4u * L.W, s);
     cudaMemcpyAsync(d_ints, ints.data(), 12u * h, cudaMemcpyHostToDevice, s);
     cudaMemcpyAsync(d_hpos, hpos.data(), 24u * h, cudaMemcpyHostToDevice, s);
     cudaMemcpyAsync(st->corner, corner.data(), 12u * h, cudaMemcpyHostToDevice, s);
