@@ -311,10 +311,7 @@ int batch_build(cbt_state* const* states, uint32_t n, char* region, cudaStream_t
         B->fused_grid = static_cast<int>(std::min<uint32_t>(work, static_cast<uint32_t>(per_sm * B->sms)));
         // the single-instance frame spreads classify, the walks and the rows
         // of its export over the whole grid, so a small instance also gets
-        // every SM; but with at most one item per thread of two blocks per SM
-        // (pools of 2^16) the other blocks only make each barrier and table
-        // scan longer: a cube's frame (2^16) takes 52.8 us with two blocks per
-        // SM and 58.8 with four, the dodecahedron planet's (2^17) 75.8 and 75.6
+        // every SM
         const int per_sm1 = n == 1 ? frame1_blocks_per_sm() : 0;
         if (per_sm1 > 0) B->fused_grid1 = (B->cap[0] <= kFrame1SmallCap ? std::min(per_sm1, 2) : per_sm1) * B->sms;
     }

@@ -13,9 +13,13 @@
 //
 // The two prefix sums of the per-step kernels (decoupled look-back) become
 // reduce-then-scan here: tile sums, a barrier, then each tile adds the sums
-// before it (the gate), or the fill adds its tile's prefix (the allocation). State between phases lives in the slot arrays (command words,
-// scan words); each block keeps its instance descriptor and frame
-// parameters in shared memory across tiles and phases. Reads of data other
+// before it (the gate), or the fill adds its tile's prefix (the allocation).
+// State between phases lives in the slot arrays (command words, scan words);
+// each block keeps its instance descriptor and frame parameters in shared
+// memory across tiles and phases. A pool above the single-instance frame's
+// tables is a batch of one with an instantiation of its own, whose classify and
+// walks can take tiles in parts and whose export follows the compaction as a
+// phase (P8). Reads of data other
 // blocks wrote in an earlier phase follow a barrier whose fences order them.
 // Every wait is bounded: a barrier that runs out sets the batch's abort word,
 // every later wait then returns at once, and the instances report kErrTimeout.
@@ -1418,12 +1422,16 @@ __global__ void __launch_bounds__(kFThreads) k_wait_selftest(BatchGlobals* bg, i
 // ===================================================== one instance, fewer phases
 //
 // k_frame1: the frame of a single instance (a batch of one), with the same
-// results as k_frame in six phases, or five when the frame's requests all
-// fit the free slots or nothing is exported:
+// results as k_frame in seven phases, without P3 when the frame's requests all
+// fit the free slots, without P6 when nothing is exported. A grid barrier
+// between every two of them (four to six), but for the one after P0 where that
+// is not needed:
 //   P0 prep      frame counters; the camera-relative roots; the word-tile
-//                counts copied; the chain-mark words of the live slots and
-//                the tile counters cleared (the marks only when the last
-//                frame was not this kernel, which leaves them clear)
+//                counts copied. When the last frame was not this kernel also
+//                what that frame would have left: the chain-mark words of the
+//                live slots, the wish counters and the walk list's length
+//                cleared. When it was, and the mesh is small, every block fills
+//                the whole root table and the phase ends without a barrier
 //   P1 classify  wishes (Sec. 3.3 GenerateCommands), in 32-item chunks dealt
 //                warp-major over the grid; the items that need a walk
 //                appended to the frame's walk list; per scan tile the split
@@ -1459,9 +1467,21 @@ __global__ void __launch_bounds__(kFThreads) k_wait_selftest(BatchGlobals* bg, i
 // The instance descriptor and the frame parameters are read from the launch
 // parameters (a copy in shared memory would be reloaded after every store
 // through a generic pointer).
+//
+// From one frame to the next: while the instance's flag word freel_full says
+// that its last frame was this kernel, a free list of every zero bit is kept
+// (freel or freel2), the ones before each word tile (one half of tpre), and the
+// chain marks (chg) of the live slots, the wish counters (wish), the cleared
+// bits (clr) and the walk list's length (nwalk) are 0: P5's final part leaves
+// them so. All of it lies in the instance's workspace, none in that of the
+// handle that launches the frame; every other form of the frame clears the flag.
 
 constexpr uint32_t kMaxTiles1 = kFBuf / 2;  // scan tiles and word tiles the shared tables hold
-constexpr uint32_t kLocalRoots = 64;        // meshes up to this many halfedges: every block fills the root table
+// Meshes up to kLocalRoots halfedges: every block fills the root table. With
+// and without the barrier this saves, us a frame: 24 halfedges 46.8 and 45.3, 60
+// 59.0 and 57.0 (with cached points 48.8 and 47.1), 96 47.4 and 47.4, 104 46.1 and
+// 44.9, 208 46.0 and 46.8: the line lies where the gain is sure.
+constexpr uint32_t kLocalRoots = 64;
 
 // Exclusive prefix sums of n <= kMaxTiles1 pairs over the block: thread x
 // takes the consecutive entries [x k, x k + k), k = ceil(n / threads), loads
@@ -1527,8 +1547,7 @@ __device__ __forceinline__ uint32_t* free_list1(const BatchDev& bt, Carry carry,
 __device__ __forceinline__ unsigned long long* tile_counts(const BatchDev& bt) {
     return bt.status + 2u * bt.Titems;
 }
-// Per scan tile: the split wishes' lower-bound costs (P1), then the
-// allocation sums (P4).
+// Per scan tile: the split wishes' lower-bound costs (P1).
 __device__ __forceinline__ unsigned long long* wish_counts(const BatchDev& bt) { return bt.inst0.wish; }
 // The chain marks of P2 (one word per slot; the per-step frame's list of
 // changed items uses the same array).
@@ -1589,7 +1608,7 @@ __device__ void frame_init1(const BatchDev& bt, uint32_t tbits, uint32_t N) {
 }
 
 // P0 (single instance): the frame's counters, and what classify needs from
-// other blocks: the camera-relative roots, the wish counts and the walk
+// other blocks: the camera-relative roots, the wish counters and the walk
 // list's length cleared, and the chain-mark words of the live slots cleared
 // unless the last frame (this kernel) left them 0.
 __device__ void phase_prep1(const BatchDev& bt, uint32_t tbits, uint32_t N) {

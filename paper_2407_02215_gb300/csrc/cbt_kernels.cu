@@ -1,7 +1,7 @@
 // Kernels of one frame of the CBT bisection update for sm_103a.
 //
-// Frame = k_prep, k_classify, k_gate, k_scatter, k_alloc, k_free, k_fill,
-// k_cbt [, k_vertices], each launched once for a whole batch of independent
+// Frame = k_prep, k_classify, k_walk, k_gate, k_scatter, k_alloc, k_free,
+// k_fill, k_cbt, k_compact [, k_vertices], each launched once for a whole batch of independent
 // instances (a single instance is a batch of one). Item kernels walk global
 // tiles of 1024 live indices; tile t belongs to the instance b with
 // tile_base[b] <= t < tile_base[b+1], recomputed on the device each frame
@@ -9,6 +9,7 @@
 // prefix scans and the reduction are single-pass decoupled look-back scans
 // over tiles handed out by an atomic ticket, so a tile only waits for tiles
 // owned by running blocks; the first tile of each instance starts its own
+// prefix.
 #include "cbt_kernels.cuh"
 #include "cbt_phases.cuh"
 
@@ -718,6 +719,7 @@ __global__ void __launch_bounds__(kThreads) k_leaves(Inst I, uint32_t* slots, ui
     }
 }
 
+// The FP32 vertices of every instance's live bisectors, ascending slot order,
 // over static tiles of its pool capacity (tiles past the live count exit).
 template <int F>
 __global__ void __launch_bounds__(kThreads, 3) k_vertices(BatchDev bt) {

@@ -39,7 +39,15 @@ cudaError_t launch_frame(const BatchDev& bt, int form, int grid, cudaStream_t s)
 // It holds its scan-tile and word-tile tables in shared memory, so it takes
 // pools of at most kFrame1MaxCap slots with 64-word tiles.
 constexpr uint32_t kFrame1MaxCap = 1u << 22;
-constexpr uint32_t kFrame1SmallCap = 1u << 16;  // pools up to this run with two blocks per SM
+// Pools up to kFrame1SmallCap slots run with two blocks per SM instead of the
+// four that fit: with at most one item per thread of those the other blocks
+// only make each barrier and table scan longer. Two and four, us a frame, pools
+// of 2^16: a cube 45.3 and 52.8, the dodecahedron planet 57.0 and 63.4, with
+// waves 65.7 and 70.8, with cached points 47.1 and 52.3, cube-spheres in fixed
+// point 47.4 and 52.6 and in FP64 55.6 and 61.9, a displaced grid 56.8 and 61.5;
+// 2^14 the same by 4 to 6 us. At 2^17 it depends: the cube 49.4 and 54.8, the
+// planet 75.2 and 78.9, with waves 92.4 and 92.2, with cached points 66.2 and 64.6.
+constexpr uint32_t kFrame1SmallCap = 1u << 16;
 constexpr uint32_t kFrame1TileWords = 64;
 constexpr int kFrame1Phases = 7;
 int frame1_blocks_per_sm();

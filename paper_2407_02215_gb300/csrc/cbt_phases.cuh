@@ -752,12 +752,6 @@ __device__ __forceinline__ uint32_t classify_item(const Inst& I, const FrameP& f
     return store_command(I, fp, i, s, j, split, merge, kept, s_cnt);
 }
 
-// Pointer chases of the frame, after classify: the compatibility-chain cost
-// of every split wish (command form of Alg. 3) and the Alg. 4 group of every
-// merge wish with an even heap ID, whose smallest member records the members
-// (for the gate, the allocation and the fill). The items that need a walk
-// are packed per tile in shared memory first, so that whole warps walk.
-
 // ------------------------------------------------------------ allocation
 
 __device__ __forceinline__ uint32_t leaves_of(uint32_t sb) {
@@ -1218,12 +1212,6 @@ static __device__ uint32_t fill_merge(const Inst& I, uint32_t dest, const uint4 
     }
     return relinked;
 }
-
-// FillNewBlocks + UpdateNeighbors + UpdateBitfield for the changed
-// bisectors, one per thread over the instance's compacted list (written in
-// ascending slot order by k_alloc): a split bisector clears its bit and
-// writes its family; the smallest member of a merge group clears its
-// members' bits and writes the parents.
 
 // The three vertices of bisector j into r; false (error word set, r not
 // written) when j does not decode to a root of this mesh.
