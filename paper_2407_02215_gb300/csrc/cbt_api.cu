@@ -221,6 +221,9 @@ struct cbt_state {
     Inst inst;
     uint32_t* corner;  // [H][3] global points of the root corners: vert[h], vert[next h], V + face[h]
     uint32_t npts;     // global points: 1 + the largest in corner
+    // carried from frame to frame by the single-instance frame (null in pools it does not take)
+    uint32_t* tpre;
+    unsigned long long* wish;
     uint32_t* h_ix;  // pinned counts, after self's frame parameters: of the last cbt_index (words 0 to 2) and
                      // cbt_vertices (3)
     void* workspace;
@@ -295,7 +298,11 @@ int batch_build(cbt_state* const* states, uint32_t n, char* region, cudaStream_t
     std::vector<Inst> insts(n);
     for (uint32_t b = 0; b < n; ++b) insts[b] = states[b]->inst;
     std::memset(&d.inst0, 0, sizeof(Inst));
-    if (n == 1) d.inst0 = insts[0];
+    if (n == 1) {
+        d.inst0 = insts[0];
+        d.tpre = states[0]->tpre;
+        d.wish = states[0]->wish;
+    }
     int rc = CBT_OK;
     if (cudaMemcpyAsync(region + B->L.inst, insts.data(), sizeof(Inst) * n, cudaMemcpyHostToDevice, s) ||
         cudaMemsetAsync(d.bg, 0, sizeof(BatchGlobals), s) ||
@@ -628,8 +635,8 @@ extern "C" int cbt_create(int32_t H, const int32_t* twin, const int32_t* next, c
     if (L.cap <= kFrame1MaxCap) {
         I.freel2 = reinterpret_cast<uint32_t*>(b + L.freel2);
         I.clr = reinterpret_cast<uint32_t*>(b + L.clr);
-        I.tpre = reinterpret_cast<uint32_t*>(b + L.tpre);
-        I.wish = reinterpret_cast<unsigned long long*>(b + L.wish);
+        st->tpre = reinterpret_cast<uint32_t*>(b + L.tpre);
+        st->wish = reinterpret_cast<unsigned long long*>(b + L.wish);
     }
     I.scan = reinterpret_cast<uint32_t*>(b + L.scan);
     I.grp = reinterpret_cast<uint4*>(b + L.grp);

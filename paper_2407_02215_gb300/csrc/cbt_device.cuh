@@ -139,12 +139,6 @@ struct Inst {
     uint32_t pad_;
     uint32_t* freel2;       // single-instance frame: the other free list
     uint32_t* clr;          // single-instance frame: the frame's cleared bits, 0 between frames
-    // What freel_full vouches for lies with the instance, not with the batch that launches the frame:
-    // cbt_update and a batch of one may take turns on it.
-    uint32_t* tpre;            // single-instance frame: [2][word tiles] ones before each word tile of the next
-                               // frame's starting bitfield (which: freel_full)
-    unsigned long long* wish;  // single-instance frame: [item tiles] the split wishes' lower-bound costs per scan
-                               // tile, 0 between frames of that kernel
     const uint32_t* rbnd;   // bit h: halfedge h has no Twin (mesh boundary), [ceil(H / 32)]
 };
 
@@ -230,6 +224,12 @@ struct BatchDev {
     uint32_t* vcount;            // the export on its own (B == 1): the live count goes here, in mapped
                                  // host memory, and nothing else is written when it exceeds vcap
     uint32_t timing;             // one-launch frame: record phase boundaries
+    // B == 1, what the instance's freel_full vouches for: in the instance's workspace, not in the batch's,
+    // since cbt_update and a batch of one may take turns on it
+    unsigned long long* wish;    // single-instance frame: [Titems] the split wishes' lower-bound costs per scan
+                                 // tile, 0 between frames of that kernel
+    uint32_t* tpre;              // single-instance frame: [2][Twords] ones before each word tile of
+                                 // the next frame's starting bitfield (which: the instance's freel_full)
 };
 
 constexpr int kThreads = 256;

@@ -1548,7 +1548,7 @@ __device__ __forceinline__ unsigned long long* tile_counts(const BatchDev& bt) {
     return bt.status + 2u * bt.Titems;
 }
 // Per scan tile: the split wishes' lower-bound costs (P1).
-__device__ __forceinline__ unsigned long long* wish_counts(const BatchDev& bt) { return bt.inst0.wish; }
+__device__ __forceinline__ unsigned long long* wish_counts(const BatchDev& bt) { return bt.wish; }
 // The chain marks of P2 (one word per slot; the per-step frame's list of
 // changed items uses the same array).
 __device__ __forceinline__ uint32_t* chain_marks(const Inst& I) { return I.chg; }
@@ -2365,8 +2365,8 @@ __device__ void phase_final1(const BatchDev& bt, FCtx& c, bool all_granted, uint
     // frame in the other buffer
     const unsigned long long* tc = tile_counts(bt);
     const uint32_t cur = carry.buffer();
-    const uint32_t* tpre_in = I.tpre + cur * bt.Twords;
-    uint32_t* tpre_out = I.tpre + (cur ^ 1u) * bt.Twords;
+    const uint32_t* tpre_in = bt.tpre + cur * bt.Twords;
+    uint32_t* tpre_out = bt.tpre + (cur ^ 1u) * bt.Twords;
     if (carry.ok()) {
         for (uint32_t t = threadIdx.x; t < nt; t += kFThreads) s_old[t] = __ldcg(tpre_in + t);
         __syncthreads();
